@@ -307,6 +307,7 @@ __device__ __forceinline__ float load_acc(const float* p, int64_t i, float) { re
 __device__ __forceinline__ double load_acc(const double* p, int64_t i, double) { return p[i]; }
 
 constexpr int kGemvCols = 8;
+constexpr int kGemvRows = 2;   // rows of a thread in flight
 
 // The value the passes sketch for element `i` of the box's rows, per format:
 // plain (f64 / f32 / bf16), BF16x2 (hi + lo with hi = bf16(x), lo = bf16(x -
@@ -330,68 +331,109 @@ __device__ __forceinline__ Tacc row_value(const Tm* m, int64_t i, const float* s
   }
 }
 
+// Block (x, y) sums its rows of D[c] = sum_row m[row] B[c][map(row)] for the
+// kGemvCols columns of group y.  Bound by memory latency at the sizes boxes
+// have (a 32^3 box: 32768 rows, 18 to 40 columns, 2.6 MB of B out of L2): one
+// column group per block and kGemvRows rows per thread in flight put the
+// loads of a 32^3 box on 320 blocks instead of 32 that walked the groups in
+// turn (28 us before).  The blocks of group 0 also write the walk's copy of
+// their rows, and block (0, 0) the copy of the other side's row, which were
+// two launches of their own.
 template <typename Tm, typename Ts, typename Tacc, int MODE = RV_PLAIN>
-__global__ void __launch_bounds__(256) side_gemv_kernel(SideSpec s, const Ts* src, int64_t src_ld,
-                                                        int cut, const Tm* m, int64_t rows,
-                                                        int cols, int64_t rpb, Tacc* part,
-                                                        const float* scale) {
+__global__ void __launch_bounds__(256) side_gemv_kernel(const __grid_constant__ SideSpec s,
+                                                        const Ts* src, int64_t src_ld, int cut,
+                                                        const Tm* m, int64_t rows, int cols,
+                                                        int64_t rpb, Tacc* part,
+                                                        const float* scale, Tacc* mcopy,
+                                                        const Ts* brow, Tacc* bcopy, int bcols) {
   __shared__ Tacc red[8][kGemvCols];
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int64_t r0 = (int64_t)blockIdx.x * rpb;
   const int64_t r1 = r0 + rpb < rows ? r0 + rpb : rows;
-  for (int c0 = 0; c0 < cols; c0 += kGemvCols) {
-    Tacc acc[kGemvCols];
+  const int c0 = blockIdx.y * kGemvCols;
+  const int nc = cols - c0 < kGemvCols ? cols - c0 : kGemvCols;
+  const bool copy = mcopy && blockIdx.y == 0;
+  if (bcopy && blockIdx.x == 0 && blockIdx.y == 0)
+    for (int c = threadIdx.x; c < bcols; c += blockDim.x) bcopy[c] = load_acc(brow, c, Tacc(0));
+  Tacc acc[kGemvCols];
 #pragma unroll
-    for (int k = 0; k < kGemvCols; ++k) acc[k] = 0;
-    for (int64_t row = r0 + threadIdx.x; row < r1; row += blockDim.x) {
-      int64_t f = row;
-      if (cut) {
-        int64_t rem = row, stride = 1;
-        f = 0;
+  for (int k = 0; k < kGemvCols; ++k) acc[k] = 0;
+  for (int64_t base = r0 + threadIdx.x; base < r1; base += (int64_t)kGemvRows * blockDim.x) {
+    Tacc mv[kGemvRows];
+    int64_t f[kGemvRows];
+#pragma unroll
+    for (int u = 0; u < kGemvRows; ++u) {
+      const int64_t row = base + (int64_t)u * blockDim.x;
+      const bool in = row < r1;
+      mv[u] = in ? row_value<MODE, Tm, Tacc>(m, row, scale) : Tacc(0);
+      if (in && copy) mcopy[row] = mv[u];
+      f[u] = in ? row : -1;
+      if (cut && in) {
+        // the row's place in the whole-tensor block
+        int64_t full = 0, stride = 1;
+        uint64_t rem = (uint64_t)row;
         for (int mm = s.nmodes - 1; mm >= 0; --mm) {
-          const int64_t i = rem % s.ext[mm];
-          rem /= s.ext[mm];
-          f += (s.off[mm] + i) * stride;
+          const uint64_t e = (uint64_t)s.ext[mm];
+          const uint64_t q = (rem | e) >> 32 ? rem / e : (uint64_t)((uint32_t)rem / (uint32_t)e);
+          full += (s.off[mm] + (int64_t)(rem - q * e)) * stride;
+          rem = q;
           stride *= s.full[mm];
         }
+        f[u] = full;
       }
-      const Tacc mv = row_value<MODE, Tm, Tacc>(m, row, scale);
+    }
+#pragma unroll
+    for (int u = 0; u < kGemvRows; ++u)
 #pragma unroll
       for (int k = 0; k < kGemvCols; ++k)
-        if (c0 + k < cols) acc[k] += mv * load_acc(src, (int64_t)(c0 + k) * src_ld + f, Tacc(0));
-    }
+        if (f[u] >= 0 && k < nc)
+          acc[k] += mv[u] * load_acc(src, (int64_t)(c0 + k) * src_ld + f[u], Tacc(0));
+  }
 #pragma unroll
-    for (int k = 0; k < kGemvCols; ++k) {
-      Tacc v = acc[k];
-      for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
-      if (lane == 0) red[warp][k] = v;
-    }
-    __syncthreads();
-    if (threadIdx.x < kGemvCols && c0 + (int)threadIdx.x < cols) {
-      Tacc t = 0;
-      for (int w = 0; w < (int)(blockDim.x >> 5); ++w) t += red[w][threadIdx.x];
-      part[(int64_t)blockIdx.x * cols + c0 + threadIdx.x] = t;
-    }
-    __syncthreads();
+  for (int k = 0; k < kGemvCols; ++k) {
+    Tacc v = acc[k];
+    for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
+    if (lane == 0) red[warp][k] = v;
+  }
+  __syncthreads();
+  if ((int)threadIdx.x < nc) {
+    Tacc t = 0;
+    for (int w = 0; w < 8; ++w) t += red[w][threadIdx.x];
+    part[(int64_t)blockIdx.x * cols + c0 + threadIdx.x] = t;
   }
 }
 
+// One warp per column: lane l adds the partials of blocks l, l + 32, ... in
+// order, then the lanes are summed as a fixed tree (deterministic).
 template <typename Tacc>
-__global__ void gemv_reduce_kernel(const Tacc* part, int nblk, int cols, int cols_pad, Tacc* D) {
-  for (int c = blockIdx.x * blockDim.x + threadIdx.x; c < cols_pad; c += gridDim.x * blockDim.x) {
-    Tacc t = 0;
-    if (c < cols)
-      for (int b = 0; b < nblk; ++b) t += part[(int64_t)b * cols + c];
-    D[c] = t;
-  }
+__global__ void __launch_bounds__(256) gemv_reduce_kernel(const Tacc* part, int nblk, int cols,
+                                                          int cols_pad, Tacc* D) {
+  const int lane = threadIdx.x & 31;
+  const int c = blockIdx.x * 8 + (threadIdx.x >> 5);
+  if (c >= cols_pad) return;
+  Tacc t = 0;
+  if (c < cols)
+    for (int b = lane; b < nblk; b += 32) t += part[(int64_t)b * cols + c];
+  for (int o = 16; o > 0; o >>= 1) t += __shfl_xor_sync(0xffffffffu, t, o);
+  if (lane == 0) D[c] = t;
+}
+
+// Rows of a block: two batches per thread at least (512 rows), more once the
+// grid fills the GPU eight times over.
+static void gemv_shape(int64_t rows, int cols, int64_t* nblk, int64_t* rpb) {
+  const int64_t groups = std::max<int64_t>(1, ceil_div(cols, kGemvCols));
+  const int64_t most = std::max<int64_t>(1, (int64_t)num_sms() * 8 / groups);
+  *nblk = std::max<int64_t>(1, std::min<int64_t>(ceil_div(rows, 512), most));
+  *rpb = ceil_div(rows, *nblk);
 }
 
 ttnn_status launch_side_gemv(const SideSpec& s, const void* src, int64_t src_ld, bool cut,
                              const void* m, int m_store, const float* scale, int64_t rows,
-                             int cols, int cols_pad, void* D, int d_f64, void* part,
+                             int cols, int cols_pad, void* D, int d_f64, void* mcopy,
+                             const void* brow, void* bcopy, int bcols, void* part,
                              int64_t part_bytes, cudaStream_t st, bool dry, int64_t* need) {
-  const int64_t nblk = std::max<int64_t>(1, std::min<int64_t>(ceil_div(rows, 1024), (int64_t)num_sms() * 4));
-  const int64_t rpb = ceil_div(rows, nblk);
+  int64_t nblk, rpb;
+  gemv_shape(rows, cols, &nblk, &rpb);
   const int64_t bytes = nblk * std::max(cols, 1) * (d_f64 ? 8 : 4);
   if (dry) {
     if (need) *need = bytes;
@@ -401,73 +443,40 @@ ttnn_status launch_side_gemv(const SideSpec& s, const void* src, int64_t src_ld,
     set_error("rank-one pass: scratch too small");
     return TTNN_ENOMEM;
   }
-  if (cols_pad == 0) return TTNN_OK;
-  if (d_f64) {
-    if (m_store != 0 || s.store != 0) {
+  if (cols > 0 || mcopy || bcopy) {
+    const dim3 grid((unsigned)nblk, (unsigned)std::max<int64_t>(1, ceil_div(cols, kGemvCols)), 1);
+    const int ct = cut ? 1 : 0;
+    if (d_f64 && m_store == 0 && s.store == 0)
+      side_gemv_kernel<double, double, double><<<grid, 256, 0, st>>>(
+          s, (const double*)src, src_ld, ct, (const double*)m, rows, cols, rpb, (double*)part,
+          scale, (double*)mcopy, (const double*)brow, (double*)bcopy, bcols);
+    else if (!d_f64 && m_store == 1 && s.store == 1)
+      side_gemv_kernel<float, float, float><<<grid, 256, 0, st>>>(
+          s, (const float*)src, src_ld, ct, (const float*)m, rows, cols, rpb, (float*)part, scale,
+          (float*)mcopy, (const float*)brow, (float*)bcopy, bcols);
+    else if (!d_f64 && m_store == 2 && s.store == 2)
+      side_gemv_kernel<uint16_t, uint16_t, float><<<grid, 256, 0, st>>>(
+          s, (const uint16_t*)src, src_ld, ct, (const uint16_t*)m, rows, cols, rpb, (float*)part,
+          scale, (float*)mcopy, (const uint16_t*)brow, (float*)bcopy, bcols);
+    else if (!d_f64 && m_store == kStoreSplit && s.store == 2)
+      side_gemv_kernel<float, uint16_t, float, RV_SPLIT><<<grid, 256, 0, st>>>(
+          s, (const uint16_t*)src, src_ld, ct, (const float*)m, rows, cols, rpb, (float*)part,
+          scale, (float*)mcopy, (const uint16_t*)brow, (float*)bcopy, bcols);
+    else if (!d_f64 && m_store == kStoreFp8 && s.store == 2 && scale)
+      side_gemv_kernel<uint8_t, uint16_t, float, RV_FP8><<<grid, 256, 0, st>>>(
+          s, (const uint16_t*)src, src_ld, ct, (const uint8_t*)m, rows, cols, rpb, (float*)part,
+          scale, (float*)mcopy, (const uint16_t*)brow, (float*)bcopy, bcols);
+    else {
       set_error("rank-one pass: unsupported formats");
       return TTNN_EUNSUPPORTED;
     }
-    if (cols > 0)
-      side_gemv_kernel<double, double, double><<<(unsigned)nblk, 256, 0, st>>>(
-          s, (const double*)src, src_ld, cut ? 1 : 0, (const double*)m, rows, cols, rpb,
-          (double*)part, scale);
-  } else if (m_store == 1 && s.store == 1) {
-    if (cols > 0)
-      side_gemv_kernel<float, float, float><<<(unsigned)nblk, 256, 0, st>>>(
-          s, (const float*)src, src_ld, cut ? 1 : 0, (const float*)m, rows, cols, rpb,
-          (float*)part, scale);
-  } else if (m_store == 2 && s.store == 2) {
-    if (cols > 0)
-      side_gemv_kernel<uint16_t, uint16_t, float><<<(unsigned)nblk, 256, 0, st>>>(
-          s, (const uint16_t*)src, src_ld, cut ? 1 : 0, (const uint16_t*)m, rows, cols, rpb,
-          (float*)part, scale);
-  } else if (m_store == kStoreSplit && s.store == 2) {
-    if (cols > 0)
-      side_gemv_kernel<float, uint16_t, float, RV_SPLIT><<<(unsigned)nblk, 256, 0, st>>>(
-          s, (const uint16_t*)src, src_ld, cut ? 1 : 0, (const float*)m, rows, cols, rpb,
-          (float*)part, scale);
-  } else if (m_store == kStoreFp8 && s.store == 2 && scale) {
-    if (cols > 0)
-      side_gemv_kernel<uint8_t, uint16_t, float, RV_FP8><<<(unsigned)nblk, 256, 0, st>>>(
-          s, (const uint16_t*)src, src_ld, cut ? 1 : 0, (const uint8_t*)m, rows, cols, rpb,
-          (float*)part, scale);
-  } else {
-    set_error("rank-one pass: unsupported formats");
-    return TTNN_EUNSUPPORTED;
+    TTNN_TRY(check_launch("side_gemv_kernel"));
   }
-  if (cols > 0) TTNN_TRY(check_launch("side_gemv_kernel"));
-  const unsigned rb = (unsigned)std::max<int64_t>(1, std::min<int64_t>(ceil_div(cols_pad, 256), 64));
+  if (cols_pad == 0) return TTNN_OK;
+  const unsigned rb = (unsigned)ceil_div(cols_pad, 8);
   if (d_f64) gemv_reduce_kernel<double><<<rb, 256, 0, st>>>((const double*)part, (int)nblk, cols, cols_pad, (double*)D);
   else gemv_reduce_kernel<float><<<rb, 256, 0, st>>>((const float*)part, (int)nblk, cols, cols_pad, (float*)D);
   return check_launch("gemv_reduce_kernel");
-}
-
-template <typename Ts, typename Td, int MODE = RV_PLAIN>
-__global__ void to_walk_kernel(const Ts* src, Td* dst, int64_t n, const float* scale) {
-  for (int64_t e = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; e < n;
-       e += (int64_t)gridDim.x * blockDim.x)
-    dst[e] = row_value<MODE, Ts, Td>(src, e, scale);
-}
-
-ttnn_status launch_to_walk(const void* src, int src_store, const float* scale, void* dst,
-                           int d_f64, int64_t n, cudaStream_t st) {
-  if (n == 0) return TTNN_OK;
-  const unsigned blocks = (unsigned)std::min<int64_t>(ceil_div(n, 256), (int64_t)num_sms() * 8);
-  if (!d_f64 && src_store == 2)
-    to_walk_kernel<uint16_t, float><<<blocks, 256, 0, st>>>((const uint16_t*)src, (float*)dst, n, scale);
-  else if (!d_f64 && src_store == 1)
-    to_walk_kernel<float, float><<<blocks, 256, 0, st>>>((const float*)src, (float*)dst, n, scale);
-  else if (d_f64 && src_store == 0)
-    to_walk_kernel<double, double><<<blocks, 256, 0, st>>>((const double*)src, (double*)dst, n, scale);
-  else if (!d_f64 && src_store == kStoreSplit)
-    to_walk_kernel<float, float, RV_SPLIT><<<blocks, 256, 0, st>>>((const float*)src, (float*)dst, n, scale);
-  else if (!d_f64 && src_store == kStoreFp8 && scale)
-    to_walk_kernel<uint8_t, float, RV_FP8><<<blocks, 256, 0, st>>>((const uint8_t*)src, (float*)dst, n, scale);
-  else {
-    set_error("walk copy: unsupported formats");
-    return TTNN_EUNSUPPORTED;
-  }
-  return check_launch("to_walk_kernel");
 }
 
 ttnn_status launch_side(const SideSpec& s, void* out, cudaStream_t st) {

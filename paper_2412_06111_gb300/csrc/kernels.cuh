@@ -121,19 +121,20 @@ ttnn_status launch_side_gather_batch(const GatherJob* jobs, int n, cudaStream_t 
 // else the row itself.  Accumulates in the walk type (f64 when d_f64) per
 // block of rows, then sums the block partials in a fixed order
 // (deterministic).  With dry, only reports the scratch bytes (`need`).
-// Row formats of launch_side_gemv / launch_to_walk beyond the storage codes
+// Row formats of launch_side_gemv beyond the storage codes
 // 0 f64, 1 f32, 2 bf16: binary32 rows sketched as bf16 hi + lo (BF16x2
 // plans), and E4M3 rows with one binary32 scale per 128 consecutive rows,
 // sketched as bf16(f32(q) * s) (E4M3 plans; `scale` required).
 constexpr int kStoreFp8 = 3, kStoreSplit = 4;
+// With mcopy, mcopy[row] = the sketched value of m[row] in the walk type is
+// written beside; with bcopy, bcopy[c] = brow[c] (side format) for c < bcols.
+// With mcopy, mcopy[row] = the sketched value of m[row] in the walk type is
+// written beside; with bcopy, bcopy[c] = brow[c] (side format) for c < bcols.
 ttnn_status launch_side_gemv(const SideSpec& s, const void* src, int64_t src_ld, bool cut,
                              const void* m, int m_store, const float* scale, int64_t rows,
-                             int cols, int cols_pad, void* D, int d_f64, void* part,
+                             int cols, int cols_pad, void* D, int d_f64, void* mcopy,
+                             const void* brow, void* bcopy, int bcols, void* part,
                              int64_t part_bytes, cudaStream_t st, bool dry, int64_t* need);
-// dst[e] = the value sketched for src[e] (format src_store as above) in the
-// walk type (f32, or f64 when d_f64) for e < n.
-ttnn_status launch_to_walk(const void* src, int src_store, const float* scale, void* dst,
-                           int d_f64, int64_t n, cudaStream_t st);
 
 // misc
 ttnn_status launch_fill_zero(void* p, int64_t bytes, cudaStream_t st);

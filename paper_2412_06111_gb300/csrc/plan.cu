@@ -1339,18 +1339,18 @@ ttnn_status run_dense_update(ttnn_plan_s& P, void* acc, const void* data, const 
     void* Dout = r1 == 1 ? (void*)D2 : (void*)D1;
     int64_t need = 0;
     TTNN_TRY(launch_side_gemv(gs, nullptr, 0, false, nullptr, r1_store, nullptr, r1_rows, gcols,
-                              gpad, nullptr, P.walk_f64, nullptr, 0, st, true, &need));
+                              gpad, nullptr, P.walk_f64, nullptr, nullptr, nullptr, 0, nullptr, 0, st,
+                              true, &need));
     char* part = ws.alloc(need);
     if (!dry) {
       ++P.n_simt_pass;
-      const int pstore = r1_store, sstore = P.side_store, wf64 = P.walk_f64 ? 1 : 0;
+      const int pstore = r1_store, wf64 = P.walk_f64 ? 1 : 0;
+      void* const mcopy = Mw != (const char*)data ? (void*)Mw : nullptr;
+      void* const bcopy = bw != (const char*)r1_brow ? (void*)bw : nullptr;
       auto go = [=](cudaStream_t s) -> ttnn_status {
-        if (Mw != (const char*)data)
-          TTNN_TRY(launch_to_walk(data, pstore, tile_scale, (void*)Mw, wf64, r1_rows, s));
-        if (bw != (const char*)r1_brow)
-          TTNN_TRY(launch_to_walk(r1_brow, sstore, nullptr, (void*)bw, wf64, r1_bpad, s));
         return launch_side_gemv(gs, gsrc, gld, gcut, data, pstore, tile_scale, r1_rows, gcols,
-                                gpad, Dout, wf64, part, need, s, false, nullptr);
+                                gpad, Dout, wf64, mcopy, r1_brow, bcopy, r1_bpad, part, need, s,
+                                false, nullptr);
       };
       if (batch) batch->passes.push_back(go);
       else TTNN_TRY(go(st));
