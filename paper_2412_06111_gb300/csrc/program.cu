@@ -10,9 +10,12 @@
 namespace ttnn {
 
 constexpr int kExecThreads = 256;
-static_assert(sizeof(LevelBatch) <= 32000, "level batch must fit the kernel parameter space");
+static_assert(sizeof(LevelBatch<WalkOp, kLargeOps>) <= 32000 &&
+                  sizeof(LevelBatch<CpOp, kLargeOps>) <= 32000,
+              "level batch must fit the kernel parameter space");
 constexpr int kMpKC2 = 32;
 constexpr size_t kExecSmem = 48 * 1024;
+constexpr size_t kKgemmSmem = 48 * 1024;
 
 static int exec_sms() {
   static int n = 0;
@@ -29,7 +32,7 @@ static int exec_sms() {
 // device parts
 // ---------------------------------------------------------------------------
 template <typename Tin, typename Tw, typename Tout, typename Tacc, typename I>
-__device__ void dev_contract(const DevOp& op, int64_t blk) {
+__device__ void dev_contract(const WalkOp& op, int64_t blk) {
   const Contract& c = op.c;
   const int g = op.g;
   const I J = (I)c.J, Q = (I)c.Q, NB = (I)c.NB;
@@ -91,7 +94,7 @@ __device__ void dev_contract(const DevOp& op, int64_t blk) {
 }
 
 template <typename T, typename I>
-__device__ void dev_reduce(const DevOp& op, int64_t blk) {
+__device__ void dev_reduce(const WalkOp& op, int64_t blk) {
   const Contract& c = op.c;
   const I total = (I)(c.P * c.NB * c.Q * c.J);
   const I o = (I)(blk * kExecThreads) + (I)threadIdx.x;
@@ -115,7 +118,7 @@ __device__ void dev_reduce(const DevOp& op, int64_t blk) {
 // Mode product as a batched small GEMM over one chunk of CH batch items:
 // out[p,b,q,j] (+)= alpha * sum_i W[i*wsI + b*wsB] * in[p,i,q,j].
 template <typename T, typename I>
-__device__ void dev_mp(const DevOp& op, int64_t blk, unsigned char* smem) {
+__device__ void dev_mp(const WalkOp& op, int64_t blk, unsigned char* smem) {
   const Contract& c = op.c;
   const int BG = op.BG, CG = op.CG, CH = op.CH;
   const int WB = 4 * BG, WC = 4 * CG;
@@ -208,7 +211,7 @@ __device__ void dev_mp(const DevOp& op, int64_t blk, unsigned char* smem) {
 constexpr int kWsMaxNI = 128;
 
 template <int NBT, typename I>
-__device__ void dev_mpw(const DevOp& op, int64_t blk, unsigned char* smem) {
+__device__ void dev_mpw(const WalkOp& op, int64_t blk, unsigned char* smem) {
   const Contract& c = op.c;
   float* Ws = (float*)smem;                 // [NI][NBT]
   const int NI = (int)c.NI, NB = (int)c.NB;
@@ -275,7 +278,7 @@ __device__ void dev_mpw(const DevOp& op, int64_t blk, unsigned char* smem) {
 // tiles (coalesced loads) into partial[split][p][b][q][j].
 constexpr int kKredTile = 64;
 
-__device__ void dev_kred(const DevOp& op, int64_t blk, unsigned char* smem) {
+__device__ void dev_kred(const WalkOp& op, int64_t blk, unsigned char* smem) {
   const Contract& c = op.c;
   const int NB = (int)c.NB, J = (int)c.J;
   const int64_t items = c.P * c.Q;
@@ -366,7 +369,7 @@ __device__ __forceinline__ float kg_weight(const Contract& c, int64_t i, int b) 
 }
 
 template <typename I>
-__device__ void dev_kgemm(const DevOp& op, int64_t blk, unsigned char* smem) {
+__device__ void dev_kgemm(const WalkOp& op, int64_t blk, unsigned char* smem) {
   const Contract& c = op.c;
   float* Ws = (float*)smem;                       // [kKgKT][kKgMB]
   float* Is = Ws + kKgKT * kKgMB;                 // [kKgKT][kKgLd]
@@ -512,7 +515,7 @@ __device__ __forceinline__ void scatter_decode(const Scatter& s, I e, int64_t* i
 }
 
 template <typename T, typename I>
-__device__ void dev_scatter(const DevOp& op, int64_t blk) {
+__device__ void dev_scatter(const WalkOp& op, int64_t blk) {
   const Scatter& s = op.s;
   I total = 1;
   for (int a = 0; a < s.nd; ++a) total *= (I)s.size[a];
@@ -560,8 +563,7 @@ __device__ void dev_scatter(const DevOp& op, int64_t blk) {
   }
 }
 
-__device__ void dev_proj(const DevOp& op, int64_t blk) {
-  const Proj& m = op.pj;
+__device__ void dev_proj(const Proj& m, int64_t blk) {
   const int64_t e = blk * kExecThreads + threadIdx.x;
   if (e >= (int64_t)m.nq * m.ncols) return;
   const int q = (int)(e / m.ncols), j = (int)(e % m.ncols);
@@ -577,8 +579,7 @@ __device__ void dev_proj(const DevOp& op, int64_t blk) {
   m.out[(int64_t)q * m.ldo + j] = acc;
 }
 
-__device__ void dev_outer(const DevOp& op, int64_t blk) {
-  const Outer& m = op.ou;
+__device__ void dev_outer(const Outer& m, int64_t blk) {
   int64_t total = 1;
   for (int a = 0; a < m.A; ++a) total *= m.n[a];
   const int64_t e = blk * kExecThreads + threadIdx.x;
@@ -602,96 +603,95 @@ __device__ void dev_outer(const DevOp& op, int64_t blk) {
   else ((float*)m.out)[oo] += (float)(m.alpha * acc);
 }
 
-__device__ void dev_eye(const DevOp& op, int64_t blk) {
+__device__ void dev_eye(const WalkOp& op, int64_t blk) {
   const int64_t n = op.eye_n;
   const int64_t e = blk * kExecThreads + threadIdx.x;
   if (e < n * n) ((double*)op.c.out)[e] = (e / n == e % n) ? 1.0 : 0.0;
 }
 
-template <typename I>
-__device__ __forceinline__ void dispatch(const DevOp& op, int64_t blk, unsigned char* dsm) {
+// The op kinds of one accumulator type and index width.  Each (type, width)
+// pair has a kernel of its own: a small level's time is mostly instruction
+// fetch (16 to 20 stalled warps per issue before, with every kind, both types
+// and both widths in one kernel), so a launch carries only the code its ops
+// can reach.
+template <bool F64, typename I>
+__device__ __forceinline__ void dispatch(const WalkOp& op, int64_t blk, unsigned char* dsm) {
+  typedef typename std::conditional<F64, double, float>::type T;
   switch (op.kind) {
     case OP_CONTRACT:
-      if (op.tin == ET_F32 && op.tw == ET_F32 && op.tout == ET_F32)
-        dev_contract<float, float, float, float, I>(op, blk);
-      else if (op.tin == ET_F64 && op.tout == ET_F64 && op.tw == ET_F64)
-        dev_contract<double, double, double, double, I>(op, blk);
-      else
-        dev_contract<float, double, double, double, I>(op, blk);
+      if (!F64) dev_contract<T, T, T, T, I>(op, blk);
+      else if (op.tin == ET_F64) dev_contract<double, double, double, double, I>(op, blk);
+      else dev_contract<float, double, double, double, I>(op, blk);
+      break;
+    case OP_SCATTER: dev_scatter<T, I>(op, blk); break;
+    case OP_REDUCE: dev_reduce<T, I>(op, blk); break;
+    case OP_EYE:
+      if (F64) dev_eye(op, blk);
       break;
     case OP_MP:
+      if (F64) break;   // binary64 products stay in the lane-group form
       if (op.CG == 0) {   // weight-stationary variant, NBT = op.BG
         switch (op.BG) {
           case 8: dev_mpw<8, I>(op, blk, dsm); break;
           case 16: dev_mpw<16, I>(op, blk, dsm); break;
           default: dev_mpw<32, I>(op, blk, dsm); break;
         }
-      } else if (op.tout == ET_F64) {
-        dev_mp<double, I>(op, blk, dsm);
       } else {
         dev_mp<float, I>(op, blk, dsm);
       }
       break;
-    case OP_SCATTER:
-      if (op.tout == ET_F64) dev_scatter<double, I>(op, blk);
-      else dev_scatter<float, I>(op, blk);
-      break;
-    case OP_REDUCE:
-      if (op.tout == ET_F64) dev_reduce<double, I>(op, blk);
-      else dev_reduce<float, I>(op, blk);
-      break;
-    case OP_EYE:
-      dev_eye(op, blk);
-      break;
     case OP_KRED:
-      dev_kred(op, blk, dsm);
+      if (!F64) dev_kred(op, blk, dsm);
       break;
-    case OP_PROJ:
-      dev_proj(op, blk);
-      break;
-    case OP_OUTER:
-      dev_outer(op, blk);
-      break;
-    default:
-      break;
+    default: break;
   }
 }
 
-__global__ void __launch_bounds__(kExecThreads, 3) level_kernel(const __grid_constant__ LevelBatch lb) {
-  extern __shared__ __align__(16) unsigned char dsm[];
-  const int64_t b = blockIdx.x;
+// The op that holds block b, and b's place among its blocks.
+template <typename Batch>
+__device__ __forceinline__ int op_of_block(const Batch& lb, int b, int64_t* blk) {
   int lo = 0, hi = lb.nops - 1;
   while (lo < hi) {
     const int mid = (lo + hi + 1) / 2;
     if (lb.start[mid] <= b) lo = mid;
     else hi = mid - 1;
   }
-  const DevOp& op = lb.ops[lo];
-  const int64_t blk = b - lb.start[lo];
-  if (op.idx32) dispatch<uint32_t>(op, blk, dsm);
-  else dispatch<int64_t>(op, blk, dsm);
+  *blk = b - lb.start[lo];
+  return lo;
 }
 
-// The split-K GEMM ops of a level in a kernel of their own: its code stays
-// small enough for the instruction caches (the generic level kernel's many op
-// kinds do not, and its ops stall on instruction fetch).
+template <bool F64, typename I, int CAP>
+__global__ void __launch_bounds__(kExecThreads, 3)
+    level_kernel(const __grid_constant__ LevelBatch<WalkOp, CAP> lb) {
+  extern __shared__ __align__(16) unsigned char dsm[];
+  int64_t blk;
+  const int k = op_of_block(lb, (int)blockIdx.x, &blk);
+  dispatch<F64, I>(lb.ops[k], blk, dsm);
+}
+
+// CP updates: projections and outer-product sums.
+template <int CAP>
+__global__ void __launch_bounds__(kExecThreads)
+    cp_level_kernel(const __grid_constant__ LevelBatch<CpOp, CAP> lb) {
+  int64_t blk;
+  const CpOp& op = lb.ops[op_of_block(lb, (int)blockIdx.x, &blk)];
+  if (op.kind == OP_PROJ) dev_proj(op.pj, blk);
+  else dev_outer(op.ou, blk);
+}
+
+// The split-K GEMM ops of a level in a kernel of their own (apart from the
+// code of the other kinds).
 // MINB resident blocks per SM: 2 (128 registers) for levels of a few waves,
 // 3 (80 registers) for levels of many waves, where the extra warps hide more
 // shared-memory latency and the coarser last wave costs little.
-template <int MINB>
-__global__ void __launch_bounds__(kExecThreads, MINB) kgemm_level_kernel(const __grid_constant__ LevelBatch lb) {
+template <int MINB, int CAP>
+__global__ void __launch_bounds__(kExecThreads, MINB)
+    kgemm_level_kernel(const __grid_constant__ LevelBatch<WalkOp, CAP> lb) {
   extern __shared__ __align__(16) unsigned char dsm[];
-  const int64_t b = blockIdx.x;
-  int lo = 0, hi = lb.nops - 1;
-  while (lo < hi) {
-    const int mid = (lo + hi + 1) / 2;
-    if (lb.start[mid] <= b) lo = mid;
-    else hi = mid - 1;
-  }
-  const DevOp& op = lb.ops[lo];
-  const int64_t blk = b - lb.start[lo];
+  int64_t blk;
+  const int k = op_of_block(lb, (int)blockIdx.x, &blk);
   // one instantiation (64-bit column decoding: a few divisions per thread)
-  dev_kgemm<int64_t>(op, blk, dsm);
+  dev_kgemm<int64_t>(lb.ops[k], blk, dsm);
 }
 
 // ---------------------------------------------------------------------------
@@ -865,25 +865,12 @@ int Program::levels() const {
   return m;
 }
 
-static DevOp to_dev(const Op& o) {
-  DevOp d;
-  memset(&d, 0, sizeof(d));
-  d.kind = o.kind;
-  d.tin = o.tin;
-  d.tw = o.tw;
-  d.tout = o.tout;
-  d.c = o.c;
-  if (o.kind == OP_PROJ) d.pj = o.pj;
-  else if (o.kind == OP_OUTER) d.ou = o.ou;
-  else d.s = o.s;
-  d.g = o.g;
-  d.nsplit = o.nsplit;
-  d.chunk = o.chunk;
-  d.partial = o.partial;
-  d.BG = o.BG;
-  d.CG = o.CG;
-  d.CH = o.CH;
-  d.eye_n = o.eye_n;
+// Launch groups of a level: one kernel each.
+enum LaunchGroup { LG_KGEMM = 0, LG_F32, LG_F32_WIDE, LG_F64, LG_F64_WIDE, LG_CP, LG_COUNT };
+
+static LaunchGroup group_of(const Op& o) {
+  if (o.kind == OP_KGEMM) return LG_KGEMM;
+  if (o.kind == OP_PROJ || o.kind == OP_OUTER) return LG_CP;
   // 32-bit decoding when every extent and count stays below 2^31
   const int64_t lim = (int64_t(1) << 31) - 1;
   int64_t m = o.c.P * o.c.NB * o.c.Q * o.c.J * std::max(o.nsplit, 1);
@@ -894,8 +881,88 @@ static DevOp to_dev(const Op& o) {
   }
   m = std::max(m, o.eye_n * o.eye_n);
   m = std::max(m, o.blocks * kExecThreads);
-  d.idx32 = m < lim;
-  return d;
+  if (o.tout == ET_F64) return m < lim ? LG_F64 : LG_F64_WIDE;
+  return m < lim ? LG_F32 : LG_F32_WIDE;
+}
+
+static void to_dev(const Op& o, WalkOp* d) {
+  d->kind = o.kind;
+  d->tin = o.tin;
+  if (o.kind == OP_SCATTER) d->s = o.s;
+  else d->c = o.c;
+  d->g = o.g;
+  d->nsplit = o.nsplit;
+  d->chunk = o.chunk;
+  d->partial = o.partial;
+  d->BG = o.BG;
+  d->CG = o.CG;
+  d->CH = o.CH;
+  d->eye_n = o.eye_n;
+}
+
+static void to_dev(const Op& o, CpOp* d) {
+  d->kind = o.kind;
+  if (o.kind == OP_PROJ) d->pj = o.pj;
+  else d->ou = o.ou;
+}
+
+template <typename OpT, int CAP>
+static int64_t fill_batch(LevelBatch<OpT, CAP>& b, const Op* const* ops, int n) {
+  b.nops = n;
+  int64_t blocks = 0;
+  for (int k = 0; k < n; ++k) {
+    b.start[k] = (int)blocks;
+    to_dev(*ops[k], &b.ops[k]);
+    blocks += ops[k]->blocks;
+    if (blocks >= (int64_t(1) << 31)) return -1;
+  }
+  b.start[n] = (int)blocks;
+  return blocks;
+}
+
+template <int CAP>
+static ttnn_status launch_group(LaunchGroup g, const Op* const* ops, int n, cudaStream_t st) {
+  int64_t blocks;
+  if (g == LG_CP) {
+    LevelBatch<CpOp, CAP> b;
+    if ((blocks = fill_batch(b, ops, n)) > 0)
+      cp_level_kernel<CAP><<<(unsigned)blocks, kExecThreads, 0, st>>>(b);
+  } else {
+    LevelBatch<WalkOp, CAP> b;
+    blocks = fill_batch(b, ops, n);
+    const unsigned gr = (unsigned)blocks;
+    if (blocks <= 0) {
+    } else if (g == LG_KGEMM) {
+      // at least three full waves at three blocks per SM: the 80-register form
+      if (blocks >= 9 * (int64_t)exec_sms())
+        kgemm_level_kernel<3, CAP><<<gr, kExecThreads, kKgemmSmem, st>>>(b);
+      else
+        kgemm_level_kernel<2, CAP><<<gr, kExecThreads, kKgemmSmem, st>>>(b);
+    } else if (g == LG_F32) {
+      level_kernel<false, uint32_t, CAP><<<gr, kExecThreads, kExecSmem, st>>>(b);
+    } else if (g == LG_F32_WIDE) {
+      level_kernel<false, int64_t, CAP><<<gr, kExecThreads, kExecSmem, st>>>(b);
+    } else if (g == LG_F64) {
+      level_kernel<true, uint32_t, CAP><<<gr, kExecThreads, 0, st>>>(b);
+    } else {
+      level_kernel<true, int64_t, CAP><<<gr, kExecThreads, 0, st>>>(b);
+    }
+  }
+  if (blocks < 0) {
+    set_error("program level too large");
+    return TTNN_EUNSUPPORTED;
+  }
+  if (blocks == 0) return TTNN_OK;
+  return check_launch(g == LG_KGEMM ? "kgemm_level_kernel" : g == LG_CP ? "cp_level_kernel" : "level_kernel");
+}
+
+static ttnn_status launch_ops(LaunchGroup g, const std::vector<const Op*>& ops, cudaStream_t st) {
+  for (size_t k = 0; k < ops.size(); k += kLargeOps) {
+    const int n = (int)std::min<size_t>(ops.size() - k, kLargeOps);
+    TTNN_TRY(n <= kSmallOps ? launch_group<kSmallOps>(g, ops.data() + k, n, st)
+                            : launch_group<kLargeOps>(g, ops.data() + k, n, st));
+  }
+  return TTNN_OK;
 }
 
 // A second stream per host thread and device for the split-K GEMM launches
@@ -934,48 +1001,56 @@ static ttnn_status fork_stream(ForkStream** out) {
   return TTNN_OK;
 }
 
+// Debugging: one op alone, timed (the stream is synchronised) and printed.
+static ttnn_status dump_op(const Op& o, int lvl, cudaStream_t st) {
+  cudaEvent_t a = nullptr, e = nullptr;
+  TTNN_TRY_CUDA(cudaEventCreate(&a));
+  TTNN_TRY_CUDA(cudaEventCreate(&e));
+  TTNN_TRY_CUDA(cudaEventRecord(a, st));
+  TTNN_TRY(launch_ops(group_of(o), {&o}, st));
+  TTNN_TRY_CUDA(cudaEventRecord(e, st));
+  TTNN_TRY_CUDA(cudaEventSynchronize(e));
+  float ms = 0.f;
+  cudaEventElapsedTime(&ms, a, e);
+  cudaEventDestroy(a);
+  cudaEventDestroy(e);
+  fprintf(stderr, "[ttnn] %8.1f us  ", ms * 1e3f);
+  if (o.kind == OP_SCATTER)
+    fprintf(stderr, "[ttnn] L%d scatter nd %d nsc %d blocks %lld\n", lvl, o.s.nd, o.s.nsc,
+            (long long)o.blocks);
+  else
+    fprintf(stderr,
+            "[ttnn] L%d kind %d P %lld NI %lld NB %lld Q %lld J %lld isJ %lld wsJ %lld "
+            "wsQ %lld wsP %lld g %d nsplit %d blocks %lld\n",
+            lvl, (int)o.kind, (long long)o.c.P, (long long)o.c.NI, (long long)o.c.NB,
+            (long long)o.c.Q, (long long)o.c.J, (long long)o.c.isJ, (long long)o.c.wsJ,
+            (long long)o.c.wsQ, (long long)o.c.wsP, o.g, o.nsplit, (long long)o.blocks);
+  return TTNN_OK;
+}
+
 ttnn_status Program::run(cudaStream_t st, bool dump) {
   const int L = levels();
-  // per level: the split-K GEMM ops in one launch of their kernel, every
-  // other op in one level_kernel launch; when a level has both, the GEMM
-  // launch goes on the fork stream and runs beside the other
+  // per level: the split-K GEMM ops in one launch of their kernel, the other
+  // ops in one launch per type; when a level has both, the GEMM launch goes
+  // on the fork stream and runs beside the others
   ForkStream* fs = nullptr;
-  LevelBatch lb[2];
-  cudaStream_t gst = st;   // stream of the GEMM launches
-  auto flush = [&](int k) -> ttnn_status {
-    LevelBatch& b = lb[k];
-    if (b.nops == 0) return TTNN_OK;
-    const int64_t blocks = b.start[b.nops];
-    if (blocks > 0) {
-      if (blocks >= (int64_t(1) << 31)) {
-        set_error("program level too large");
-        return TTNN_EUNSUPPORTED;
-      }
-      if (k == 0) {
-        // at least three full waves at three blocks per SM: the 80-register form
-        if (blocks >= 9 * (int64_t)exec_sms())
-          kgemm_level_kernel<3><<<(unsigned)blocks, kExecThreads, kExecSmem, gst>>>(b);
-        else
-          kgemm_level_kernel<2><<<(unsigned)blocks, kExecThreads, kExecSmem, gst>>>(b);
-        TTNN_TRY(check_launch("kgemm_level_kernel"));
-      } else {
-        level_kernel<<<(unsigned)blocks, kExecThreads, kExecSmem, st>>>(b);
-        TTNN_TRY(check_launch("level_kernel"));
-      }
-    }
-    b.nops = 0;
-    return TTNN_OK;
-  };
+  std::vector<const Op*> group[LG_COUNT];
   for (int lvl = 1; lvl <= L; ++lvl) {
-    for (int k = 0; k < 2; ++k) {
-      lb[k].nops = 0;
-      lb[k].start[0] = 0;
+    for (auto& g : group) g.clear();
+    bool other = false;
+    for (const Op& o : ops_) {
+      if (o.level != lvl || o.blocks == 0) continue;
+      if (dump) {
+        TTNN_TRY(dump_op(o, lvl, st));
+        continue;
+      }
+      const LaunchGroup g = group_of(o);
+      group[g].push_back(&o);
+      other = other || g != LG_KGEMM;
     }
-    bool has[2] = {false, false};
-    for (const Op& o : ops_)
-      if (o.level == lvl && o.blocks > 0) has[o.kind == OP_KGEMM ? 0 : 1] = true;
-    gst = st;
-    if (has[0] && has[1] && !dump) {
+    const bool fork = other && !group[LG_KGEMM].empty();
+    cudaStream_t gst = st;   // stream of the GEMM launches
+    if (fork) {
       if (!fs) TTNN_TRY(fork_stream(&fs));
       if (fs) {
         TTNN_TRY_CUDA(cudaEventRecord(fs->fork, st));
@@ -983,49 +1058,9 @@ ttnn_status Program::run(cudaStream_t st, bool dump) {
         gst = fs->st;
       }
     }
-    for (int pass = 0; pass < 2; ++pass) {
-      for (const Op& o : ops_) {
-        if (o.level != lvl || o.blocks == 0) continue;
-        const int k = o.kind == OP_KGEMM ? 0 : 1;
-        if (k != pass) continue;
-        LevelBatch& b = lb[k];
-        if (dump) {
-          // debugging: each op alone, timed (the stream is synchronised)
-          cudaEvent_t a = nullptr, e = nullptr;
-          TTNN_TRY_CUDA(cudaEventCreate(&a));
-          TTNN_TRY_CUDA(cudaEventCreate(&e));
-          b.ops[0] = to_dev(o);
-          b.start[0] = 0;
-          b.start[1] = o.blocks;
-          b.nops = 1;
-          TTNN_TRY_CUDA(cudaEventRecord(a, st));
-          TTNN_TRY(flush(k));
-          TTNN_TRY_CUDA(cudaEventRecord(e, st));
-          TTNN_TRY_CUDA(cudaEventSynchronize(e));
-          float ms = 0.f;
-          cudaEventElapsedTime(&ms, a, e);
-          cudaEventDestroy(a);
-          cudaEventDestroy(e);
-          fprintf(stderr, "[ttnn] %8.1f us  ", ms * 1e3f);
-          if (o.kind == OP_SCATTER)
-            fprintf(stderr, "[ttnn] L%d scatter nd %d nsc %d blocks %lld\n", lvl, o.s.nd, o.s.nsc,
-                    (long long)o.blocks);
-          else
-            fprintf(stderr,
-                    "[ttnn] L%d kind %d P %lld NI %lld NB %lld Q %lld J %lld isJ %lld wsJ %lld "
-                    "wsQ %lld wsP %lld g %d nsplit %d blocks %lld\n",
-                    lvl, (int)o.kind, (long long)o.c.P, (long long)o.c.NI, (long long)o.c.NB,
-                    (long long)o.c.Q, (long long)o.c.J, (long long)o.c.isJ, (long long)o.c.wsJ,
-                    (long long)o.c.wsQ, (long long)o.c.wsP, o.g, o.nsplit, (long long)o.blocks);
-          continue;
-        }
-        if (b.nops == kMaxLevelOps) TTNN_TRY(flush(k));
-        b.ops[b.nops] = to_dev(o);
-        b.start[b.nops + 1] = b.start[b.nops] + o.blocks;
-        ++b.nops;
-      }
-      TTNN_TRY(flush(pass));
-    }
+    for (int g = 0; g < LG_COUNT; ++g)
+      if (!group[g].empty())
+        TTNN_TRY(launch_ops((LaunchGroup)g, group[g], g == LG_KGEMM ? gst : st));
     if (gst != st) {
       TTNN_TRY_CUDA(cudaEventRecord(fs->join, gst));
       TTNN_TRY_CUDA(cudaStreamWaitEvent(st, fs->join, 0));

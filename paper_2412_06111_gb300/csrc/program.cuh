@@ -64,31 +64,43 @@ struct Op {
   int level = 0;
 };
 
-// Device-side copy of an op (plain data, fits the kernel parameter space).
-struct DevOp {
-  int kind, tin, tw, tout;
-  Contract c;
+// Device-side copies of ops (plain data, passed as kernel parameters): the
+// walk / assembly kinds and the CP kinds are apart so that neither pays for
+// the other's size.
+struct WalkOp {
+  int kind, tin, g, nsplit;
+  int BG, CG, CH;
   union {
+    Contract c;
     Scatter s;
+  };
+  int64_t chunk;
+  void* partial;
+  int64_t eye_n;
+  WalkOp() {}   // filled field by field on the host
+};
+struct CpOp {
+  int kind;
+  union {
     Proj pj;
     Outer ou;
   };
-  DevOp() {}   // filled field by field (after a memset) on the host
-  int g, nsplit;
-  int64_t chunk;
-  void* partial;
-  int BG, CG, CH;
-  int64_t eye_n;
-  int idx32;   // every index of the op fits 31 bits: decode with 32-bit math
+  CpOp() {}
 };
 
-constexpr int kMaxLevelOps = 34;   // ops per batched launch (parameter space)
+// The ops of one launch.  Most levels hold a few ops: they travel in a small
+// batch (about 4 KB of kernel parameters); a launch with the large one costs
+// 1 us more on the host and 2 to 3 us more on the device (measured with a
+// 31 KB batch against 4 KB).
+constexpr int kSmallOps = 8;
+constexpr int kLargeOps = 48;
 
+template <typename OpT, int CAP>
 struct LevelBatch {
   LevelBatch() {}
   int nops;
-  int64_t start[kMaxLevelOps + 1];   // prefix sums of blocks
-  DevOp ops[kMaxLevelOps];
+  int start[CAP + 1];   // prefix sums of blocks
+  OpT ops[CAP];
 };
 
 class Program {
