@@ -267,6 +267,7 @@ ttnn_status ttnn_plan_create(const ttnn_tree* tree, int32_t d, const int64_t* di
     need_u = std::max(need_u, cp_update_need(P));
   if ((s = run_recover(P, nullptr, nullptr, st, true, &need_r))) return fail(s);
   P.ws_bytes = need_u + 4096;
+  P.ws_limit = P.ws_bytes;
   if ((s = palloc((void**)&P.ws, P.ws_bytes)) != TTNN_OK) return fail(s);
   P.ws_rec_bytes = need_r + 4096;
   if ((s = palloc((void**)&P.ws_rec, P.ws_rec_bytes)) != TTNN_OK) return fail(s);

@@ -25,9 +25,9 @@ const char* last_error();
     }                                                                         \
   } while (0)
 
-#define TTNN_TRY(expr)                 \
+#define TTNN_TRY(...)                  \
   do {                                 \
-    ttnn_status s_ = (expr);           \
+    ttnn_status s_ = (__VA_ARGS__);    \
     if (s_ != TTNN_OK) return s_;      \
   } while (0)
 

@@ -130,6 +130,13 @@ ttnn_status ttnn_update_dense_static(ttnn_state_t S, const void* data, const int
   const cudaStream_t st = (cudaStream_t)stream;
   // the scratch this update needs (recorded once per box shape, then cached)
   int64_t need = 0;
+  const int64_t limit0 = P.ws_limit;
+  struct Restore {
+    ttnn_plan_s& P;
+    int64_t limit;
+    ~Restore() { P.ws_limit = limit; }
+  } restore{P, limit0};
+  P.ws_limit = kStaticScratchBytes;
   TTNN_TRY(dense_update_need(P, b, &need));
   TTNN_CHECK_ARG(need <= kStaticScratchBytes,
                  "this update needs %lld bytes of scratch; ttnn_update_dense_static has %lld "

@@ -499,10 +499,10 @@ struct Geometry {
 
 ttnn_status smem_limit_once(const void* func, int slot) {
   static std::mutex mu;
-  static bool done[4][64] = {};
+  static bool done[24][64] = {};
   int dev = 0;
   TTNN_TRY_CUDA(cudaGetDevice(&dev));
-  if (slot < 0 || slot >= 4 || dev < 0 || dev >= 64) {
+  if (slot < 0 || slot >= 24 || dev < 0 || dev >= 64) {
     set_error("internal: shared-memory limit slot");
     return TTNN_EUNSUPPORTED;
   }

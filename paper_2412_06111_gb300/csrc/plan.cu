@@ -9,8 +9,10 @@
 #include <functional>
 #include <numeric>
 
+#include "gemm_tc.cuh"
 #include "plan.cuh"
 #include "program.cuh"
+#include "tc_ptx.cuh"
 
 namespace ttnn {
 
@@ -1071,6 +1073,12 @@ static void side_spec_common(ttnn_plan_s& P, const Box& box, int lo, int hi, Sid
   s.store = P.side_store;
 }
 
+// Smallest tensor or box (entries) whose products take the tensor-core GEMM
+// rather than the SIMT one: its three extra launches pay from about there
+// (2.4e6 bfloat16 entries 77 against 87 us per update, 2.7e6 binary32 ones
+// 129 against 128, 4.9e6 of either 106 against 148; 1.3e5: 89 against 83).
+constexpr int64_t kTcgMinEntries = int64_t(1) << 21;
+
 static int store_bytes(int store) { return store == 0 ? 8 : store == 1 ? 4 : store == 2 ? 2 : 1; }
 
 ttnn_status make_side(ttnn_plan_s& P, const Box& box, int which, void* out, int64_t ld,
@@ -1159,6 +1167,7 @@ ttnn_status UpdateBatch::launch(cudaStream_t st) {
 ttnn_status dense_update_need(ttnn_plan_s& P, const Box& box, int64_t* need) {
   std::vector<int64_t> key = box.ext;
   key.push_back(box.full ? 1 : 0);
+  key.push_back(P.ws_limit);
   auto it = P.ws_need_cache.find(key);
   if (it != P.ws_need_cache.end()) {
     *need = it->second;
@@ -1330,6 +1339,40 @@ ttnn_status run_dense_update(ttnn_plan_s& P, void* acc, const void* data, const 
   const bool use_tc = (P.tc_ok || f32s) && !(P.flags & TTNN_FLAG_SIMT_PASS) &&
                       (cvt ? cvt_pass_supported(P, nL, nR) : tc_pass_supported(P, nL, nR)) ==
                           TTNN_OK;
+  // the tensor-core GEMM, for boxes the passes above do not take
+  TcGemm tg[2];
+  int ntg = 0;
+  bool tcg = !r1 && !P.walk_f64 && (P.pass_store == 1 || P.pass_store == 2) &&
+             P.dtype != TTNN_BF16X2 && !(P.flags & TTNN_FLAG_SIMT_PASS) &&
+             nL * nR >= kTcgMinEntries;
+  int64_t tcg_need = 0;
+  if (tcg) {
+    if (P.wR > 0) {
+      TcGemm& t = tg[ntg++];
+      t.I = nL; t.Jn = P.wR; t.K = nR;
+      t.A = data; t.lda = nR; t.mn = 0; t.type = P.pass_store;
+      t.B = sR; t.ldb = nR; t.C = (float*)D1; t.ldc = P.wRpad;
+    }
+    if (P.wL > 0) {
+      TcGemm& t = tg[ntg++];
+      t.I = nR; t.Jn = P.wL; t.K = nL;
+      t.A = data; t.lda = nR; t.mn = 1; t.type = P.pass_store;
+      t.B = sL; t.ldb = nL; t.C = (float*)D2; t.ldc = P.wLpad;
+    }
+    tcg = ntg > 0;
+    for (int k = 0; k < ntg; ++k) tcg = tcg && tcg_supported(tg[k]);
+  }
+  if (tcg) {
+    TTNN_TRY(launch_tcg(tg, ntg, tc::sm_count(), nullptr, 0, nullptr, 0, st, true, &tcg_need));
+    if (P.ws_limit == INT64_MAX) {
+      // sizing: room for the odd-sized boxes of this tensor too (the need
+      // grows with the extents)
+      const int64_t mark = ws.top;
+      ws.alloc(tcg_need);
+      ws.top = mark;
+    }
+    tcg = !use_tc && round_up(ws.top, 256) + tcg_need <= P.ws_limit;
+  }
   if (r1) {
     const int64_t mark = ws.top;
     SideSpec gs;
@@ -1392,8 +1435,24 @@ ttnn_status run_dense_update(ttnn_plan_s& P, void* acc, const void* data, const 
       return TTNN_EUNSUPPORTED;
     }
     const int in_type = P.pass_store == 0 ? 0 : P.pass_store == 1 ? 1 : 2;
-    if (!dry) ++P.n_simt_pass;
-    if (P.wR > 0) {
+    if (!dry) ++(tcg ? P.n_tc_pass : P.n_simt_pass);
+    if (tcg) {
+      const int64_t mark = ws.top;
+      int* const err = P.err_dev;
+      const uint64_t wait_ns = (P.flags & TTNN_FLAG_WAIT_TEST) ? 0 : tc::kTimeoutNs;
+      const int64_t need = tcg_need;
+      char* tw = ws.alloc(need);
+      if (!dry) {
+        const int sms = tc::pass_sms(P);
+        auto go = [tg, ntg, sms, err, wait_ns, tw, need](cudaStream_t s) {
+          return launch_tcg(tg, ntg, sms, err, wait_ns, tw, need, s, false, nullptr);
+        };
+        if (batch) batch->passes.push_back(go);
+        else TTNN_TRY(go(st));
+      }
+      ws.top = mark;
+    }
+    if (P.wR > 0 && !tcg) {
       Gemm g;
       g.I = nL; g.Jn = P.wR; g.K = nR;
       g.A = data; g.asi = nR; g.ask = 1;
@@ -1408,7 +1467,7 @@ ttnn_status run_dense_update(ttnn_plan_s& P, void* acc, const void* data, const 
       }
       ws.top = mark;
     }
-    if (P.wL > 0) {
+    if (P.wL > 0 && !tcg) {
       Gemm g;
       g.I = nR; g.Jn = P.wL; g.K = nL;
       g.A = data; g.asi = 1; g.ask = nR;

@@ -73,12 +73,17 @@ struct ttnn_plan_s {
   void* dxy = nullptr;          // unstructured DRMs of every node, walk type (TTNN_FLAG_DENSE_DRM)
   char* ws = nullptr;
   int64_t ws_bytes = 0;
+  // scratch an update may plan with: unbounded while the plan is created
+  // (its workspace is sized then), later that workspace's size.  Forms that
+  // need more than the one they replace are taken only within it.
+  int64_t ws_limit = INT64_MAX;
   // the recovery's own scratch: a recovery may run on another stream while
   // the next update of another state of the plan uses `ws`
   char* ws_rec = nullptr;
   int64_t ws_rec_bytes = 0;
   int64_t dev_bytes = 0;        // device memory the plan holds (all its allocations)
-  // workspace bytes a dense update needs, by box extents (+ whole-tensor flag)
+  // workspace bytes a dense update needs, by box extents, whole-tensor flag
+  // and scratch limit
   std::map<std::vector<int64_t>, int64_t> ws_need_cache;
   ttnn::QrJob* jobs_dev = nullptr;
   std::vector<ttnn::QrJob> jobs_host;   // what jobs_dev holds (upload skipped when unchanged)
