@@ -60,6 +60,7 @@ static void free_plan(ttnn_plan_s* P) {
   cudaFree(P->xWo);
   cudaFree(P->sideRs);
   cudaFree(P->sideLs);
+  cudaFree(P->prep_block);
   cudaFree(P->dxy);
   cudaFree(P->ws);
   cudaFree(P->ws_rec);
@@ -242,6 +243,10 @@ ttnn_status ttnn_plan_create(const ttnn_tree* tree, int32_t d, const int64_t* di
       if ((s = launch_split_bf16((const float*)P.sideL, eL, P.sideLs, (char*)P.sideLs + eL * 2,
                                  st)) != TTNN_OK)
         return fail(s);
+    }
+    if (const int64_t bytes = tcg_plan_bytes(P)) {
+      if ((s = palloc(&P.prep_block, bytes)) != TTNN_OK) return fail(s);
+      if ((s = tcg_plan_prepare(P, st)) != TTNN_OK) return fail(s);
     }
     if (omega_via_d2(P, nL, nR)) {
       if ((s = palloc(&P.xWo, (int64_t)P.rXL * nR * (P.walk_f64 ? 8 : 4))) != TTNN_OK) return fail(s);

@@ -511,16 +511,15 @@ __global__ void __launch_bounds__(256) tcg_pieces_kernel(const float* part, int6
   const int64_t rows = min((int64_t)kTileM, I - (int64_t)it * kTileM);
   const int n4 = (int)(rows * Npad / 4);
   const int64_t tile4 = (int64_t)kTileM * Npad / 4;
+  // only the first CTA's range can begin in an earlier tile
   const float4* p4 = reinterpret_cast<const float4*>(part);
+  const float4* f4 = p4 + (int64_t)(2 * c0 + ((int)(total * c0 / G / nkt) < it)) * tile4;
   float4* o4 = reinterpret_cast<float4*>(C) + (int64_t)it * tile4;
-  // CTA c's piece of this tile: its first unless its range begins in an earlier one
-  auto piece = [&](int c) {
-    return p4 + (int64_t)(2 * c + ((int)(total * c / G / nkt) < it)) * tile4;
-  };
   for (int e = blockIdx.y * 256 + threadIdx.x; e < n4; e += gridDim.y * 256) {
-    float4 a = piece(c0)[e];
+    float4 a = f4[e];
+#pragma unroll 4
     for (int c = c0 + 1; c <= c1; ++c) {
-      const float4 v = piece(c)[e];
+      const float4 v = p4[(int64_t)(2 * c) * tile4 + e];
       a.x += v.x;
       a.y += v.y;
       a.z += v.z;
@@ -572,101 +571,124 @@ static ttnn_status tcg_major(bool mn, const TcgGeometry& o, const CUtensorMap& m
 }  // namespace tc
 
 bool tcg_supported(const TcGemm& g) {
+  if (g.type == 0) return zgemm_supported(g);
   const int64_t lim = int64_t(1) << 31;
   if ((g.type != 1 && g.type != 2) || g.I < 1 || g.Jn < 1 || g.K < 1) return false;
   if (g.Jn > tc::kTcgMaxN || g.ldc != round_up(g.Jn, 16)) return false;
   // 32-bit tile counts and TMA coordinates
-  return g.I < lim - 256 && g.K < lim - 256 && ceil_div(g.I, (int64_t)128) * 608 < lim;
+  return g.I < lim - 256 && g.K < lim - 256;
 }
 
-ttnn_status launch_tcg(const TcGemm* g, int n, int sms, int* err, uint64_t wait_ns, void* ws,
-                       int64_t ws_bytes, cudaStream_t st, bool dry, int64_t* need) {
+int64_t tcg_prep_bytes(const TcGemm& g) {
+  return g.type == 0 ? zgemm_prep_bytes(g) : tc::tcg_geometry(g, 1).b_bytes;
+}
+
+ttnn_status tcg_prepare(const TcGemm* g, int n, void* const* dst, cudaStream_t st) {
   using namespace tc;
-  TcgGeometry o[2];
-  int64_t b_bytes = 0, p_bytes = 0;
-  for (int k = 0; k < n; ++k) {
-    o[k] = tcg_geometry(g[k], sms);
-    b_bytes += o[k].b_bytes;
-    p_bytes = std::max(p_bytes, o[k].p_bytes);   // the products run in order
-  }
-  if (dry) {
-    *need = b_bytes + p_bytes + 256;
-    return TTNN_OK;
-  }
-  char* w = (char*)ws + (256 - ((uintptr_t)ws & 255)) % 256;
-  if (w + b_bytes + p_bytes > (char*)ws + ws_bytes) {
-    set_error("tensor-core GEMM: workspace too small");
-    return TTNN_ENOMEM;
-  }
+  if (g[0].type == 0) return zgemm_prepare(g, n, dst, st);
   PrepBatch pb;
   pb.n = n;
   pb.type = g[0].type;
-  int64_t blocks = 0, at = 0;
+  int64_t blocks = 0;
   for (int k = 0; k < n; ++k) {
+    const TcgGeometry o = tcg_geometry(g[k], 1);
     PrepJob& j = pb.job[k];
     j.src = g[k].B;
-    j.dst = (uint16_t*)(w + at);
+    j.dst = (uint16_t*)dst[k];
     j.ldb = g[k].ldb;
     j.K = g[k].K;
-    j.Kpad = o[k].Kpad;
+    j.Kpad = o.Kpad;
     j.Jn = g[k].Jn;
-    j.Npad = o[k].Npad;
+    j.Npad = o.Npad;
     j.start = blocks;
     blocks += ceil_div(j.Npad * j.Kpad / 2, (int64_t)256 * kPrepPairs);
-    at += o[k].b_bytes;
   }
   if (blocks >= (int64_t(1) << 31)) {
     set_error("tensor-core GEMM: operand too large");
     return TTNN_EUNSUPPORTED;
   }
   tcg_prepare_kernel<<<(unsigned)blocks, 256, 0, st>>>(pb);
-  TTNN_TRY(check_launch("tcg_prepare_kernel"));
-  float* part = (float*)(w + b_bytes);
+  return check_launch("tcg_prepare_kernel");
+}
+
+static ttnn_status launch_tcg_one(const TcGemm& g, const void* prep, void* pieces, int sms, int* err,
+                                  uint64_t wait_ns, cudaStream_t st) {
+  using namespace tc;
+  const TcgGeometry o = tcg_geometry(g, sms);
+  CUtensorMap mB;
+  TTNN_TRY(encode_map(&mB, prep, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2, o.Kpad, (int64_t)o.NS * o.Npad,
+                      64u, (uint32_t)o.Npad, CU_TENSOR_MAP_SWIZZLE_128B));
+  TcgParams p;
+  p.A = g.A;
+  p.lda = g.lda;
+  p.I = g.I;
+  p.K = g.K;
+  p.nI = o.nI;
+  p.nkt = o.nkt;
+  p.Npad = o.Npad;
+  p.stages = o.stages;
+  // Chain of leading products per drain: 128 k (8 MMAs).  Long binary32
+  // reductions take 256: their sums err less than the SIMT GEMM's by more
+  // than the longer chain adds (64^4 x 8 slab: 4.2e-7 against 9.8e-7; short
+  // ones would lose that margin), and the drains cost 10 % of the time.
+  p.group = g.type == 2 ? 1 : g.K >= 2048 ? 4 : 2;
+  p.C = (float*)g.C;
+  p.part = (float*)pieces;
+  p.err = err;
+  p.wait_ns = wait_ns;
+  const int64_t inner = g.mn ? g.I : g.K;
+  const int pair = g.type == 2 ? 4 : 8;
+  const bool vec = inner % 2 == 0 && g.lda % 2 == 0 && (uintptr_t)g.A % pair == 0;
+  const bool mn = g.mn != 0, wide = o.Npad > 64;
+  if (g.type == 2 && vec)
+    TTNN_TRY(wide ? tcg_major<uint16_t, true, kTcgMaxN>(mn, o, mB, p, st)
+                  : tcg_major<uint16_t, true, 64>(mn, o, mB, p, st));
+  else if (g.type == 2)
+    TTNN_TRY(wide ? tcg_major<uint16_t, false, kTcgMaxN>(mn, o, mB, p, st)
+                  : tcg_major<uint16_t, false, 64>(mn, o, mB, p, st));
+  else if (vec)
+    TTNN_TRY(wide ? tcg_major<float, true, kTcgMaxN>(mn, o, mB, p, st)
+                  : tcg_major<float, true, 64>(mn, o, mB, p, st));
+  else
+    TTNN_TRY(wide ? tcg_major<float, false, kTcgMaxN>(mn, o, mB, p, st)
+                  : tcg_major<float, false, 64>(mn, o, mB, p, st));
+  if (o.grid == 1) return TTNN_OK;
+  const int per = (int)std::max<int64_t>(1, std::min<int64_t>(8, 608 / std::max(1, o.nI)));
+  tcg_pieces_kernel<<<dim3((unsigned)o.nI, (unsigned)per), 256, 0, st>>>(
+      (const float*)pieces, g.I, o.nI, o.nkt, o.grid, o.Npad, (float*)g.C);
+  return check_launch("tcg_pieces_kernel");
+}
+
+ttnn_status launch_tcg(const TcGemm* g, int n, int sms, int* err, uint64_t wait_ns, void* ws,
+                       int64_t ws_bytes, cudaStream_t st, bool dry, int64_t* need) {
+  int64_t b_bytes = 0, p_bytes = 0;
+  void* dst[2] = {nullptr, nullptr};
+  TcGemm todo[2];
+  int nt = 0;
+  char* w = (char*)ws + (256 - ((uintptr_t)ws & 255)) % 256;
   for (int k = 0; k < n; ++k) {
-    CUtensorMap mB;
-    TTNN_TRY(encode_map(&mB, pb.job[k].dst, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2, o[k].Kpad,
-                        (int64_t)o[k].NS * o[k].Npad, 64u, (uint32_t)o[k].Npad,
-                        CU_TENSOR_MAP_SWIZZLE_128B));
-    TcgParams p;
-    p.A = g[k].A;
-    p.lda = g[k].lda;
-    p.I = g[k].I;
-    p.K = g[k].K;
-    p.nI = o[k].nI;
-    p.nkt = o[k].nkt;
-    p.Npad = o[k].Npad;
-    p.stages = o[k].stages;
-    // Chain of leading products per drain: 128 k (8 MMAs).  Long binary32
-    // reductions take 256: their sums err less than the SIMT GEMM's by more
-    // than the longer chain adds (64^4 x 8 slab: 4.2e-7 against 9.8e-7; short
-    // ones would lose that margin), and the drains cost 10 % of the time.
-    p.group = g[k].type == 2 ? 1 : g[k].K >= 2048 ? 4 : 2;
-    p.C = g[k].C;
-    p.part = part;
-    p.err = err;
-    p.wait_ns = wait_ns;
-    const int64_t inner = g[k].mn ? g[k].I : g[k].K;
-    const int pair = g[k].type == 2 ? 4 : 8;
-    const bool vec = inner % 2 == 0 && g[k].lda % 2 == 0 && (uintptr_t)g[k].A % pair == 0;
-    const bool mn = g[k].mn != 0, wide = o[k].Npad > 64;
-    if (g[k].type == 2 && vec)
-      TTNN_TRY(wide ? tcg_major<uint16_t, true, kTcgMaxN>(mn, o[k], mB, p, st)
-                    : tcg_major<uint16_t, true, 64>(mn, o[k], mB, p, st));
-    else if (g[k].type == 2)
-      TTNN_TRY(wide ? tcg_major<uint16_t, false, kTcgMaxN>(mn, o[k], mB, p, st)
-                    : tcg_major<uint16_t, false, 64>(mn, o[k], mB, p, st));
-    else if (vec)
-      TTNN_TRY(wide ? tcg_major<float, true, kTcgMaxN>(mn, o[k], mB, p, st)
-                    : tcg_major<float, true, 64>(mn, o[k], mB, p, st));
-    else
-      TTNN_TRY(wide ? tcg_major<float, false, kTcgMaxN>(mn, o[k], mB, p, st)
-                    : tcg_major<float, false, 64>(mn, o[k], mB, p, st));
-    if (o[k].grid > 1) {
-      const int per = (int)std::max<int64_t>(1, std::min<int64_t>(8, 608 / std::max(1, o[k].nI)));
-      tcg_pieces_kernel<<<dim3((unsigned)o[k].nI, (unsigned)per), 256, 0, st>>>(
-          part, g[k].I, o[k].nI, o[k].nkt, o[k].grid, o[k].Npad, g[k].C);
-      TTNN_TRY(check_launch("tcg_pieces_kernel"));
-    }
+    // the products run in order and share the room of their pieces
+    p_bytes = std::max(p_bytes, g[k].type == 0 ? zgemm_piece_bytes(g[k], sms)
+                                               : tc::tcg_geometry(g[k], sms).p_bytes);
+    if (g[k].prep) continue;
+    todo[nt] = g[k];
+    dst[nt++] = w + b_bytes;
+    b_bytes += tcg_prep_bytes(g[k]);
+  }
+  if (dry) {
+    *need = b_bytes + p_bytes + 256;
+    return TTNN_OK;
+  }
+  if (w + b_bytes + p_bytes > (char*)ws + ws_bytes) {
+    set_error("tensor-core GEMM: workspace too small");
+    return TTNN_ENOMEM;
+  }
+  if (nt > 0) TTNN_TRY(tcg_prepare(todo, nt, dst, st));
+  nt = 0;
+  for (int k = 0; k < n; ++k) {
+    const void* prep = g[k].prep ? g[k].prep : dst[nt++];
+    TTNN_TRY(g[k].type == 0 ? launch_zgemm(g[k], prep, w + b_bytes, sms, err, wait_ns, st)
+                            : launch_tcg_one(g[k], prep, w + b_bytes, sms, err, wait_ns, st));
   }
   return TTNN_OK;
 }

@@ -497,19 +497,19 @@ struct Geometry {
   size_t smem;
 };
 
-ttnn_status smem_limit_once(const void* func, int slot) {
+ttnn_status smem_limit_once(const void* func, int slot, int bytes) {
   static std::mutex mu;
-  static bool done[24][64] = {};
+  static bool done[32][64] = {};
   int dev = 0;
   TTNN_TRY_CUDA(cudaGetDevice(&dev));
-  if (slot < 0 || slot >= 24 || dev < 0 || dev >= 64) {
+  if (slot < 0 || slot >= 32 || dev < 0 || dev >= 64) {
     set_error("internal: shared-memory limit slot");
     return TTNN_EUNSUPPORTED;
   }
   std::lock_guard<std::mutex> lk(mu);
   if (!done[slot][dev]) {
     TTNN_TRY_CUDA(cudaFuncSetAttribute(func, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                       kSmemBudget));
+                                       bytes));
     done[slot][dev] = true;
   }
   return TTNN_OK;

@@ -1073,12 +1073,6 @@ static void side_spec_common(ttnn_plan_s& P, const Box& box, int lo, int hi, Sid
   s.store = P.side_store;
 }
 
-// Smallest tensor or box (entries) whose products take the tensor-core GEMM
-// rather than the SIMT one: its three extra launches pay from about there
-// (2.4e6 bfloat16 entries 77 against 87 us per update, 2.7e6 binary32 ones
-// 129 against 128, 4.9e6 of either 106 against 148; 1.3e5: 89 against 83).
-constexpr int64_t kTcgMinEntries = int64_t(1) << 21;
-
 static int store_bytes(int store) { return store == 0 ? 8 : store == 1 ? 4 : store == 2 ? 2 : 1; }
 
 ttnn_status make_side(ttnn_plan_s& P, const Box& box, int which, void* out, int64_t ld,
@@ -1156,6 +1150,77 @@ bool omega_via_d2(const ttnn_plan_s& P, int64_t nL, int64_t nR) {
   const TNode& yc = P.nodes[P.ychild];
   return P.yside == 1 && !P.walk_f64 && !yc.identity && P.wYL > 0 && P.rXL > 0 &&
          yc.r <= P.rXL && nR * 2 <= nL && !(P.flags & TTNN_FLAG_DENSE_DRM);
+}
+
+// Smallest tensor or box (entries) whose products take the tensor-core GEMM
+// rather than the SIMT one: its three extra launches pay from about there
+// (2.4e6 bfloat16 entries 77 against 87 us per update, 2.7e6 binary32 ones
+// 129 against 128, 4.9e6 of either 106 against 148; 1.3e5: 89 against 83).
+constexpr int64_t kTcgMinEntries = int64_t(1) << 21;
+// The same for binary64 (64 entries: 58 against 56 us per update, 1296: 61
+// against 92, 24^4: 83 against 124, 20^6: 1003 against 6036).
+constexpr int64_t kZgemmMinEntries = 1024;
+
+// The products of an nL x nR box as tensor-core GEMMs (operand pointers left
+// empty); false where they are not taken.
+static bool tcg_products(const ttnn_plan_s& P, int64_t nL, int64_t nR, TcGemm* tg, int* n) {
+  *n = 0;
+  if (P.pass_store > 2 || P.dtype == TTNN_BF16X2 || (P.flags & TTNN_FLAG_SIMT_PASS)) return false;
+  if (nL * nR < (P.walk_f64 ? kZgemmMinEntries : kTcgMinEntries)) return false;
+  if (P.wR > 0) {   // D1 = M B_R^T
+    TcGemm& t = tg[(*n)++];
+    t = TcGemm();
+    t.I = nL; t.Jn = P.wR; t.K = nR;
+    t.lda = nR; t.mn = 0; t.type = P.pass_store;
+    t.ldb = nR; t.ldc = P.wRpad;
+  }
+  if (P.wL > 0) {   // D2 = M^T B_L^T
+    TcGemm& t = tg[(*n)++];
+    t = TcGemm();
+    t.I = nR; t.Jn = P.wL; t.K = nL;
+    t.lda = nR; t.mn = 1; t.type = P.pass_store;
+    t.ldb = nL; t.ldc = P.wLpad;
+  }
+  for (int k = 0; k < *n; ++k)
+    if (!tcg_supported(tg[k])) return false;
+  return *n > 0;
+}
+
+// The prepared operands of whole-tensor updates that take the tensor-core
+// GEMM, kept with the cached side blocks (256-byte aligned parts of one
+// allocation, P.prep[0] for D1 and P.prep[1] for D2).
+static bool full_products(const ttnn_plan_s& P, TcGemm* tg, int* n) {
+  int64_t nL = 1, nR = 1;
+  for (int m = P.Llo; m < P.Lhi; ++m) nL *= P.dims[m];
+  for (int m = P.Rlo; m < P.Rhi; ++m) nR *= P.dims[m];
+  if (nL == 1 || nR == 1 || !tcg_products(P, nL, nR, tg, n)) return false;
+  const bool passes = P.dtype == TTNN_F32 ? P.sideRs && cvt_pass_supported(P, nL, nR) == TTNN_OK
+                                          : tc_pass_supported(P, nL, nR) == TTNN_OK;
+  return !passes;
+}
+
+int64_t tcg_plan_bytes(const ttnn_plan_s& P) {
+  TcGemm tg[2];
+  int n;
+  if (!P.sideR || (P.wL > 0 && !P.sideL) || !full_products(P, tg, &n)) return 0;
+  int64_t b = 0;
+  for (int k = 0; k < n; ++k) b += tcg_prep_bytes(tg[k]);
+  return b;
+}
+
+ttnn_status tcg_plan_prepare(ttnn_plan_s& P, cudaStream_t st) {
+  TcGemm tg[2];
+  int n;
+  if (!full_products(P, tg, &n)) return TTNN_OK;
+  void* dst[2];
+  char* at = (char*)P.prep_block;
+  for (int k = 0; k < n; ++k) {
+    tg[k].B = tg[k].mn ? P.sideL : P.sideR;
+    dst[k] = at;
+    P.prep[tg[k].mn] = at;
+    at += tcg_prep_bytes(tg[k]);
+  }
+  return tcg_prepare(tg, n, dst, st);
 }
 
 ttnn_status UpdateBatch::launch(cudaStream_t st) {
@@ -1342,35 +1407,18 @@ ttnn_status run_dense_update(ttnn_plan_s& P, void* acc, const void* data, const 
   // the tensor-core GEMM, for boxes the passes above do not take
   TcGemm tg[2];
   int ntg = 0;
-  bool tcg = !r1 && !P.walk_f64 && (P.pass_store == 1 || P.pass_store == 2) &&
-             P.dtype != TTNN_BF16X2 && !(P.flags & TTNN_FLAG_SIMT_PASS) &&
-             nL * nR >= kTcgMinEntries;
+  bool tcg = !r1 && tcg_products(P, nL, nR, tg, &ntg);
   int64_t tcg_need = 0;
   if (tcg) {
-    if (P.wR > 0) {
-      TcGemm& t = tg[ntg++];
-      t.I = nL; t.Jn = P.wR; t.K = nR;
-      t.A = data; t.lda = nR; t.mn = 0; t.type = P.pass_store;
-      t.B = sR; t.ldb = nR; t.C = (float*)D1; t.ldc = P.wRpad;
+    for (int k = 0; k < ntg; ++k) {
+      tg[k].A = data;
+      tg[k].B = tg[k].mn ? sL : sR;
+      tg[k].C = tg[k].mn ? D2 : D1;
+      if (box.full && P.prep[tg[k].mn]) tg[k].prep = P.prep[tg[k].mn];
     }
-    if (P.wL > 0) {
-      TcGemm& t = tg[ntg++];
-      t.I = nR; t.Jn = P.wL; t.K = nL;
-      t.A = data; t.lda = nR; t.mn = 1; t.type = P.pass_store;
-      t.B = sL; t.ldb = nL; t.C = (float*)D2; t.ldc = P.wLpad;
-    }
-    tcg = ntg > 0;
-    for (int k = 0; k < ntg; ++k) tcg = tcg && tcg_supported(tg[k]);
   }
   if (tcg) {
     TTNN_TRY(launch_tcg(tg, ntg, tc::sm_count(), nullptr, 0, nullptr, 0, st, true, &tcg_need));
-    if (P.ws_limit == INT64_MAX) {
-      // sizing: room for the odd-sized boxes of this tensor too (the need
-      // grows with the extents)
-      const int64_t mark = ws.top;
-      ws.alloc(tcg_need);
-      ws.top = mark;
-    }
     tcg = !use_tc && round_up(ws.top, 256) + tcg_need <= P.ws_limit;
   }
   if (r1) {

@@ -70,6 +70,9 @@ struct ttnn_plan_s {
   // tensor-core pass of whole-tensor updates)
   void* sideRs = nullptr;
   void* sideLs = nullptr;
+  // whole-tensor updates on the tensor-core GEMM: its prepared operands
+  void* prep_block = nullptr;
+  void* prep[2] = {nullptr, nullptr};
   void* dxy = nullptr;          // unstructured DRMs of every node, walk type (TTNN_FLAG_DENSE_DRM)
   char* ws = nullptr;
   int64_t ws_bytes = 0;
@@ -181,6 +184,10 @@ ttnn_status launch_quantize_fp8(const float* src, int64_t rows, int64_t cols, ui
 ttnn_status make_side(ttnn_plan_s& P, const Box& box, int which, void* out, int64_t ld,
                       cudaStream_t st, std::vector<GatherJob>* defer = nullptr);
 ttnn_status launch_split_bf16(const float* src, int64_t n, void* hi, void* lo, cudaStream_t st);
+// Device bytes of those prepared operands (0: none), and their preparation
+// into P.prep_block once the side blocks are there.
+int64_t tcg_plan_bytes(const ttnn_plan_s& P);
+ttnn_status tcg_plan_prepare(ttnn_plan_s& P, cudaStream_t st);
 ttnn_status make_side_xo(ttnn_plan_s& P, const Box& box, void* out, int64_t ld, cudaStream_t st);
 // Omega of an L-side Y child is taken through D2 (a reduction over the R
 // index) for whole 2-D boxes of nL x nR

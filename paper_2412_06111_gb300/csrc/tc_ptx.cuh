@@ -92,6 +92,11 @@ __host__ __device__ constexpr uint32_t idesc_bf16(int M, int N, bool a_mn_major)
          ((uint32_t)(N >> 3) << 17) | ((uint32_t)(M >> 4) << 24);
 }
 
+// The same for binary16 operands (formats 0).
+__host__ __device__ constexpr uint32_t idesc_f16(int M, int N, bool a_mn_major) {
+  return idesc_bf16(M, N, a_mn_major) & ~((1u << 7) | (1u << 10));
+}
+
 __device__ __forceinline__ void mma_bf16(uint32_t d_tmem, uint64_t a, uint64_t b, uint32_t idesc,
                                          uint32_t accumulate) {
   asm volatile(
@@ -124,10 +129,11 @@ __device__ __forceinline__ void tmem_wait_ld() {
 }
 
 // Host helpers (pass_tc.cu).
-// Raises a kernel's dynamic shared memory limit to kSmemBudget, once per
+// Raises a kernel's dynamic shared memory limit (to kSmemBudget unless its
+// static shared memory leaves less), once per
 // device.  Setting it per launch to the launch's own size would race between
 // host threads launching the same kernel with different sizes.
-ttnn_status smem_limit_once(const void* func, int slot);
+ttnn_status smem_limit_once(const void* func, int slot, int bytes = kSmemBudget);
 ttnn_status encode_map(CUtensorMap* m, const void* ptr, CUtensorMapDataType dt, int esize,
                        int64_t inner, int64_t outer, uint32_t box_inner, uint32_t box_outer,
                        CUtensorMapSwizzle sw);
