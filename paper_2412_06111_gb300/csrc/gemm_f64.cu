@@ -627,7 +627,7 @@ static ZGeometry z_geometry(const TcGemm& g, int sms) {
 
 template <bool MN, bool VEC>
 static ttnn_status z_launch(const ZGeometry& o, const CUtensorMap& mB, const ZParams& p, cudaStream_t st) {
-  constexpr int slot = 20 + (MN ? 2 : 0) + (VEC ? 1 : 0);
+  constexpr int slot = 32 + (MN ? 2 : 0) + (VEC ? 1 : 0);
   TTNN_TRY(smem_limit_once((const void*)zgemm_kernel<MN, VEC>, slot, kZSmem));
   zgemm_kernel<MN, VEC><<<o.grid, kZThreads, o.smem, st>>>(mB, p);
   return check_launch("zgemm_kernel");
@@ -638,6 +638,7 @@ static ttnn_status z_launch(const ZGeometry& o, const CUtensorMap& mB, const ZPa
 bool zgemm_supported(const TcGemm& g) {
   const int64_t lim = int64_t(1) << 31;
   if (g.type != 0 || g.I < 1 || g.Jn < 1 || g.K < 1 || g.Jn > 256) return false;
+  if (g.trans || g.nb != 1 || g.b[0].nkr || g.b[0].sk != 1) return false;
   // 64-bit integer sums of 2^46 per drain of 32 k; 32-bit tile counts
   return g.K <= (int64_t(1) << 21) && g.I < lim - 256 && g.ldc == round_up(g.Jn, 16);
 }
@@ -653,13 +654,13 @@ ttnn_status zgemm_prepare(const TcGemm* g, int n, void* const* dst, cudaStream_t
   for (int k = 0; k < n; ++k) {
     const ZGeometry o = z_geometry(g[k], 1);
     ZPrepJob& j = b.job[k];
-    j.B = (const double*)g[k].B;
+    j.B = (const double*)g[k].b[0].p;
     j.eb = (uint32_t*)dst[k];
     j.out = (uint32_t*)((char*)dst[k] + kZExpBytes);
-    j.ldb = g[k].ldb;
+    j.ldb = g[k].b[0].sj;
     j.K = g[k].K;
     j.Kpad = o.Kpad;
-    j.Jn = (int)g[k].Jn;
+    j.Jn = g[k].Jn;
     j.W = o.W;
     most = std::max(most, g[k].K);
     w = std::max(w, o.W);

@@ -6,12 +6,11 @@
 // products run on the tensor cores.
 //
 // Precision.  bfloat16 operands are multiplied as they are.  A binary32
-// operand is cut into three bfloat16 pieces that sum to it exactly (8 + 8 + 8
-// significand bits, each cut towards zero, so no piece overflows); the six
-// products down to 2^-16 of the leading one are formed, the other three
-// (2^-24 and below) are left out.  The tensor core truncates when it adds to
-// its binary32 accumulator, so chains are short: the leading products of 128
-// k go into one accumulator, those of each lower order into another, and the
+// operand is cut into three bfloat16 pieces that sum to it exactly (cut3); the
+// six products down to 2^-16 of the leading one are formed, the other three
+// (2^-24 and below, of either sign) are left out.  The tensor core truncates when it adds to
+// its binary32 accumulator, so chains are short: the leading products of 32 to
+// 256 k go into one accumulator, those of each lower order into another, and the
 // epilogue warps add them to registers with rounding to nearest.  The pieces
 // of B sit below one another in shared memory, so piece i of A meets all the
 // pieces of B it is multiplied with in one MMA of up to three times the
@@ -20,13 +19,14 @@
 // instead of six.
 //
 // Warp roles: warp 0 copies B tiles by TMA, warp 1 owns TMEM and issues the
-// MMAs, warps 2-5 drain accumulators (TMEM lane quarter = warp % 4), the
-// other 16 (8) load, convert and store A tiles (128-byte swizzle).  Every
-// wait is bounded; on expiry the kernel sets an error bit, drains its own
-// copies and MMAs, frees TMEM and returns.
+// MMAs, the next 4 or 8 drain accumulators (TMEM lane quarter = warp % 4), the
+// last 16 load, convert and store A tiles (128-byte swizzle).  Every wait is
+// bounded; on expiry the kernel sets an error bit, drains its own copies and
+// MMAs, frees TMEM and returns.
 #include <cuda_bf16.h>
 
 #include <algorithm>
+#include <type_traits>
 
 #include "gemm_tc.cuh"
 #include "tc_ptx.cuh"
@@ -34,26 +34,52 @@
 namespace ttnn {
 namespace tc {
 
-constexpr int kTcgMaxN = 80;      // columns an epilogue thread accumulates
-// Converter warps: 16 hide the most latency; products wider than 64 columns
-// need the registers of eight of them for the epilogue's sums.
-template <int NW>
-__host__ __device__ constexpr int tcg_conv_warps() { return NW <= 64 ? 16 : 8; }
-template <int NW>
-__host__ __device__ constexpr int tcg_threads() { return 192 + 32 * tcg_conv_warps<NW>(); }
+constexpr int kTcgMaxN = 80;      // columns of a product
+constexpr int kTcgConv = 16;      // converter warps (8 left the latency of the loads bare: twice the time)
+// Epilogue warps: one per lane quarter, or for products of more than 64
+// columns two (a half of the columns each: 80 sums do not fit the registers
+// that 16 converter warps leave; with two throughout, the converters spill).
+template <int EPI>
+__host__ __device__ constexpr int tcg_threads() { return 32 * (2 + EPI + kTcgConv); }
 constexpr int kTcgMaxStages = 6;
 
-struct TcgParams {
+struct TcgProb {
+  CUtensorMap mapB;
   const void* A;
   int64_t lda, I, K;
-  int nI, nkt;           // row tiles, k tiles
+  float* C;
+  int64_t ldc, unit0;    // first (row tile, k tile) of the product in the launch
+  int nkt, tile0;        // k tiles, first row tile in the launch
+  int chain;             // MMAs (of 16 k) per drain of the accumulators: 2 (not bfloat16), 4, 8 or 16
+  int trans;
+};
+struct TcgParams {
+  int n, tiles;          // products, row tiles of all of them
   int Npad, stages;
-  int group;             // k tiles per drain of the accumulators
-  float* C;              // [I][Npad]
+  int64_t units;         // (row tile, k tile) pairs of all of them
   float* part;           // pieces [2 grid][128][Npad]
   int* err;
   uint64_t wait_ns;
+  TcgProb prob[kTcgBatch];
 };
+static_assert(sizeof(TcgParams) <= 4096, "a launch's products travel in the kernel parameters");
+
+// The product of row tile `it` of the launch.
+__device__ __forceinline__ int tcg_prob(const TcgParams& p, int it) {
+  int q = 0;
+  while (q + 1 < p.n && it >= p.prob[q + 1].tile0) ++q;
+  return q;
+}
+// The row tile that holds unit u.
+__device__ __forceinline__ int tcg_tile(const TcgParams& p, int64_t u) {
+  int q = 0;
+  while (q + 1 < p.n && u >= p.prob[q + 1].unit0) ++q;
+  return p.prob[q].tile0 + (int)((u - p.prob[q].unit0) / p.prob[q].nkt);
+}
+// The first unit of row tile `it` (of product q).
+__device__ __forceinline__ int64_t tcg_unit(const TcgParams& p, int q, int it) {
+  return p.prob[q].unit0 + (int64_t)(it - p.prob[q].tile0) * p.prob[q].nkt;
+}
 
 // Shape of a form: pieces per element, k of a tile, accumulators, converter
 // groups (each converts a tile in turn; at most the number of stages, so that
@@ -67,6 +93,10 @@ struct Form<uint16_t> {
 template <>
 struct Form<float> {
   static constexpr int NS = 3, KT = 64, NACC = 3, NG = 2;
+};
+template <>
+struct Form<double> {   // rounded to binary32 on the way
+  static constexpr int NS = 3, KT = 64, NACC = 3, NG = 1;
 };
 
 // Two adjacent elements of a row, as loaded.  VEC: extents, stride and base
@@ -105,18 +135,36 @@ struct Pair<float, VEC> {
   }
 };
 
+template <bool VEC>
+struct Pair<double, VEC> {
+  double x, y;
+  __device__ void load(const double* p, bool a, bool b) {
+    if (VEC) {
+      const double2 v = a ? __ldg(reinterpret_cast<const double2*>(p)) : make_double2(0., 0.);
+      x = v.x;
+      y = v.y;
+    } else {
+      x = a ? __ldg(p) : 0.;
+      y = b ? __ldg(p + 1) : 0.;
+    }
+  }
+};
+
 // The three pieces of two binary32 values, packed (x in the low half).  The
-// rest of an infinity is NaN: a non-finite entry makes every result it
-// reaches NaN.
+// first is cut toward zero, so that no finite value overflows; the second is
+// rounded, which leaves the third either sign: the piece products left out
+// then average to nothing (a 200-rank tree's Psi erred by 6.2e-7 with both cut
+// toward zero, 4.8e-7 so).  The rest of an infinity is NaN: a non-finite entry
+// makes every result it reaches NaN.
 __device__ __forceinline__ void cut3(float x, float y, uint32_t* w) {
   const uint32_t ux = __float_as_uint(x), uy = __float_as_uint(y);
   w[0] = __byte_perm(ux, uy, 0x7632);
   x -= __uint_as_float(ux & 0xFFFF0000u);
   y -= __uint_as_float(uy & 0xFFFF0000u);
-  const uint32_t vx = __float_as_uint(x), vy = __float_as_uint(y);
-  w[1] = __byte_perm(vx, vy, 0x7632);
-  x -= __uint_as_float(vx & 0xFFFF0000u);
-  y -= __uint_as_float(vy & 0xFFFF0000u);
+  const __nv_bfloat162 v = __floats2bfloat162_rn(x, y);
+  w[1] = *reinterpret_cast<const uint32_t*>(&v);
+  x -= __uint_as_float(w[1] << 16);
+  y -= __uint_as_float(w[1] & 0xFFFF0000u);
   w[2] = __byte_perm(__float_as_uint(x), __float_as_uint(y), 0x7632);
 }
 
@@ -131,16 +179,17 @@ __device__ __forceinline__ void tmem_ld8(uint32_t taddr, uint32_t* r) {
       : "r"(taddr));
 }
 
-// NW: the columns an epilogue thread holds sums of (Npad <= NW).
-template <typename T, bool MN, bool VEC, int NW>
-__global__ void __launch_bounds__(tcg_threads<NW>(), 1)
-    tcg_kernel(const __grid_constant__ CUtensorMap mapB, const TcgParams p) {
+// EPI epilogue warps.
+template <typename T, bool MN, bool VEC, int EPI>
+__global__ void __launch_bounds__(tcg_threads<EPI>(), 1)
+    tcg_kernel(const __grid_constant__ TcgParams p) {
   using F = Form<T>;
+  constexpr int NW = EPI == 4 ? 64 : kTcgMaxN / 2;   // columns an epilogue thread holds sums of
   constexpr int NS = F::NS, KT = F::KT, NACC = F::NACC;
   constexpr int R = MN ? KT : kTileM;            // tile rows in memory order
   constexpr int CB = MN ? 2 : KT / 64;           // 64-column boxes of a row
   constexpr int NG = F::NG;                      // converter groups, a tile each in turn
-  constexpr int NCW = tcg_conv_warps<NW>() / NG; // warps of a group
+  constexpr int NCW = kTcgConv / NG;             // warps of a group
   constexpr int RW = R / NCW;                    // rows of a converter warp (4, 8 or 16)
   constexpr int NP = RW * CB;                    // pairs of a converter thread per tile
   constexpr uint32_t kBox = R * 128;             // bytes of a box
@@ -157,13 +206,12 @@ __global__ void __launch_bounds__(tcg_threads<NW>(), 1)
   const int S = p.stages;
   const uint32_t b_piece = (uint32_t)p.Npad * KT * 2;
   const uint32_t stage_bytes = NS * (kPiece + b_piece);
-  // The (row tile, k tile) grid in row-major order is cut into gridDim.x even
-  // ranges, one per CTA.  Row tiles within one range go to C; only the first
-  // and the last of a range can be pieces of a tile (slots 2 c and 2 c + 1 of
-  // CTA c), which are summed afterwards in CTA order.
-  const int64_t total = (int64_t)p.nI * p.nkt;
-  const int64_t u0 = total * blockIdx.x / gridDim.x, u1 = total * (blockIdx.x + 1) / gridDim.x;
-  const int i0 = (int)(u0 / p.nkt), i1 = u1 > u0 ? (int)((u1 - 1) / p.nkt) + 1 : i0;
+  // The (row tile, k tile) units of all products, in order, are cut into
+  // gridDim.x even ranges, one per CTA.  Row tiles within one range go to C;
+  // only the first and the last of a range can be pieces of a tile (slots 2 c
+  // and 2 c + 1 of CTA c), which are summed afterwards in CTA order.
+  const int64_t u0 = p.units * blockIdx.x / gridDim.x, u1 = p.units * (blockIdx.x + 1) / gridDim.x;
+  const int i0 = tcg_tile(p, u0), i1 = u1 > u0 ? tcg_tile(p, u1 - 1) + 1 : i0;
 
   if (threadIdx.x == 0) {
     abort_flag = 0;
@@ -174,7 +222,7 @@ __global__ void __launch_bounds__(tcg_threads<NW>(), 1)
     }
     for (int k = 0; k < 2; ++k) {
       mbar_init(smem_u32(&bar_full[k]), 1);
-      mbar_init(smem_u32(&bar_free[k]), 4);
+      mbar_init(smem_u32(&bar_free[k]), EPI);
     }
     mbar_init(smem_u32(&bar_done), 1);
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
@@ -190,11 +238,13 @@ __global__ void __launch_bounds__(tcg_threads<NW>(), 1)
   fence_after();
   const uint32_t tmem = tmem_slot;
 
-  // this CTA's k tiles of row tile `it`
+  // this CTA's k tiles of row tile `it`, and its product
   auto range = [&](int it, int* kt0, int* kt1) {
-    const int64_t r = (int64_t)it * p.nkt;
+    const int q = tcg_prob(p, it);
+    const int64_t r = tcg_unit(p, q, it);
     *kt0 = (int)(max(u0, r) - r);
-    *kt1 = (int)(min(u1, r + p.nkt) - r);
+    *kt1 = (int)(min(u1, r + p.prob[q].nkt) - r);
+    return q;
   };
 
   if (warp == 0) {
@@ -207,7 +257,7 @@ __global__ void __launch_bounds__(tcg_threads<NW>(), 1)
       bool ok = true;
       for (int it = i0; it < i1 && ok; ++it) {
         int kt0, kt1;
-        range(it, &kt0, &kt1);
+        const CUtensorMap* mapB = &p.prob[range(it, &kt0, &kt1)].mapB;
         for (int kt = kt0; kt < kt1; ++kt) {
           ok = mbar_wait(smem_u32(&bar_empty[stage]), ph ^ 1, &abort_flag, p.wait_ns);
           if (!ok) break;
@@ -218,7 +268,7 @@ __global__ void __launch_bounds__(tcg_threads<NW>(), 1)
           for (int s = 0; s < NS; ++s)
 #pragma unroll
             for (int h = 0; h < KT / 64; ++h)
-              tma_2d(sb + s * b_piece + h * (b_piece / (KT / 64)), &mapB, kt * KT + h * 64,
+              tma_2d(sb + s * b_piece + h * (b_piece / (KT / 64)), mapB, kt * KT + h * 64,
                      s * p.Npad, bar, pol_keep);
           used |= 1u << stage;
           last_ph = (last_ph & ~(1u << stage)) | (ph << stage);
@@ -245,44 +295,58 @@ __global__ void __launch_bounds__(tcg_threads<NW>(), 1)
       bool ok = true;
       for (int it = i0; it < i1 && ok; ++it) {
         int kt0, kt1;
-        range(it, &kt0, &kt1);
-        for (int g0 = kt0; g0 < kt1 && ok; g0 += p.group) {
-          ok = mbar_wait(smem_u32(&bar_free[buf]), fph, &abort_flag, p.wait_ns);
+        const int chain = p.prob[range(it, &kt0, &kt1)].chain;
+        int steps = 0;      // MMAs deep the accumulators at hand are
+        for (int kt = kt0; kt < kt1; ++kt) {
+          ok = mbar_wait(smem_u32(&bar_a[stage]), ph, &abort_flag, p.wait_ns) &&
+               mbar_wait(smem_u32(&bar_b[stage]), ph, &abort_flag, p.wait_ns);
           if (!ok) break;
-          fence_after();
-          const uint32_t d = tmem + buf * NACC * p.Npad;
-          const int g1 = min(g0 + p.group, kt1);
-          for (int kt = g0; kt < g1; ++kt) {
-            ok = mbar_wait(smem_u32(&bar_a[stage]), ph, &abort_flag, p.wait_ns) &&
-                 mbar_wait(smem_u32(&bar_b[stage]), ph, &abort_flag, p.wait_ns);
-            if (!ok) break;
+          const uint32_t sa = base + stage * stage_bytes;
+          const uint32_t sb = sa + NS * kPiece;
+          // the MMAs of `n` k steps from k0 on (unrolled: this thread's issue
+          // rate bounds the kernel when each drain is short)
+          auto issue = [&](auto first, auto count) {
+            constexpr int k0 = decltype(first)::value, n = decltype(count)::value;
+            if (steps == 0) {
+              ok = mbar_wait(smem_u32(&bar_free[buf]), fph, &abort_flag, p.wait_ns);
+              if (!ok) return;
+            }
             fence_after();
-            const uint32_t sa = base + stage * stage_bytes;
-            const uint32_t sb = sa + NS * kPiece;
+            const uint32_t d = tmem + buf * NACC * p.Npad;
 #pragma unroll
             for (int ia = 0; ia < NS; ++ia) {
               // piece ia of A against pieces 0 .. NS - 1 - ia of B: orders ia .. NS - 1
               const uint32_t id = idesc_bf16(kTileM, (NS - ia) * p.Npad, MN);
 #pragma unroll
-              for (int kk = 0; kk < KT / 16; ++kk) {
+              for (int kk = k0; kk < k0 + n; ++kk) {
                 const uint64_t da =
                     MN ? sdesc(sa + ia * kPiece + kk * 2048, kBox, 1024)
                        : sdesc(sa + ia * kPiece + (kk >> 2) * kBox + (kk & 3) * 32, 16, 1024);
                 const uint64_t db =
                     sdesc(sb + (kk >> 2) * (p.Npad * 128) + (kk & 3) * 32, 16, 1024);
-                mma_bf16(d + ia * p.Npad, da, db, id, kt > g0 || kk > 0 || ia > 0);
+                mma_bf16(d + ia * p.Npad, da, db, id, steps > 0 || kk > k0 || ia > 0);
               }
             }
-            mma_commit(smem_u32(&bar_empty[stage]));
-            if (++stage == S) {
-              stage = 0;
-              ph ^= 1;
+            steps += n;
+            if (steps >= chain || (kt + 1 == kt1 && k0 + n == KT / 16)) {
+              mma_commit(smem_u32(&bar_full[buf]));
+              buf ^= 1;
+              if (buf == 0) fph ^= 1;
+              steps = 0;
             }
+          };
+          if (chain >= KT / 16) {
+            issue(std::integral_constant<int, 0>(), std::integral_constant<int, KT / 16>());
+          } else if constexpr (NS > 1) {   // chains of two
+            issue(std::integral_constant<int, 0>(), std::integral_constant<int, 2>());
+            if (ok) issue(std::integral_constant<int, 2>(), std::integral_constant<int, 2>());
           }
           if (!ok) break;
-          mma_commit(smem_u32(&bar_full[buf]));
-          buf ^= 1;
-          if (buf == 0) fph ^= 1;
+          mma_commit(smem_u32(&bar_empty[stage]));
+          if (++stage == S) {
+            stage = 0;
+            ph ^= 1;
+          }
         }
       }
       if (!ok) {
@@ -291,11 +355,9 @@ __global__ void __launch_bounds__(tcg_threads<NW>(), 1)
       }
       mma_commit(smem_u32(&bar_done));
     }
-  } else if (warp >= 6) {
+  } else if (warp >= 2 + EPI) {
     // ---------------- converters ----------------
-    const int cw = (warp - 6) % NCW, grp = (warp - 6) / NCW;
-    const T* A = (const T*)p.A;
-    const int64_t rows = MN ? p.K : p.I, cols = MN ? p.I : p.K;
+    const int cw = (warp - 2 - EPI) % NCW, grp = (warp - 2 - EPI) / NCW;
     int stage = 0;
     uint32_t ph = 0;
     bool ok = true;
@@ -303,12 +365,15 @@ __global__ void __launch_bounds__(tcg_threads<NW>(), 1)
     // it is stored, so a whole tile of loads is in flight per warp
     Pair<T, VEC> v[NP];
     int it = i0, kt = 0, kt1 = 0;
+    const T* A = nullptr;       // of the product at hand
+    int64_t lda = 0, rows = 0, cols = 0;
+    int tile0 = 0;
     const T* src = nullptr;
     int nrow = 0, ncol = 0;     // valid rows of the warp, valid columns from the lane's on
     auto aim = [&]() {
-      const int64_t r0 = (MN ? kt * (int64_t)KT : it * (int64_t)kTileM) + cw * RW;
-      const int64_t c0 = (MN ? it * (int64_t)kTileM : kt * (int64_t)KT) + 2 * lane;
-      src = A + r0 * p.lda + c0;
+      const int64_t k0 = kt * (int64_t)KT, j0 = (it - tile0) * (int64_t)kTileM;
+      const int64_t r0 = (MN ? k0 : j0) + cw * RW, c0 = (MN ? j0 : k0) + 2 * lane;
+      src = A + r0 * lda + c0;
       nrow = (int)max((int64_t)0, min((int64_t)RW, rows - r0));
       ncol = (int)max((int64_t)0, min((int64_t)256, cols - c0));
     };
@@ -318,8 +383,16 @@ __global__ void __launch_bounds__(tcg_threads<NW>(), 1)
     };
     auto load = [&](int q, bool all) {
       const int rr = q / CB, c = (q % CB) * 64;
-      v[q].load(src + (int64_t)rr * p.lda + c, all || (rr < nrow && c < ncol),
+      v[q].load(src + (int64_t)rr * lda + c, all || (rr < nrow && c < ncol),
                 all || (rr < nrow && c + 1 < ncol));
+    };
+    auto enter = [&]() {
+      const TcgProb& b = p.prob[range(it, &kt, &kt1)];
+      A = (const T*)b.A;
+      lda = b.lda;
+      rows = MN ? b.K : b.I;
+      cols = MN ? b.I : b.K;
+      tile0 = b.tile0;
     };
     // on by n tiles of this CTA's range
     auto advance = [&](int n) {
@@ -327,13 +400,13 @@ __global__ void __launch_bounds__(tcg_threads<NW>(), 1)
       while (it < i1 && kt >= kt1) {
         n = kt - kt1;
         if (++it < i1) {
-          range(it, &kt, &kt1);
+          enter();
           kt += n;
         }
       }
     };
     if (it < i1) {
-      range(it, &kt, &kt1);
+      enter();
       advance(grp);
       stage = grp % S;
       ph = (uint32_t)(grp / S) & 1u;
@@ -362,7 +435,7 @@ __global__ void __launch_bounds__(tcg_threads<NW>(), 1)
           st_shared(o, v[q].word());
         } else {
           uint32_t w[3];
-          cut3(v[q].x, v[q].y, w);
+          cut3((float)v[q].x, (float)v[q].y, w);
 #pragma unroll
           for (int s = 0; s < 3; ++s) st_shared(o + s * kPiece, w[s]);
         }
@@ -394,27 +467,29 @@ __global__ void __launch_bounds__(tcg_threads<NW>(), 1)
       atomicOr(p.err, 64);
     }
   } else {
-    // ---------------- epilogue (warps 2..5) ----------------
+    // ---------------- epilogue ----------------
     const int q = warp & 3;
+    const int cn = p.Npad * 4 / EPI, cb = (warp - 2) / 4 * cn;   // this warp's columns (a multiple of 8)
     const uint32_t lane_off = (uint32_t)(32 * q) << 16;
     int buf = 0;
     uint32_t fph = 0;
     bool ok = true;
     for (int it = i0; it < i1 && ok; ++it) {
       int kt0, kt1;
-      range(it, &kt0, &kt1);
+      const TcgProb& b = p.prob[range(it, &kt0, &kt1)];
       float acc[NW];
 #pragma unroll
       for (int c = 0; c < NW; ++c) acc[c] = 0.f;
-      for (int g0 = kt0; g0 < kt1; g0 += p.group) {
+      const int drains = ((kt1 - kt0) * (KT / 16) + b.chain - 1) / b.chain;
+      for (int g = 0; g < drains; ++g) {
         ok = mbar_wait(smem_u32(&bar_full[buf]), fph, &abort_flag, p.wait_ns);
         ok = __all_sync(0xffffffffu, ok);
         if (!ok) break;
         fence_after();
-        const uint32_t d = tmem + lane_off + buf * NACC * p.Npad;
+        const uint32_t d = tmem + lane_off + buf * NACC * p.Npad + cb;
 #pragma unroll
         for (int cg = 0; cg < NW; cg += 8) {
-          if (cg >= p.Npad) continue;
+          if (cg >= cn) continue;
           uint32_t x[NACC][8];
 #pragma unroll
           for (int o = 0; o < NACC; ++o) tmem_ld8(d + o * p.Npad + cg, x[o]);
@@ -434,15 +509,20 @@ __global__ void __launch_bounds__(tcg_threads<NW>(), 1)
         if (buf == 0) fph ^= 1;
       }
       if (!ok) break;
-      const bool whole = kt0 == 0 && kt1 == p.nkt;
-      const int64_t row = (int64_t)it * kTileM + 32 * q + lane;
-      if (row < p.I) {
-        float* dst = whole ? p.C + row * p.Npad
+      const bool whole = kt0 == 0 && kt1 == b.nkt;
+      const int64_t row = (int64_t)(it - b.tile0) * kTileM + 32 * q + lane;
+      if (row < b.I && whole && b.trans) {
+        float* out = b.C + cb * b.ldc + row;
+#pragma unroll
+        for (int c = 0; c < NW; ++c)
+          if (c < cn) out[(int64_t)c * b.ldc] = acc[c];
+      } else if (row < b.I) {
+        float* dst = whole ? b.C + row * b.ldc
                            : p.part + ((int64_t)(2 * blockIdx.x + (it > i0)) * kTileM + 32 * q + lane) * p.Npad;
-        float4* out = reinterpret_cast<float4*>(dst);
+        float4* out = reinterpret_cast<float4*>(dst + cb);
 #pragma unroll
         for (int c = 0; c < NW / 4; ++c)
-          if (4 * c < p.Npad) out[c] = make_float4(acc[4 * c], acc[4 * c + 1], acc[4 * c + 2], acc[4 * c + 3]);
+          if (4 * c < cn) out[c] = make_float4(acc[4 * c], acc[4 * c + 1], acc[4 * c + 2], acc[4 * c + 3]);
       }
     }
     if (!ok) {
@@ -464,216 +544,284 @@ __global__ void __launch_bounds__(tcg_threads<NW>(), 1)
 // The B operands as the kernel's TMA reads them: [NS][Npad][Kpad] bfloat16,
 // zero beyond the operand.
 struct PrepJob {
-  const void* src;
+  TcCols c[2];
   uint16_t* dst;
-  int64_t ldb, K, Kpad, Jn, Npad;
-  int64_t start;   // first block
+  int64_t K, Kpad;
+  int nb, Npad, bf16, start;   // start: first block
 };
 struct PrepBatch {
-  int n, type;
-  PrepJob job[2];
+  int n;
+  PrepJob job[kTcgBatch];
 };
-constexpr int kPrepPairs = 4;   // pairs of a thread
+constexpr int kPrepRows = 8;   // rows of a thread
 
-__global__ void __launch_bounds__(256) tcg_prepare_kernel(const __grid_constant__ PrepBatch b) {
-  const PrepJob& j = b.job[b.n > 1 && (int64_t)blockIdx.x >= b.job[1].start ? 1 : 0];
-  const int64_t half = j.Kpad / 2, pairs = j.Npad * half;
-  const int64_t e0 = ((int64_t)blockIdx.x - j.start) * (256 * kPrepPairs) + threadIdx.x;
+__device__ __forceinline__ float prep_value(const TcCols& c, int64_t j, int64_t k) {
+  if (c.nkr == 0) return ((const float*)c.p)[j * c.sj + k * c.sk];
+  float v = 1.f;
+  uint32_t rem = (uint32_t)k;
 #pragma unroll
-  for (int u = 0; u < kPrepPairs; ++u) {
-    const int64_t e = e0 + u * 256;
-    if (e >= pairs) return;
-    const int64_t row = e / half, k = 2 * (e - row * half);
-    const bool a = row < j.Jn && k < j.K, c = row < j.Jn && k + 1 < j.K;
-    const int64_t at = row * j.ldb + k;
-    uint32_t* out = reinterpret_cast<uint32_t*>(j.dst) + e;
-    if (b.type == 2) {
-      const uint16_t* s = (const uint16_t*)j.src;
-      *out = (a ? (uint32_t)s[at] : 0u) | ((c ? (uint32_t)s[at + 1] : 0u) << 16);
+  for (int f = 3; f >= 0; --f) {
+    if (f >= c.nkr) continue;
+    const uint32_t q = rem / (uint32_t)c.krn[f];
+    v *= c.kr[f][(int64_t)(rem - q * (uint32_t)c.krn[f]) * c.ki[f] + j * c.kj[f]];
+    rem = q;
+  }
+  return v;
+}
+
+// Blocks of a job: 256 pairs of k by kPrepRows rows.
+__global__ void __launch_bounds__(256) tcg_prepare_kernel(const __grid_constant__ PrepBatch b) {
+  int at = 0;
+  while (at + 1 < b.n && (int)blockIdx.x >= b.job[at + 1].start) ++at;
+  const PrepJob& j = b.job[at];
+  const int half = (int)(j.Kpad / 2), kblocks = (half + 255) / 256;
+  const int blk = (int)blockIdx.x - j.start;
+  const int kp = blk % kblocks * 256 + (int)threadIdx.x, row0 = blk / kblocks * kPrepRows;
+  if (kp >= half) return;
+  const int64_t k = 2 * (int64_t)kp, pairs = (int64_t)j.Npad * half;
+#pragma unroll
+  for (int u = 0; u < kPrepRows; ++u) {
+    int row = row0 + u;
+    uint32_t* out = reinterpret_cast<uint32_t*>(j.dst) + (int64_t)row * half + kp;
+    const bool second = row >= j.c[0].n && j.nb > 1;
+    const TcCols& c = j.c[second ? 1 : 0];
+    if (second) row -= j.c[0].n;
+    const bool in = row < c.n && k < j.K, in1 = in && k + 1 < j.K;
+    if (j.bf16) {
+      const uint16_t* s = (const uint16_t*)c.p + row * c.sj + k * c.sk;
+      *out = (in ? (uint32_t)s[0] : 0u) | ((in1 ? (uint32_t)s[c.sk] : 0u) << 16);
     } else {
-      const float* s = (const float*)j.src;
       uint32_t w[3];
-      cut3(a ? s[at] : 0.f, c ? s[at + 1] : 0.f, w);
+      cut3(in ? prep_value(c, row, k) : 0.f, in1 ? prep_value(c, row, k + 1) : 0.f, w);
 #pragma unroll
       for (int q = 0; q < 3; ++q) out[q * pairs] = w[q];
     }
   }
 }
 
-// Sums the pieces of the row tiles that more than one CTA worked on.
-__global__ void __launch_bounds__(256) tcg_pieces_kernel(const float* part, int64_t I, int nI,
-                                                         int nkt, int G, int Npad, float* C) {
-  const int it = blockIdx.x;
-  const int64_t total = (int64_t)nI * nkt;
-  auto owner = [&](int64_t u) { return (int)(((u + 1) * G - 1) / total); };
-  const int c0 = owner((int64_t)it * nkt), c1 = owner((int64_t)(it + 1) * nkt - 1);
-  if (c0 == c1) return;
-  const int64_t rows = min((int64_t)kTileM, I - (int64_t)it * kTileM);
-  const int n4 = (int)(rows * Npad / 4);
-  const int64_t tile4 = (int64_t)kTileM * Npad / 4;
+// Sums the pieces of the row tiles that more than one CTA worked on: block c
+// takes the tile in which CTA c's range begins, if it is the first to begin
+// inside it.
+__global__ void __launch_bounds__(256) tcg_pieces_kernel(const __grid_constant__ TcgParams p, int G) {
+  const int c = blockIdx.x + 1;
+  const int64_t u = p.units * c / G, before = p.units * (c - 1) / G;
+  const int it = tcg_tile(p, u), q = tcg_prob(p, it);
+  const TcgProb& b = p.prob[q];
+  const int64_t first = tcg_unit(p, q, it);
+  if (u == first || before > first) return;
+  const int c0 = c - 1, c1 = (int)(((first + b.nkt) * G - 1) / p.units);
+  const int64_t r0 = (int64_t)(it - b.tile0) * kTileM;
+  const int rows = (int)min((int64_t)kTileM, b.I - r0);
+  const int64_t tile = (int64_t)kTileM * p.Npad;
   // only the first CTA's range can begin in an earlier tile
-  const float4* p4 = reinterpret_cast<const float4*>(part);
-  const float4* f4 = p4 + (int64_t)(2 * c0 + ((int)(total * c0 / G / nkt) < it)) * tile4;
-  float4* o4 = reinterpret_cast<float4*>(C) + (int64_t)it * tile4;
-  for (int e = blockIdx.y * 256 + threadIdx.x; e < n4; e += gridDim.y * 256) {
-    float4 a = f4[e];
+  const float* p0 = p.part + (2 * c0 + (before < first)) * tile;
+  const int per = p.Npad / 4;
+  for (int e = blockIdx.y * 256 + threadIdx.x; e < rows * per; e += gridDim.y * 256) {
+    // transposed results: consecutive threads take consecutive rows
+    const int r = b.trans ? e % rows : e / per, c4 = b.trans ? e / rows : e % per;
+    const int64_t at = (int64_t)r * p.Npad + 4 * c4;
+    float4 a = *reinterpret_cast<const float4*>(p0 + at);
 #pragma unroll 4
-    for (int c = c0 + 1; c <= c1; ++c) {
-      const float4 v = p4[(int64_t)(2 * c) * tile4 + e];
+    for (int d = c; d <= c1; ++d) {
+      const float4 v = *reinterpret_cast<const float4*>(p.part + (int64_t)(2 * d) * tile + at);
       a.x += v.x;
       a.y += v.y;
       a.z += v.z;
       a.w += v.w;
     }
-    o4[e] = a;
+    if (b.trans) {
+      float* o = b.C + (int64_t)4 * c4 * b.ldc + r0 + r;
+      o[0] = a.x;
+      o[b.ldc] = a.y;
+      o[2 * b.ldc] = a.z;
+      o[3 * b.ldc] = a.w;
+    } else {
+      *reinterpret_cast<float4*>(b.C + (r0 + r) * b.ldc + 4 * c4) = a;
+    }
   }
 }
 
-struct TcgGeometry {
-  int NS, KT, Npad, nI, nkt, stages, grid;
-  int64_t Kpad, b_bytes, p_bytes;
-  size_t smem;
-};
+static int tcg_pieces_of(const TcGemm& g) { return g.type == 2 ? 1 : 3; }
+static int tcg_kt(const TcGemm& g) { return g.type == 2 ? 128 : 64; }
+static int tcg_npad(const TcGemm& g) { return (int)round_up(g.Jn, 16); }
 
-static TcgGeometry tcg_geometry(const TcGemm& g, int sms) {
-  TcgGeometry o;
-  o.NS = g.type == 2 ? 1 : 3;
-  o.KT = g.type == 2 ? 128 : 64;
-  o.Npad = (int)round_up(g.Jn, 16);
-  o.nI = (int)ceil_div(g.I, (int64_t)kTileM);
-  o.nkt = (int)ceil_div(g.K, (int64_t)o.KT);
-  o.Kpad = (int64_t)o.nkt * o.KT;
-  const int64_t stage = (int64_t)o.NS * (128 * o.KT * 2 + (int64_t)o.Npad * o.KT * 2);
-  o.stages = (int)std::min<int64_t>(kTcgMaxStages, (kSmemBudget - 1024) / stage);
-  o.smem = (size_t)(1024 + o.stages * stage);
-  // at least two tiles per CTA: a shorter range is mostly fill and drain
-  o.grid = (int)std::max<int64_t>(1, std::min<int64_t>((int64_t)o.nI * o.nkt / 2, sms));
-  o.b_bytes = round_up((int64_t)o.NS * o.Npad * o.Kpad * 2, 256);
-  o.p_bytes = (int64_t)2 * sms * kTileM * o.Npad * 4;   // (as for a full grid: grows with the shape only)
-  return o;
-}
-
-template <typename T, bool MN, bool VEC, int NW>
-static ttnn_status tcg_launch(const TcgGeometry& o, const CUtensorMap& mB, const TcgParams& p,
-                              cudaStream_t st) {
-  constexpr int slot = 4 + (NW > 64 ? 8 : 0) + (sizeof(T) == 4 ? 4 : 0) + (MN ? 2 : 0) + (VEC ? 1 : 0);
-  TTNN_TRY(smem_limit_once((const void*)tcg_kernel<T, MN, VEC, NW>, slot));
-  tcg_kernel<T, MN, VEC, NW><<<o.grid, tcg_threads<NW>(), o.smem, st>>>(mB, p);
+template <typename T, bool MN, bool VEC, int EPI>
+static ttnn_status tcg_launch(const TcgParams& p, int grid, size_t smem, cudaStream_t st) {
+  constexpr int kind = sizeof(T) == 2 ? 0 : sizeof(T) == 4 ? 1 : 2;
+  constexpr int slot = 8 + kind * 8 + (EPI > 4 ? 4 : 0) + (MN ? 2 : 0) + (VEC ? 1 : 0);
+  TTNN_TRY(smem_limit_once((const void*)tcg_kernel<T, MN, VEC, EPI>, slot));
+  tcg_kernel<T, MN, VEC, EPI><<<grid, tcg_threads<EPI>(), smem, st>>>(p);
   return check_launch("tcg_kernel");
 }
 
-template <typename T, bool VEC, int NW>
-static ttnn_status tcg_major(bool mn, const TcgGeometry& o, const CUtensorMap& mB,
-                             const TcgParams& p, cudaStream_t st) {
-  return mn ? tcg_launch<T, true, VEC, NW>(o, mB, p, st) : tcg_launch<T, false, VEC, NW>(o, mB, p, st);
+template <typename T, bool VEC, int EPI>
+static ttnn_status tcg_major(bool mn, const TcgParams& p, int grid, size_t smem, cudaStream_t st) {
+  return mn ? tcg_launch<T, true, VEC, EPI>(p, grid, smem, st)
+            : tcg_launch<T, false, VEC, EPI>(p, grid, smem, st);
+}
+
+template <typename T>
+static ttnn_status tcg_form(bool vec, bool mn, const TcgParams& p, int grid, size_t smem,
+                            cudaStream_t st) {
+  if (p.Npad > 64 || sizeof(T) == 2)   // (bfloat16 converters need the fewest registers)
+    return vec ? tcg_major<T, true, 8>(mn, p, grid, smem, st) : tcg_major<T, false, 8>(mn, p, grid, smem, st);
+  return vec ? tcg_major<T, true, 4>(mn, p, grid, smem, st) : tcg_major<T, false, 4>(mn, p, grid, smem, st);
+}
+
+// Pairs in one load need even extents and strides and an aligned base.
+static bool tcg_vec(const TcGemm& g) {
+  const int pair = g.type == 2 ? 4 : g.type == 1 ? 8 : 16;
+  return (g.mn ? g.I : g.K) % 2 == 0 && g.lda % 2 == 0 && (uintptr_t)g.A % pair == 0;
+}
+
+// One launch: up to kTcgBatch products of one type, majorness, width and vec.
+static ttnn_status tcg_batch(const TcGemm* const* g, int n, void* pieces, int sms, int* err,
+                             uint64_t wait_ns, cudaStream_t st) {
+  TcgParams p;
+  const TcGemm& f = *g[0];
+  const int NS = tcg_pieces_of(f), KT = tcg_kt(f);
+  p.n = n;
+  p.Npad = tcg_npad(f);
+  p.tiles = 0;
+  p.units = 0;
+  for (int k = 0; k < n; ++k) {
+    TcgProb& q = p.prob[k];
+    const int64_t nI = ceil_div(g[k]->I, (int64_t)kTileM);
+    q.nkt = (int)ceil_div(g[k]->K, (int64_t)KT);
+    TTNN_TRY(encode_map(&q.mapB, g[k]->prep, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2, (int64_t)q.nkt * KT,
+                        (int64_t)NS * p.Npad, 64u, (uint32_t)p.Npad, CU_TENSOR_MAP_SWIZZLE_128B));
+    q.A = g[k]->A;
+    q.lda = g[k]->lda;
+    q.I = g[k]->I;
+    q.K = g[k]->K;
+    q.C = (float*)g[k]->C;
+    q.ldc = g[k]->ldc;
+    q.trans = g[k]->trans;
+    q.unit0 = p.units;
+    q.tile0 = p.tiles;
+    // Chain of leading products per drain: 8 MMAs (128 k).  Long binary32
+    // reductions take 16: their sums err less than the SIMT GEMM's by more
+    // than the longer chain adds (64^4 x 8 slab: 4.2e-7 against 9.8e-7; short
+    // ones would lose that margin), and the drains cost 10 % of the time.
+    q.chain = g[k]->chain ? g[k]->chain : f.type != 2 && g[k]->K >= 2048 ? 16 : 8;
+    p.tiles += (int)nI;
+    p.units += nI * q.nkt;
+  }
+  const int64_t stage = (int64_t)NS * (128 * KT * 2 + (int64_t)p.Npad * KT * 2);
+  p.stages = (int)std::min<int64_t>(kTcgMaxStages, (kSmemBudget - 1024) / stage);
+  p.part = (float*)pieces;
+  p.err = err;
+  p.wait_ns = wait_ns;
+  const size_t smem = (size_t)(1024 + p.stages * stage);
+  // at least two units per CTA: a shorter range is mostly fill and drain
+  const int grid = (int)std::max<int64_t>(1, std::min<int64_t>(p.units / 2, sms));
+  const bool vec = tcg_vec(f), mn = f.mn != 0;
+  if (f.type == 2) TTNN_TRY(tcg_form<uint16_t>(vec, mn, p, grid, smem, st));
+  else if (f.type == 1) TTNN_TRY(tcg_form<float>(vec, mn, p, grid, smem, st));
+  else TTNN_TRY(tcg_form<double>(vec, mn, p, grid, smem, st));
+  if (grid == 1) return TTNN_OK;
+  tcg_pieces_kernel<<<dim3((unsigned)(grid - 1), 4), 256, 0, st>>>(p, grid);
+  return check_launch("tcg_pieces_kernel");
 }
 
 }  // namespace tc
 
+int tcg_sms() { return tc::sm_count(); }
+uint64_t tcg_wait_ns() { return tc::kTimeoutNs; }
+
 bool tcg_supported(const TcGemm& g) {
   if (g.type == 0) return zgemm_supported(g);
   const int64_t lim = int64_t(1) << 31;
-  if ((g.type != 1 && g.type != 2) || g.I < 1 || g.Jn < 1 || g.K < 1) return false;
-  if (g.Jn > tc::kTcgMaxN || g.ldc != round_up(g.Jn, 16)) return false;
-  // 32-bit tile counts and TMA coordinates
+  if (g.type < 1 || g.type > 3 || g.I < 1 || g.Jn < 1 || g.K < 1) return false;
+  if (g.Jn > tc::kTcgMaxN) return false;
+  // float4 rows of C
+  if (!g.trans && (g.ldc < round_up(g.Jn, 16) || g.ldc % 4)) return false;
+  // 32-bit tile counts (of kTcgBatch products) and TMA coordinates
   return g.I < lim - 256 && g.K < lim - 256;
 }
 
 int64_t tcg_prep_bytes(const TcGemm& g) {
-  return g.type == 0 ? zgemm_prep_bytes(g) : tc::tcg_geometry(g, 1).b_bytes;
+  if (g.type == 0) return zgemm_prep_bytes(g);
+  return round_up((int64_t)tc::tcg_pieces_of(g) * tc::tcg_npad(g) * round_up(g.K, (int64_t)tc::tcg_kt(g)) * 2, 256);
+}
+
+int64_t tcg_piece_bytes(const TcGemm& g, int sms) {
+  return g.type == 0 ? zgemm_piece_bytes(g, sms) : (int64_t)2 * sms * tc::kTileM * tc::tcg_npad(g) * 4;
 }
 
 ttnn_status tcg_prepare(const TcGemm* g, int n, void* const* dst, cudaStream_t st) {
   using namespace tc;
   if (g[0].type == 0) return zgemm_prepare(g, n, dst, st);
-  PrepBatch pb;
-  pb.n = n;
-  pb.type = g[0].type;
-  int64_t blocks = 0;
-  for (int k = 0; k < n; ++k) {
-    const TcgGeometry o = tcg_geometry(g[k], 1);
-    PrepJob& j = pb.job[k];
-    j.src = g[k].B;
-    j.dst = (uint16_t*)dst[k];
-    j.ldb = g[k].ldb;
-    j.K = g[k].K;
-    j.Kpad = o.Kpad;
-    j.Jn = g[k].Jn;
-    j.Npad = o.Npad;
-    j.start = blocks;
-    blocks += ceil_div(j.Npad * j.Kpad / 2, (int64_t)256 * kPrepPairs);
+  for (int k0 = 0; k0 < n; k0 += kTcgBatch) {
+    PrepBatch pb;
+    pb.n = std::min(n - k0, kTcgBatch);
+    int64_t blocks = 0;
+    for (int k = 0; k < pb.n; ++k) {
+      const TcGemm& m = g[k0 + k];
+      PrepJob& j = pb.job[k];
+      j.c[0] = m.b[0];
+      j.c[1] = m.b[1];
+      j.nb = m.nb;
+      j.dst = (uint16_t*)dst[k0 + k];
+      j.K = m.K;
+      j.Kpad = round_up(m.K, (int64_t)tcg_kt(m));
+      j.Npad = tcg_npad(m);
+      j.bf16 = m.type == 2;
+      j.start = (int)blocks;
+      blocks += ceil_div(j.Kpad / 2, (int64_t)256) * (j.Npad / kPrepRows);
+      if (blocks >= (int64_t(1) << 31)) {
+        set_error("tensor-core GEMM: operand too large");
+        return TTNN_EUNSUPPORTED;
+      }
+    }
+    tcg_prepare_kernel<<<(unsigned)blocks, 256, 0, st>>>(pb);
+    TTNN_TRY(check_launch("tcg_prepare_kernel"));
   }
-  if (blocks >= (int64_t(1) << 31)) {
-    set_error("tensor-core GEMM: operand too large");
-    return TTNN_EUNSUPPORTED;
-  }
-  tcg_prepare_kernel<<<(unsigned)blocks, 256, 0, st>>>(pb);
-  return check_launch("tcg_prepare_kernel");
+  return TTNN_OK;
 }
 
-static ttnn_status launch_tcg_one(const TcGemm& g, const void* prep, void* pieces, int sms, int* err,
-                                  uint64_t wait_ns, cudaStream_t st) {
-  using namespace tc;
-  const TcgGeometry o = tcg_geometry(g, sms);
-  CUtensorMap mB;
-  TTNN_TRY(encode_map(&mB, prep, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2, o.Kpad, (int64_t)o.NS * o.Npad,
-                      64u, (uint32_t)o.Npad, CU_TENSOR_MAP_SWIZZLE_128B));
-  TcgParams p;
-  p.A = g.A;
-  p.lda = g.lda;
-  p.I = g.I;
-  p.K = g.K;
-  p.nI = o.nI;
-  p.nkt = o.nkt;
-  p.Npad = o.Npad;
-  p.stages = o.stages;
-  // Chain of leading products per drain: 128 k (8 MMAs).  Long binary32
-  // reductions take 256: their sums err less than the SIMT GEMM's by more
-  // than the longer chain adds (64^4 x 8 slab: 4.2e-7 against 9.8e-7; short
-  // ones would lose that margin), and the drains cost 10 % of the time.
-  p.group = g.type == 2 ? 1 : g.K >= 2048 ? 4 : 2;
-  p.C = (float*)g.C;
-  p.part = (float*)pieces;
-  p.err = err;
-  p.wait_ns = wait_ns;
-  const int64_t inner = g.mn ? g.I : g.K;
-  const int pair = g.type == 2 ? 4 : 8;
-  const bool vec = inner % 2 == 0 && g.lda % 2 == 0 && (uintptr_t)g.A % pair == 0;
-  const bool mn = g.mn != 0, wide = o.Npad > 64;
-  if (g.type == 2 && vec)
-    TTNN_TRY(wide ? tcg_major<uint16_t, true, kTcgMaxN>(mn, o, mB, p, st)
-                  : tcg_major<uint16_t, true, 64>(mn, o, mB, p, st));
-  else if (g.type == 2)
-    TTNN_TRY(wide ? tcg_major<uint16_t, false, kTcgMaxN>(mn, o, mB, p, st)
-                  : tcg_major<uint16_t, false, 64>(mn, o, mB, p, st));
-  else if (vec)
-    TTNN_TRY(wide ? tcg_major<float, true, kTcgMaxN>(mn, o, mB, p, st)
-                  : tcg_major<float, true, 64>(mn, o, mB, p, st));
-  else
-    TTNN_TRY(wide ? tcg_major<float, false, kTcgMaxN>(mn, o, mB, p, st)
-                  : tcg_major<float, false, 64>(mn, o, mB, p, st));
-  if (o.grid == 1) return TTNN_OK;
-  const int per = (int)std::max<int64_t>(1, std::min<int64_t>(8, 608 / std::max(1, o.nI)));
-  tcg_pieces_kernel<<<dim3((unsigned)o.nI, (unsigned)per), 256, 0, st>>>(
-      (const float*)pieces, g.I, o.nI, o.nkt, o.grid, o.Npad, (float*)g.C);
-  return check_launch("tcg_pieces_kernel");
+ttnn_status tcg_run(const TcGemm* g, int n, void* pieces, int sms, int* err, uint64_t wait_ns,
+                    cudaStream_t st) {
+  auto alike = [](const TcGemm& a, const TcGemm& b) {
+    return a.type == b.type && a.mn == b.mn && tc::tcg_npad(a) == tc::tcg_npad(b) &&
+           tc::tcg_vec(a) == tc::tcg_vec(b);
+  };
+  std::vector<char> done(n, 0);
+  for (int k = 0; k < n; ++k) {
+    if (done[k]) continue;
+    if (g[k].type == 0) {
+      TTNN_TRY(launch_zgemm(g[k], g[k].prep, pieces, sms, err, wait_ns, st));
+      continue;
+    }
+    const TcGemm* batch[kTcgBatch];
+    int m = 0;
+    int64_t tiles = 0;
+    for (int l = k; l < n && m < kTcgBatch; ++l) {
+      const int64_t t = ceil_div(g[l].I, (int64_t)tc::kTileM);
+      if (done[l] || !alike(g[k], g[l]) || (m > 0 && tiles + t >= (int64_t(1) << 30))) continue;
+      batch[m++] = &g[l];
+      tiles += t;
+      done[l] = 1;
+    }
+    TTNN_TRY(tc::tcg_batch(batch, m, pieces, sms, err, wait_ns, st));
+  }
+  return TTNN_OK;
 }
 
 ttnn_status launch_tcg(const TcGemm* g, int n, int sms, int* err, uint64_t wait_ns, void* ws,
                        int64_t ws_bytes, cudaStream_t st, bool dry, int64_t* need) {
   int64_t b_bytes = 0, p_bytes = 0;
-  void* dst[2] = {nullptr, nullptr};
-  TcGemm todo[2];
-  int nt = 0;
+  std::vector<TcGemm> all(g, g + n), todo;
+  std::vector<void*> dst;
   char* w = (char*)ws + (256 - ((uintptr_t)ws & 255)) % 256;
-  for (int k = 0; k < n; ++k) {
-    // the products run in order and share the room of their pieces
-    p_bytes = std::max(p_bytes, g[k].type == 0 ? zgemm_piece_bytes(g[k], sms)
-                                               : tc::tcg_geometry(g[k], sms).p_bytes);
-    if (g[k].prep) continue;
-    todo[nt] = g[k];
-    dst[nt++] = w + b_bytes;
-    b_bytes += tcg_prep_bytes(g[k]);
+  for (TcGemm& m : all) {
+    // the launches run in order and share the room of their pieces
+    p_bytes = std::max(p_bytes, tcg_piece_bytes(m, sms));
+    if (m.prep) continue;
+    todo.push_back(m);
+    dst.push_back(w + b_bytes);
+    m.prep = w + b_bytes;
+    b_bytes += tcg_prep_bytes(m);
   }
   if (dry) {
     *need = b_bytes + p_bytes + 256;
@@ -683,14 +831,8 @@ ttnn_status launch_tcg(const TcGemm* g, int n, int sms, int* err, uint64_t wait_
     set_error("tensor-core GEMM: workspace too small");
     return TTNN_ENOMEM;
   }
-  if (nt > 0) TTNN_TRY(tcg_prepare(todo, nt, dst, st));
-  nt = 0;
-  for (int k = 0; k < n; ++k) {
-    const void* prep = g[k].prep ? g[k].prep : dst[nt++];
-    TTNN_TRY(g[k].type == 0 ? launch_zgemm(g[k], prep, w + b_bytes, sms, err, wait_ns, st)
-                            : launch_tcg_one(g[k], prep, w + b_bytes, sms, err, wait_ns, st));
-  }
-  return TTNN_OK;
+  if (!todo.empty()) TTNN_TRY(tcg_prepare(todo.data(), (int)todo.size(), dst.data(), st));
+  return tcg_run(all.data(), n, w + b_bytes, sms, err, wait_ns, st);
 }
 
 }  // namespace ttnn

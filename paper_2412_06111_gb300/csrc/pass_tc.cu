@@ -499,10 +499,10 @@ struct Geometry {
 
 ttnn_status smem_limit_once(const void* func, int slot, int bytes) {
   static std::mutex mu;
-  static bool done[32][64] = {};
+  static bool done[40][64] = {};
   int dev = 0;
   TTNN_TRY_CUDA(cudaGetDevice(&dev));
-  if (slot < 0 || slot >= 32 || dev < 0 || dev >= 64) {
+  if (slot < 0 || slot >= 40 || dev < 0 || dev >= 64) {
     set_error("internal: shared-memory limit slot");
     return TTNN_EUNSUPPORTED;
   }

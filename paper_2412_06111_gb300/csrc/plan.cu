@@ -391,9 +391,9 @@ struct Ax {
   int64_t bc = 0;
 };
 struct View {
-  char* ptr;
+  char* ptr = nullptr;
   std::vector<Ax> ax;
-  int64_t ld;      // stride of the next-to-last axis
+  int64_t ld = 0;  // stride of the next-to-last axis
   // scales not yet applied: the view's values times prod_k sc_k[index on the
   // axis (kind, id)].  They are rows of the DRM factors of box-fixed modes
   // (X_mu[c, :] on the column axis, Y_mu[c, :] on a sketch axis), commute
@@ -442,6 +442,9 @@ struct Ctx {
   int64_t d2y_ld = 0;
   const char* xo = nullptr;
   int64_t nRo = 0;
+  // room for the pieces of the program's tensor-core GEMMs, and its size
+  char* tc_pieces = nullptr;
+  int64_t tc_piece_bytes = 0;
 };
 
 static int find_ax(const View& v, int kind, int id) {
@@ -582,6 +585,27 @@ static ttnn_status contract_view(Ctx& C, const View& in, int k, const void* W, i
   C.prog->add(op, in.ptr, W);
   *out = o;
   return TTNN_OK;
+}
+
+// Records the tensor-core GEMM g; its result goes to C.ws with rows of *ld
+// (g.trans: of *ld = I) elements, at *out.
+static void tc_gemm(Ctx& C, TcGemm g, std::initializer_list<const void*> in, char** out, int64_t* ld) {
+  const int64_t npad = round_up(g.Jn, (int64_t)16);
+  *ld = g.ldc = g.trans ? g.I : npad;
+  *out = C.ws.alloc(g.I * npad * 4);
+  g.C = *out;
+  TcOp op;
+  if (!g.chain) g.chain = 2;   // walks chain several products: the shortest chains
+  op.prep = C.ws.alloc(tcg_prep_bytes(g));
+  const int64_t pieces = tcg_piece_bytes(g, tcg_sms());
+  if (pieces > C.tc_piece_bytes) {
+    C.tc_pieces = C.ws.alloc(pieces);
+    C.tc_piece_bytes = pieces;
+  }
+  op.pieces = C.tc_pieces;
+  op.err = C.P.err_dev;
+  op.g = g;
+  C.prog->add(op, in);
 }
 
 static const char* facX(Ctx& C, int mode) { return C.facw + (C.P.x_off[mode] + C.box.off[mode] * C.P.rmax) * C.eb; }
@@ -1160,6 +1184,22 @@ constexpr int64_t kTcgMinEntries = int64_t(1) << 21;
 // The same for binary64 (64 entries: 58 against 56 us per update, 1296: 61
 // against 92, 24^4: 83 against 124, 20^6: 1003 against 6036).
 constexpr int64_t kZgemmMinEntries = 1024;
+// Smallest first-level product (entries, D1's padding columns counted) whose
+// Khatri-Rao prefix takes the tensor-core GEMM instead of the split-K form
+// (whole updates, bfloat16, r = 20: 64^5 541 us against 554, 96x96x64x16x32
+// 342 against 375, 56^5 387 against 388, 40^5 181 against 170), and instead of
+// contractions mode by mode where s > 32 keeps the split-K form out (64^5,
+// r = 32: 681 against 942; 40^5, r = 24: 190 against 246; 32^5 binary32,
+// r = 32: 213 against 218; 24^3 x 48^2, 0.8 M entries: 158 against 155) or a
+// reduction below 1024 stays whole in few blocks (64^4 x 8, binary32: 387
+// against 456).
+constexpr int64_t kTcPrefixEntries = int64_t(1) << 24;
+constexpr int64_t kTcWideEntries = int64_t(1) << 20;
+// Smallest input core (entries times columns) of a TTN-format update that is
+// contracted on the tensor cores (whole updates of 64^4, r + s = 75: rank 128
+// 251 us against 344, 96 219 against 243, 80 210 against 212, 64 204 against
+// 189; r + s = 25: 128 193 against 199, 104 192 against 167).
+constexpr int64_t kTcCoreWork = int64_t(3) << 24;
 
 // The products of an nL x nR box as tensor-core GEMMs (operand pointers left
 // empty); false where they are not taken.
@@ -1172,14 +1212,14 @@ static bool tcg_products(const ttnn_plan_s& P, int64_t nL, int64_t nR, TcGemm* t
     t = TcGemm();
     t.I = nL; t.Jn = P.wR; t.K = nR;
     t.lda = nR; t.mn = 0; t.type = P.pass_store;
-    t.ldb = nR; t.ldc = P.wRpad;
+    t.b[0].sj = nR; t.b[0].sk = 1; t.b[0].n = P.wR; t.ldc = P.wRpad;
   }
   if (P.wL > 0) {   // D2 = M^T B_L^T
     TcGemm& t = tg[(*n)++];
     t = TcGemm();
     t.I = nR; t.Jn = P.wL; t.K = nL;
     t.lda = nR; t.mn = 1; t.type = P.pass_store;
-    t.ldb = nL; t.ldc = P.wLpad;
+    t.b[0].sj = nL; t.b[0].sk = 1; t.b[0].n = P.wL; t.ldc = P.wLpad;
   }
   for (int k = 0; k < *n; ++k)
     if (!tcg_supported(tg[k])) return false;
@@ -1215,7 +1255,7 @@ ttnn_status tcg_plan_prepare(ttnn_plan_s& P, cudaStream_t st) {
   void* dst[2];
   char* at = (char*)P.prep_block;
   for (int k = 0; k < n; ++k) {
-    tg[k].B = tg[k].mn ? P.sideL : P.sideR;
+    tg[k].b[0].p = tg[k].mn ? P.sideL : P.sideR;
     dst[k] = at;
     P.prep[tg[k].mn] = at;
     at += tcg_prep_bytes(tg[k]);
@@ -1234,14 +1274,18 @@ ttnn_status dense_update_need(ttnn_plan_s& P, const Box& box, int64_t* need) {
   key.push_back(box.full ? 1 : 0);
   key.push_back(P.ws_limit);
   auto it = P.ws_need_cache.find(key);
-  if (it != P.ws_need_cache.end()) {
-    *need = it->second;
-    return TTNN_OK;
+  if (it == P.ws_need_cache.end()) {
+    int64_t n = 0;
+    P.roomy = true;
+    TTNN_TRY(run_dense_update(P, nullptr, nullptr, box, nullptr, 1.0, nullptr, true, &n));
+    if (n > P.ws_limit) {
+      P.roomy = false;
+      TTNN_TRY(run_dense_update(P, nullptr, nullptr, box, nullptr, 1.0, nullptr, true, &n));
+    }
+    it = P.ws_need_cache.emplace(key, std::make_pair(n, P.roomy)).first;
   }
-  int64_t n = 0;
-  TTNN_TRY(run_dense_update(P, nullptr, nullptr, box, nullptr, 1.0, nullptr, true, &n));
-  P.ws_need_cache[key] = n;
-  *need = n;
+  *need = it->second.first;
+  P.roomy = it->second.second;
   return TTNN_OK;
 }
 
@@ -1407,19 +1451,16 @@ ttnn_status run_dense_update(ttnn_plan_s& P, void* acc, const void* data, const 
   // the tensor-core GEMM, for boxes the passes above do not take
   TcGemm tg[2];
   int ntg = 0;
-  bool tcg = !r1 && tcg_products(P, nL, nR, tg, &ntg);
+  bool tcg = !r1 && !use_tc && P.roomy && tcg_products(P, nL, nR, tg, &ntg);
   int64_t tcg_need = 0;
   if (tcg) {
     for (int k = 0; k < ntg; ++k) {
       tg[k].A = data;
-      tg[k].B = tg[k].mn ? sL : sR;
+      tg[k].b[0].p = tg[k].mn ? sL : sR;
       tg[k].C = tg[k].mn ? D2 : D1;
       if (box.full && P.prep[tg[k].mn]) tg[k].prep = P.prep[tg[k].mn];
     }
-  }
-  if (tcg) {
     TTNN_TRY(launch_tcg(tg, ntg, tc::sm_count(), nullptr, 0, nullptr, 0, st, true, &tcg_need));
-    tcg = !use_tc && round_up(ws.top, 256) + tcg_need <= P.ws_limit;
   }
   if (r1) {
     const int64_t mark = ws.top;
@@ -1562,13 +1603,56 @@ ttnn_status run_dense_update(ttnn_plan_s& P, void* acc, const void* data, const 
   const TNode* krL = nullptr;
   if (P.variant == TTNN_VARIANT_TTNN && r1 == 0 && !P.walk_f64 && P.Lch.size() == 1) {
     const TNode& Lc = P.nodes[P.Lch[0]];
-    if (Lc.sketched() && !Lc.leaf && Lc.user != P.ychild && Lc.r <= P.rXL && Lc.s <= 32) {
+    if (Lc.sketched() && !Lc.leaf && Lc.user != P.ychild && Lc.r <= P.rXL) {
       const TNode& c1 = P.nodes[Lc.ch.front()];
       int64_t n1 = 1;
       for (int m = c1.lo; m < c1.hi; ++m) n1 *= box.ext[m];
       if (!c1.identity && c1.s == Lc.s && c1.lo == P.Llo && c1.hi - c1.lo <= 4 && n1 >= 512 &&
           n1 < (int64_t(1) << 31))
         krL = &Lc;
+    }
+  }
+  // With enough work that reduction runs on the tensor cores, once for both
+  // column groups: D1's columns (those of its padding too) of the remaining
+  // modes are the rows of a product with the Khatri-Rao block of c1, stored
+  // sketch axis first as the walk reads it.  Otherwise the split-K form takes
+  // it, which holds 32 columns: beyond them the modes go one by one.
+  View krG, krH;
+  if (krL) {
+    const TNode& c1 = P.nodes[krL->ch.front()];
+    TcGemm g;
+    g.K = 1;
+    for (int m = c1.lo; m < c1.hi; ++m) g.K *= box.ext[m];
+    g.I = nL / g.K * P.wRpad;
+    g.lda = g.I;
+    g.mn = 1;
+    g.A = D1;
+    g.Jn = c1.s;
+    g.trans = 1;
+    TcCols& y = g.b[0];
+    y.n = c1.s;
+    for (int m = c1.lo; m < c1.hi; ++m, ++y.nkr) {
+      y.kr[y.nkr] = (const float*)facY(C, m);
+      y.krn[y.nkr] = (int32_t)box.ext[m];
+      y.ki[y.nkr] = P.smax;
+      y.kj[y.nkr] = 1;
+    }
+    const bool split = krL->s <= 32 && g.K >= 1024;   // the split-K form would fill the chip
+    if (P.roomy && g.K * g.I >= (split ? kTcPrefixEntries : kTcWideEntries) && tcg_supported(g)) {
+      char* out;
+      int64_t ld;
+      tc_gemm(C, g, {D1}, &out, &ld);
+      krG.ptr = out;
+      krG.ld = P.wRpad;
+      krG.ax = {Ax{AX_SK, c1.user, c1.s, 0}};
+      for (const Ax& a : mode_axes(c1.hi, P.Lhi)) krG.ax.push_back(a);
+      krH = krG;
+      krG.ax.push_back(Ax{AX_J, -1, krL->r, 0});
+      krH.ptr += P.rXL * eb;
+      krH.ax[0].id = krL->user;
+      krH.ax.push_back(Ax{AX_SK, P.ychild, P.wYR, 0});
+    } else if (krL->s > 32) {
+      krL = nullptr;
     }
   }
   // L side (both variants): G over L modes from D1's X part
@@ -1578,8 +1662,9 @@ ttnn_status run_dense_update(ttnn_plan_s& P, void* acc, const void* data, const 
     if (r1 == 1) GL = bview(P.Llo, P.Lhi, Ax{AX_J, -1, 1, 0}, P.rXL, bw);
     if (krL) {
       const TNode& c1 = P.nodes[krL->ch.front()];
-      View pre;
-      TTNN_TRY(kr_prefix(C, truncate_j(GL, krL->r), c1.user, c1.lo, c1.hi, c1.s, &pre));
+      View pre = krG;
+      if (!krG.ptr)
+        TTNN_TRY(kr_prefix(C, truncate_j(GL, krL->r), c1.user, c1.lo, c1.hi, c1.s, &pre));
       TTNN_TRY(walk(C, acc, krL->user, truncate_j(GL, krL->rsub), lambda, &pre));
     }
     for (size_t k = 0; k < P.Lch.size() && !krL; ++k) {
@@ -1634,8 +1719,8 @@ ttnn_status run_dense_update(ttnn_plan_s& P, void* acc, const void* data, const 
       View cur = H;
       if (krL) {
         const TNode& c1 = P.nodes[krL->ch.front()];
-        View e;
-        TTNN_TRY(kr_prefix(C, H, krL->user, c1.lo, c1.hi, krL->s, &e));
+        View e = krH;
+        if (!krH.ptr) TTNN_TRY(kr_prefix(C, H, krL->user, c1.lo, c1.hi, krL->s, &e));
         TTNN_TRY(y_chain_rest(C, e, krL->user, c1.hi, krL->hi, &cur));
       }
       for (int k = (int)P.Lch.size() - 1; k >= 0 && !krL; --k) {
@@ -1790,11 +1875,33 @@ ttnn_status run_ttn_update(ttnn_plan_s& P, void* acc, const double* const* cores
         &prog};
   const int nn = (int)P.nodes.size();
   auto R = [&](int v) { return (int64_t)ranks_in[v]; };
+  // Large cores of binary transfer nodes (binary32 plans) are contracted on
+  // the tensor cores, straight from the binary64 input, and each is read twice:
+  // up, against UX and UY of its second child at once (T[v], whose sum over a
+  // with E_v also gives E of the first child and Psi_v), and down, against the
+  // Khatri-Rao product of E_v and UX of its first child (E of the second).
+  // The general path reads such a core, as a binary32 copy, six times.
+  std::vector<char> big(nn, 0);
+  for (int v = 0; v < nn; ++v) {
+    const TNode& nd = P.nodes[v];
+    if (P.walk_f64 || v == P.root || nd.leaf || nd.ch.size() != 2 || nd.rsub == 0) continue;
+    const int64_t c1 = R(nd.ch[0]), c2 = R(nd.ch[1]);
+    TcGemm up;
+    up.type = 3;
+    up.I = R(v) * c1;
+    up.K = c2;
+    up.Jn = P.rmax + P.smax;
+    up.ldc = round_up(up.Jn, 16);
+    big[v] = R(v) * c1 * c2 * up.Jn >= kTcCoreWork && R(v) * c1 < (int64_t(1) << 31) && nd.sketched() &&
+             !P.nodes[nd.ch[1]].identity && tcg_supported(up);
+  }
+  std::vector<View> T(nn);   // [a][b1][UX columns, UY columns, padding]
   // input cores in the walk type (binary32 plans: converted copies)
   std::vector<const char*> core(nn, nullptr);
   ConvertBatch conv;
   for (int v = 0; v < nn; ++v) {
     const TNode& nd = P.nodes[v];
+    if (big[v]) continue;
     int64_t el = 1;
     if (v != P.root) el *= R(v);
     if (nd.leaf) el *= nd.n;
@@ -1830,12 +1937,52 @@ ttnn_status run_ttn_update(ttnn_plan_s& P, void* acc, const double* const* cores
     w.ld = w.ax.back().size;
     return w;
   };
+  // W(i, x) of a two-axis view with i on axis ki, as columns x < n of a product
+  auto cols_of = [](const View& w, int ki, int n) {
+    TcCols c;
+    c.p = w.ptr;
+    c.sk = vstride(w, ki);
+    c.sj = vstride(w, 1 - ki);
+    c.n = n;
+    return c;
+  };
+  // columns [j0, j0 + n) of T[v], with the last axis `last`
+  auto t_cols = [&](int v, int64_t j0, Ax last) {
+    View w = T[v];
+    w.ptr += j0 * 4;
+    w.ax.back() = last;
+    return w;
+  };
   // up sweep: UX_v (R_v x rmax), UY_v (R_v x smax), children before parents
   std::vector<View> UX(nn), UY(nn);
   for (int li = (int)P.lex.size() - 1; li >= 0; --li) {
     const int v = P.lex[li];
     if (v == P.root) continue;
     const TNode& nd = P.nodes[v];
+    if (big[v]) {
+      const int c1 = nd.ch[0], c2 = nd.ch[1];
+      TcGemm g;
+      g.type = 3;
+      g.A = cores_in[v];
+      g.I = R(v) * R(c1);
+      g.K = R(c2);
+      g.lda = R(c2);
+      g.Jn = P.rmax + P.smax;
+      g.b[0] = cols_of(UX[c2], 0, P.rmax);
+      g.b[1] = cols_of(UY[c2], 0, P.smax);
+      g.nb = 2;
+      View& t = T[v];
+      tc_gemm(C, g, {UX[c2].ptr, UY[c2].ptr}, &t.ptr, &t.ld);
+      t.ax = {Ax{AX_SK, kRankAxis - v, R(v), 0}, Ax{AX_SK, kRankAxis - c1, R(c1), 0}, Ax{AX_J, -1, t.ld, 0}};
+      for (int which = 0; which < 2; ++which) {
+        const View& uc = which == 0 ? UX[c1] : UY[c1];
+        int64_t wsI, wsX;
+        view_w(uc, 0, &wsI, &wsX);
+        TTNN_TRY(contract_view(C, t_cols(v, which * P.rmax, Ax{AX_J, -1, which == 0 ? P.rmax : P.smax, 0}), 1,
+                               uc.ptr, wsI, wsX, 2, nullptr, which == 0 ? &UX[v] : &UY[v]));
+      }
+      continue;
+    }
     for (int which = 0; which < 2; ++which) {
       const int64_t w = which == 0 ? P.rmax : P.smax;
       View cur = core_view(v);
@@ -1890,6 +2037,37 @@ ttnn_status run_ttn_update(ttnn_plan_s& P, void* acc, const double* const* cores
     if (nd.leaf || (v != P.root && nd.rsub == 0)) continue;
     for (int c : nd.ch) {
       if (P.nodes[c].rsub == 0) continue;
+      if (big[v] && c == nd.ch[0]) {
+        int64_t wsI, wsX;
+        const int ke = find_ax(E[v], AX_SK, kRankAxis - v);
+        view_w(E[v], ke, &wsI, &wsX);
+        TTNN_TRY(contract_view(C, t_cols(v, 0, Ax{AX_J, -1, P.nodes[c].rsub, 0}), 0, E[v].ptr, wsI, wsX, 2,
+                               nullptr, &E[c]));
+        continue;
+      }
+      if (big[v]) {
+        const View* f[2] = {&E[v], &UX[nd.ch[0]]};
+        const int kf[2] = {find_ax(E[v], AX_SK, kRankAxis - v), 0};
+        TcGemm g;
+        g.type = 3;
+        g.A = cores_in[v];
+        g.mn = 1;
+        g.I = R(c);
+        g.K = R(v) * R(nd.ch[0]);
+        g.lda = R(c);
+        g.Jn = P.nodes[c].rsub;
+        g.b[0].n = g.Jn;
+        g.b[0].nkr = 2;
+        for (int k = 0; k < 2; ++k) {
+          g.b[0].kr[k] = (const float*)f[k]->ptr;
+          g.b[0].krn[k] = (int32_t)f[k]->ax[kf[k]].size;
+          view_w(*f[k], kf[k], &g.b[0].ki[k], &g.b[0].kj[k]);
+        }
+        View& e = E[c];
+        tc_gemm(C, g, {f[0]->ptr, f[1]->ptr}, &e.ptr, &e.ld);
+        e.ax = {Ax{AX_SK, kRankAxis - c, R(c), 0}, Ax{AX_J, -1, g.Jn, 0}};
+        continue;
+      }
       const int bc = kRankAxis - c;
       auto is_c = [&](const Ax& a) { return a.kind == AX_SK && a.id == bc; };
       View cur = core_view(v);
@@ -1970,6 +2148,33 @@ ttnn_status run_ttn_update(ttnn_plan_s& P, void* acc, const double* const* cores
       view_w(Et, ka, &wsI, &wsX);
       Ax nax{AX_J, -1, nd.r, 0};
       View cur;
+      if (big[v]) {
+        // T[v] against E_v over a: [j][b1][columns], its UY_c2 columns kept;
+        // then UY (or the raw core) of the first child, on the FP32 units (a
+        // fourth product in a row on the tensor cores would err more)
+        const int c1 = nd.ch[0], c2 = nd.ch[1];
+        TcGemm g;
+        g.A = T[v].ptr;
+        g.mn = 1;
+        g.I = g.lda = R(c1) * T[v].ld;
+        g.K = R(v);
+        g.Jn = nd.r;
+        g.b[0] = cols_of(Et, ka, nd.r);
+        g.trans = 1;
+        int64_t ld;
+        tc_gemm(C, g, {T[v].ptr, Et.ptr}, &cur.ptr, &ld);
+        cur.ptr += (int64_t)P.rmax * 4;
+        cur.ld = T[v].ld;
+        cur.ax = {nax, Ax{AX_SK, kRankAxis - c1, R(c1), 0}, Ax{AX_SK, c2, P.nodes[c2].s, 0}};
+        const TNode& n1 = P.nodes[c1];
+        const View W1 = n1.identity ? core_view(c1) : UY[c1];
+        view_w(W1, 0, &wsI, &wsX);
+        Ax n1ax{AX_SK, c1, n1.identity ? n1.n : (int64_t)n1.s, 0};
+        View y;
+        TTNN_TRY(contract_view(C, cur, 1, W1.ptr, wsI, wsX, -1, &n1ax, &y));
+        TTNN_TRY(scatter_into(C, y, state_at(C, acc, nd.ps_off), psi_strides(C, y, nd, true), lambda));
+        continue;
+      }
       TTNN_TRY(contract_view(C, core_view(v), 0, Et.ptr, wsI, wsX, -1, &nax, &cur));
       if (nd.leaf) {
         TTNN_TRY(scatter_into(C, cur, state_at(C, acc, nd.ps_off), {1, (int64_t)nd.r}, lambda));

@@ -77,9 +77,11 @@ struct ttnn_plan_s {
   char* ws = nullptr;
   int64_t ws_bytes = 0;
   // scratch an update may plan with: unbounded while the plan is created
-  // (its workspace is sized then), later that workspace's size.  Forms that
-  // need more than the one they replace are taken only within it.
+  // (its workspace is sized then), later that workspace's size
   int64_t ws_limit = INT64_MAX;
+  // the update at hand may take the forms that need more scratch than the
+  // ones they replace (set by dense_update_need for each update)
+  bool roomy = true;
   // the recovery's own scratch: a recovery may run on another stream while
   // the next update of another state of the plan uses `ws`
   char* ws_rec = nullptr;
@@ -87,7 +89,7 @@ struct ttnn_plan_s {
   int64_t dev_bytes = 0;        // device memory the plan holds (all its allocations)
   // workspace bytes a dense update needs, by box extents, whole-tensor flag
   // and scratch limit
-  std::map<std::vector<int64_t>, int64_t> ws_need_cache;
+  std::map<std::vector<int64_t>, std::pair<int64_t, bool>> ws_need_cache;   // bytes, roomy
   ttnn::QrJob* jobs_dev = nullptr;
   std::vector<ttnn::QrJob> jobs_host;   // what jobs_dev holds (upload skipped when unchanged)
   int* kept_dev = nullptr;
@@ -132,7 +134,9 @@ ttnn_status build_plan(ttnn_plan_s& P, const ttnn_tree* tree, int32_t d, const i
 
 // Runs (or, with dry = true, sizes) one dense update.  Returns the peak
 // workspace bytes through *peak when dry.
-// Workspace bytes a dense update of `box` needs (dry run, cached per shape).
+// Workspace bytes a dense update of `box` needs (dry run, cached per shape):
+// with the forms that need the most scratch if that is within P.ws_limit, else
+// without them (P.roomy tells).
 ttnn_status dense_update_need(ttnn_plan_s& P, const Box& box, int64_t* need);
 // Workspace bytes of a CP update (any rank: ranks are taken kProjQ at a time).
 int64_t cp_update_need(const ttnn_plan_s& P);

@@ -16,6 +16,7 @@ static_assert(sizeof(LevelBatch<WalkOp, kLargeOps>) <= 32000 &&
 constexpr int kMpKC2 = 32;
 constexpr size_t kExecSmem = 48 * 1024;
 constexpr size_t kKgemmSmem = 48 * 1024;
+constexpr size_t kLaneSmem = 8 * 32 * 8;   // one partial sum per thread of a block
 
 static int exec_sms() {
   static int n = 0;
@@ -113,6 +114,99 @@ __device__ void dev_reduce(const WalkOp& op, int64_t blk) {
   const int64_t oi = (int64_t)p * c.osP + (int64_t)b * c.osB + (int64_t)q * c.osQ + (int64_t)j * c.osJ;
   const T v = (T)c.alpha * acc;
   out[oi] = c.accumulate ? out[oi] + v : v;
+}
+
+// Contraction with a contiguous axis across the lanes: the columns j (op.CH =
+// 0: isJ = 1, weights shared with the column or not) or the outputs b (op.CH =
+// 1: J = 1, wsB = 1, every lane reads the same input).  op.BG lanes take an
+// item (8, 16 or 32: the least that hold the axis, which is cut beyond 32) and
+// op.CG warps of a block share its reduction index, summed in warp order.  A
+// lane group per output (OP_CONTRACT) reads one element of each row per lane
+// when it cuts the reduction index: 200 x 200 x 30 sums of a TTN update took
+// 76 us for 48 MB; rows are read whole here.
+template <typename Tin, typename Tw, typename T, typename I>
+__device__ void dev_lane(const WalkOp& op, int64_t blk, unsigned char* smem) {
+  const Contract& c = op.c;
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const int LW = op.BG, WS = op.CG;
+  const bool jl = op.CH == 0;
+  const I LN = (I)(jl ? c.J : c.NB);
+  const I nch = (LN + LW - 1) / LW;
+  const I NBi = jl ? (I)c.NB : (I)1, Q = (I)c.Q;
+  const I items = (I)c.P * NBi * Q, units = items * nch * (I)op.nsplit;
+  const int per = 32 / LW;
+  const I u = ((I)(blk * (8 / WS)) + (I)(warp / WS)) * per + (I)(lane / LW);
+  const int s = warp % WS;
+  const bool valid = u < units;
+  I l = 0, p = 0, b = 0, q = 0, split = 0;
+  T acc = 0;
+  if (valid) {
+    const I ch = u % nch;
+    I t = u / nch;
+    l = ch * LW + (I)(lane % LW);
+    split = t / items;
+    t -= split * items;
+    q = t % Q;
+    t /= Q;
+    b = t % NBi;
+    p = t / NBi;
+    if (l < LN) {
+      const int64_t a0 = (int64_t)split * op.chunk, a1 = min(c.NI, a0 + op.chunk);
+      const int64_t part = (a1 - a0 + WS - 1) / WS;
+      int64_t i = a0 + s * part;
+      const int64_t i1 = min(a1, i + part);
+      const Tin* ip = (const Tin*)c.in + (int64_t)p * c.isP + (int64_t)q * c.isQ + (jl ? (int64_t)l * c.isJ : 0);
+      T a1s = 0, a2s = 0, a3s = 0;
+      if (c.w) {
+        const Tw* wp = (const Tw*)c.w + (int64_t)p * c.wsP + (int64_t)q * c.wsQ +
+                       (jl ? (int64_t)b * c.wsB + (int64_t)l * c.wsJ : (int64_t)l * c.wsB);
+        for (; i + 7 < i1; i += 8) {
+          T x[8], y[8];
+#pragma unroll
+          for (int k = 0; k < 8; ++k) {
+            x[k] = (T)ip[(i + k) * c.isI];
+            y[k] = (T)wp[(i + k) * c.wsI];
+          }
+          acc += x[0] * y[0];
+          a1s += x[1] * y[1];
+          a2s += x[2] * y[2];
+          a3s += x[3] * y[3];
+          acc += x[4] * y[4];
+          a1s += x[5] * y[5];
+          a2s += x[6] * y[6];
+          a3s += x[7] * y[7];
+        }
+        for (; i < i1; ++i) acc += (T)ip[i * c.isI] * (T)wp[i * c.wsI];
+      } else {
+        for (; i + 3 < i1; i += 4) {
+          acc += (T)ip[i * c.isI];
+          a1s += (T)ip[(i + 1) * c.isI];
+          a2s += (T)ip[(i + 2) * c.isI];
+          a3s += (T)ip[(i + 3) * c.isI];
+        }
+        for (; i < i1; ++i) acc += (T)ip[i * c.isI];
+      }
+      acc = (acc + a1s) + (a2s + a3s);
+    }
+  }
+  if (WS > 1) {
+    T* red = (T*)smem;   // [8][32]
+    red[warp * 32 + lane] = acc;
+    __syncthreads();
+    if (s != 0) return;
+    for (int k = 1; k < WS; ++k) acc += red[(warp + k) * 32 + lane];
+  }
+  if (!valid || l >= LN) return;
+  const I j = jl ? l : (I)0;
+  if (!jl) b = l;
+  if (op.nsplit > 1) {
+    const int64_t o = (((int64_t)p * c.NB + b) * c.Q + q) * c.J + j;
+    ((T*)op.partial)[(int64_t)split * (c.P * c.NB * c.Q * c.J) + o] = acc;
+  } else {
+    T* out = (T*)c.out + (int64_t)p * c.osP + (int64_t)b * c.osB + (int64_t)q * c.osQ + (int64_t)j * c.osJ;
+    const T v = (T)c.alpha * acc;
+    *out = c.accumulate ? *out + v : v;
+  }
 }
 
 // Mode product as a batched small GEMM over one chunk of CH batch items:
@@ -623,6 +717,11 @@ __device__ __forceinline__ void dispatch(const WalkOp& op, int64_t blk, unsigned
       else if (op.tin == ET_F64) dev_contract<double, double, double, double, I>(op, blk);
       else dev_contract<float, double, double, double, I>(op, blk);
       break;
+    case OP_LANE:
+      if (!F64) dev_lane<T, T, T, I>(op, blk, dsm);
+      else if (op.tin == ET_F64) dev_lane<double, double, double, I>(op, blk, dsm);
+      else dev_lane<float, double, double, I>(op, blk, dsm);
+      break;
     case OP_SCATTER: dev_scatter<T, I>(op, blk); break;
     case OP_REDUCE: dev_reduce<T, I>(op, blk); break;
     case OP_EYE:
@@ -779,10 +878,37 @@ int64_t plan_contract(Op& op) {
   // binary32 mode products with reductions longer than the weight-stationary
   // form holds (e.g. a rank-200 TTN core against a sketch block) take the
   // split-K tiled form
-  if (total >= want / 4 && c.w && c.wsQ == 0 && c.wsJ == 0 && c.wsP == 0 && c.NI > kWsMaxNI &&
+  // (a product of few tiles would leave most SMs idle behind the latency of
+  // its K steps: 24 tiles of 200 rows took 31 us; the lane form below spreads it)
+  const bool few = ceil_div(c.P * c.Q * c.J, (int64_t)kKgNT) * ceil_div(c.NB, (int64_t)kKgMB) * 2 < exec_sms() &&
+                   c.J >= 16 && c.isJ == 1;
+  if (total >= want / 4 && c.w && c.wsQ == 0 && c.wsJ == 0 && c.wsP == 0 && c.NI > kWsMaxNI && !few &&
       c.NI < (int64_t(1) << 31) && op.tin == ET_F32 && op.tw == ET_F32 && op.tout == ET_F32)
     return kgemm();
   if (total >= want / 4 && mp_tiling(op)) return 0;
+  // a contiguous output axis across the lanes, where a lane group per output
+  // would cut the reduction index over the lanes of a warp
+  const bool jl = c.J >= 4 && c.isJ == 1 && (!c.w || c.wsJ <= 1);
+  const bool bl = c.J == 1 && c.NB >= 8 && c.w && c.wsB == 1;
+  if ((jl || bl) && (total * 2 <= want || few) && c.NI >= 16) {
+    const int64_t ln = jl ? c.J : c.NB;
+    const int lw = ln <= 8 ? 8 : ln <= 16 ? 16 : 32;
+    const int64_t units = (jl ? c.P * c.NB * c.Q : c.P * c.Q) * ceil_div(ln, (int64_t)lw);
+    const int64_t warps = (int64_t)exec_sms() * 24;
+    op.kind = OP_LANE;
+    op.CH = jl ? 0 : 1;
+    op.BG = lw;
+    int ws = 1;
+    while (ws < 8 && ceil_div(units, 32 / lw) * ws < warps && c.NI >= 16 * ws) ws <<= 1;
+    op.CG = ws;
+    int64_t ns = 1;
+    if (c.NI >= 2048)
+      ns = std::max<int64_t>(1, std::min<int64_t>(warps / (ceil_div(units, 32 / lw) * ws), c.NI / 512));
+    op.chunk = ceil_div(c.NI, std::min<int64_t>(ns, 256));
+    op.nsplit = (int)ceil_div(c.NI, op.chunk);
+    op.blocks = ceil_div(ceil_div(units * op.nsplit, 32 / lw), 8 / ws);
+    return op.nsplit > 1 ? total * op.nsplit : 0;
+  }
   int g = 1;
   while (g < 32 && total * g < want && c.NI >= 8 * g) g <<= 1;
   op.g = g;
@@ -840,7 +966,8 @@ void Program::add(Op op, const void* in1, const void* in2) {
                     : op.kind == OP_PROJ  ? (const void*)op.pj.out
                     : op.kind == OP_OUTER ? op.ou.out
                                           : op.c.out;
-  if (((op.kind == OP_CONTRACT || op.kind == OP_KGEMM) && op.nsplit > 1) || op.kind == OP_KRED) {
+  if (((op.kind == OP_CONTRACT || op.kind == OP_LANE || op.kind == OP_KGEMM) && op.nsplit > 1) ||
+      op.kind == OP_KRED) {
     Op part = op;
     part.level = lvl;
     ops_.push_back(part);
@@ -859,8 +986,52 @@ void Program::add(Op op, const void* in1, const void* in2) {
     if ((const char*)out >= b.lo && (const char*)out < b.hi) b.level = std::max(b.level, lvl);
 }
 
+void Program::add(const TcOp& op, std::initializer_list<const void*> in) {
+  int lvl = 0;
+  for (const void* p : in) lvl = std::max(lvl, level_of(p));
+  tcs_.push_back(op);
+  tcs_.back().level = ++lvl;
+  const char* out = (const char*)op.g.C;
+  for (Buf& b : bufs_)
+    if (out >= b.lo && out < b.hi) b.level = std::max(b.level, lvl);
+}
+
+// The tensor-core GEMMs of a level: their operands in one launch, then the
+// products (those of several plans, with error words of their own, apart).
+ttnn_status Program::run_tc(int lvl, cudaStream_t st) const {
+  std::vector<TcGemm> g;
+  std::vector<void*> prep;
+  for (const TcOp& o : tcs_) {
+    if (o.level != lvl) continue;
+    g.push_back(o.g);
+    prep.push_back(o.prep);
+  }
+  if (g.empty()) return TTNN_OK;
+  TTNN_TRY(tcg_prepare(g.data(), (int)g.size(), prep.data(), st));
+  const TcOp* first = nullptr;
+  std::vector<TcGemm> run;
+  auto flush = [&]() -> ttnn_status {
+    if (run.empty()) return TTNN_OK;
+    TTNN_TRY(tcg_run(run.data(), (int)run.size(), first->pieces, tcg_sms(), first->err, tcg_wait_ns(), st));
+    run.clear();
+    return TTNN_OK;
+  };
+  for (const TcOp& o : tcs_) {
+    if (o.level != lvl) continue;
+    if (run.empty()) first = &o;
+    else if (o.pieces != first->pieces) {
+      TTNN_TRY(flush());
+      first = &o;
+    }
+    run.push_back(o.g);
+    run.back().prep = o.prep;
+  }
+  return flush();
+}
+
 int Program::levels() const {
   int m = 0;
+  for (const TcOp& o : tcs_) m = std::max(m, o.level);
   for (const Op& o : ops_) m = std::max(m, o.level);
   return m;
 }
@@ -943,9 +1114,9 @@ static ttnn_status launch_group(LaunchGroup g, const Op* const* ops, int n, cuda
     } else if (g == LG_F32_WIDE) {
       level_kernel<false, int64_t, CAP><<<gr, kExecThreads, kExecSmem, st>>>(b);
     } else if (g == LG_F64) {
-      level_kernel<true, uint32_t, CAP><<<gr, kExecThreads, 0, st>>>(b);
+      level_kernel<true, uint32_t, CAP><<<gr, kExecThreads, kLaneSmem, st>>>(b);
     } else {
-      level_kernel<true, int64_t, CAP><<<gr, kExecThreads, 0, st>>>(b);
+      level_kernel<true, int64_t, CAP><<<gr, kExecThreads, kLaneSmem, st>>>(b);
     }
   }
   if (blocks < 0) {
@@ -1030,9 +1201,9 @@ static ttnn_status dump_op(const Op& o, int lvl, cudaStream_t st) {
 
 ttnn_status Program::run(cudaStream_t st, bool dump) {
   const int L = levels();
-  // per level: the split-K GEMM ops in one launch of their kernel, the other
-  // ops in one launch per type; when a level has both, the GEMM launch goes
-  // on the fork stream and runs beside the others
+  // per level: the tensor-core GEMMs, the split-K GEMM ops in one launch of
+  // their kernel, the other ops in one launch per type; when a level has
+  // both, the GEMM launches go on the fork stream and run beside the others
   ForkStream* fs = nullptr;
   std::vector<const Op*> group[LG_COUNT];
   for (int lvl = 1; lvl <= L; ++lvl) {
@@ -1048,7 +1219,9 @@ ttnn_status Program::run(cudaStream_t st, bool dump) {
       group[g].push_back(&o);
       other = other || g != LG_KGEMM;
     }
-    const bool fork = other && !group[LG_KGEMM].empty();
+    bool tc = false;
+    for (const TcOp& o : tcs_) tc = tc || o.level == lvl;
+    const bool fork = other && (tc || !group[LG_KGEMM].empty()) && !dump;
     cudaStream_t gst = st;   // stream of the GEMM launches
     if (fork) {
       if (!fs) TTNN_TRY(fork_stream(&fs));
@@ -1058,6 +1231,7 @@ ttnn_status Program::run(cudaStream_t st, bool dump) {
         gst = fs->st;
       }
     }
+    if (tc) TTNN_TRY(run_tc(lvl, gst));
     for (int g = 0; g < LG_COUNT; ++g)
       if (!group[g].empty())
         TTNN_TRY(launch_ops((LaunchGroup)g, group[g], g == LG_KGEMM ? gst : st));

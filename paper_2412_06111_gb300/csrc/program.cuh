@@ -4,8 +4,10 @@
 // batched launch of a kernel that dispatches per block on the op kind.
 #pragma once
 
+#include <initializer_list>
 #include <vector>
 
+#include "gemm_tc.cuh"
 #include "kernels.cuh"
 
 namespace ttnn {
@@ -14,6 +16,7 @@ enum OpKind {
   OP_CONTRACT = 0, OP_MP = 1, OP_SCATTER = 2, OP_REDUCE = 3, OP_EYE = 4, OP_KRED = 5,
   OP_PROJ = 6,    // projections of CP factors onto DRM factors (binary64)
   OP_OUTER = 7,   // sums of outer products of vector products into a sketch
+  OP_LANE = 9,    // contraction with a contiguous output axis across the lanes
   OP_KGEMM = 8    // split-K register-tiled contraction (long reduction, <= 32 outputs per column)
 };
 
@@ -58,7 +61,7 @@ struct Op {
   int nsplit = 1;       // split of the reduction index (partials + OP_REDUCE)
   int64_t chunk = 0;
   void* partial = nullptr;
-  int BG = 0, CG = 0, CH = 0;   // OP_MP tiling
+  int BG = 0, CG = 0, CH = 0;   // OP_MP tiling; OP_LANE: lanes of an item, warps, lane axis
   int64_t eye_n = 0;            // OP_EYE: n x n identity at c.out (f64)
   int64_t blocks = 0;
   int level = 0;
@@ -103,23 +106,39 @@ struct LevelBatch {
   OpT ops[CAP];
 };
 
+// A recorded tensor-core GEMM: its prepared operand, room for pieces (shared
+// by the products of a program: its launches run in order), error word.
+struct TcOp {
+  TcGemm g;
+  void* prep = nullptr;
+  void* pieces = nullptr;
+  int* err = nullptr;
+  int level = 0;
+};
+
 class Program {
  public:
   // Registers a buffer written by the program (or produced before it, level 0).
   void buffer(const void* p, int64_t bytes, int level = 0);
   // Records an op; its level follows the buffers it reads.
   void add(Op op, const void* in1, const void* in2 = nullptr);
+  // Records a tensor-core GEMM that reads `in` (A and what B is made of).
+  void add(const TcOp& op, std::initializer_list<const void*> in);
   // Launches every level in order on `st`; dump: print each op (level, kind,
   // shape, blocks) to stderr first (a plan's TTNN_FLAG_DUMP_PROGRAM).
   ttnn_status run(cudaStream_t st, bool dump = false);
   void clear() {
     ops_.clear();
+    tcs_.clear();
     bufs_.clear();
   }
   // Appends another program's ops (levels kept): programs over disjoint
   // buffers then share their level launches.
-  void absorb(const Program& o) { ops_.insert(ops_.end(), o.ops_.begin(), o.ops_.end()); }
-  size_t size() const { return ops_.size(); }
+  void absorb(const Program& o) {
+    ops_.insert(ops_.end(), o.ops_.begin(), o.ops_.end());
+    tcs_.insert(tcs_.end(), o.tcs_.begin(), o.tcs_.end());
+  }
+  size_t size() const { return ops_.size() + tcs_.size(); }
   int levels() const;
 
  private:
@@ -129,7 +148,9 @@ class Program {
     int level;
   };
   int level_of(const void* p) const;
+  ttnn_status run_tc(int lvl, cudaStream_t st) const;
   std::vector<Op> ops_;
+  std::vector<TcOp> tcs_;
   std::vector<Buf> bufs_;
 };
 
