@@ -231,17 +231,16 @@ __global__ void __launch_bounds__(kZThreads, 1)
             const uint32_t sa = base + stage * kZStage;
             const uint32_t sb = b_base + bb * b_bytes + h * (kZK * 2);
             const uint32_t d = tmem + buf * acc_cols;
+            const uint64_t a = sdesc(sa, MN ? 4096 : 16, 1024), b = sdesc(sb, 16, 1024);
 #pragma unroll
             for (int i = 0; i < kZDigits; ++i) {
               // digit i of A against digits 0 .. 7 - i of B: orders i .. 7
               const uint32_t id = idesc_f16(kTileM, (kZDigits - i) * p.Npad, MN);
 #pragma unroll
               for (int kk = 0; kk < kZK / 16; ++kk) {
-                const uint64_t da =
-                    MN ? sdesc(sa + i * 8192 + kk * 2048, 4096, 1024)
-                       : sdesc(sa + (i >> 1) * 16384 + (i & 1) * 64 + kk * 32, 16, 1024);
-                const uint64_t db = sdesc(sb + kk * 32, 16, 1024);
-                mma_bf16(d + i * p.Npad, da, db, id, i > 0 || kk > 0);
+                mma_bf16(d + i * p.Npad,
+                         sdesc_at(a, MN ? i * 8192 + kk * 2048 : (i >> 1) * 16384 + (i & 1) * 64 + kk * 32),
+                         sdesc_at(b, kk * 32), id, i > 0 || kk > 0);
               }
             }
             mma_commit(smem_u32(&bar_empty[stage]));

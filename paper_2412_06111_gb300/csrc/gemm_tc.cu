@@ -313,18 +313,17 @@ __global__ void __launch_bounds__(tcg_threads<EPI>(), 1)
             }
             fence_after();
             const uint32_t d = tmem + buf * NACC * p.Npad;
+            const uint64_t a = sdesc(sa, MN ? kBox : 16, 1024), b = sdesc(sb, 16, 1024);
 #pragma unroll
             for (int ia = 0; ia < NS; ++ia) {
               // piece ia of A against pieces 0 .. NS - 1 - ia of B: orders ia .. NS - 1
               const uint32_t id = idesc_bf16(kTileM, (NS - ia) * p.Npad, MN);
 #pragma unroll
               for (int kk = k0; kk < k0 + n; ++kk) {
-                const uint64_t da =
-                    MN ? sdesc(sa + ia * kPiece + kk * 2048, kBox, 1024)
-                       : sdesc(sa + ia * kPiece + (kk >> 2) * kBox + (kk & 3) * 32, 16, 1024);
-                const uint64_t db =
-                    sdesc(sb + (kk >> 2) * (p.Npad * 128) + (kk & 3) * 32, 16, 1024);
-                mma_bf16(d + ia * p.Npad, da, db, id, steps > 0 || kk > k0 || ia > 0);
+                mma_bf16(d + ia * p.Npad,
+                         sdesc_at(a, ia * kPiece + (MN ? kk * 2048 : (kk >> 2) * kBox + (kk & 3) * 32)),
+                         sdesc_at(b, (kk >> 2) * (p.Npad * 128) + (kk & 3) * 32), id,
+                         kk > k0 || ia > 0 || steps > 0);
               }
             }
             steps += n;

@@ -1,20 +1,28 @@
 // First-level pass for the narrow and split storage formats, on the bfloat16
 // tcgen05 tensor cores (sm_103a).  Same products as the BF16 pass:
 //   D1 = M B_R^T (nL x wR),  D2 = M^T B_L^T (nR x wL),
-// but the tile of M arrives in its storage format and converter warps turn
-// it into bfloat16 operand tiles in shared memory before the MMAs:
+// but converter warps turn the tile of M from its storage format into bfloat16
+// operand tiles in shared memory before the MMAs:
 //
 //  SPLIT (binary32 M): hi = bf16(M), lo = bf16(M - hi); both tiles are
-//    multiplied by the same bfloat16 DRM tile and summed in the TMEM
-//    accumulators (four MMA streams per tile).  The conversion is in place:
-//    each 64-column half of the binary32 tile (32 KB) becomes its hi and lo
-//    swizzled boxes (16 KB each) in the same bytes.
-//  FP8 (E4M3 M with one binary32 scale per 128 x 128 tile): the tile is
-//    dequantised to bf16(f32(q * s)) into a separate bfloat16 operand tile.
+//    multiplied by the same bfloat16 DRM tile (SPLIT3: hi also by the DRM
+//    block's own lo part) and summed in the TMEM accumulators.  The converters
+//    load M to registers, a tile ahead: 64 KB per SM stay in flight while the
+//    two stages of operand tiles (64 KB each) are written or multiplied.  By
+//    TMA and an in-place conversion, which is how this was done before, a
+//    stage could not fetch while it was converted.
+//  FP8 (E4M3 M with one binary32 scale per 128 x 128 tile): the tile arrives by
+//    TMA and is dequantised to bf16(f32(q * s)) into an operand tile.
 //
-// Pipeline per stage: TMA (raw tile + DRM tile) -> converters (4 warps) ->
-// MMA issuer -> stage free.  Warp roles (448 threads): warp 0 TMA producer,
-// warp 1 TMEM owner + MMA issuer, warps 2-5 epilogue, warps 6-13 converters.
+// Bound: HBM and the converters' share of it for SPLIT (48^5 bf16 hi + lo: 188
+// us without the MMAs, 190 with them, 150 at HBM speed; 205 before), for SPLIT3
+// with 48 MMAs per tile both (48^5: 219 without, 188 the MMAs alone, 229
+// together; 255 before), for FP8 the chain of TMA, conversion and MMAs (48^5:
+// 114; 38 at HBM speed; 118 before, and 118 with 16 converter warps).
+//
+// Pipeline per stage: TMA (DRM tile, FP8 raw tile) and converters -> MMA
+// issuer -> stage free.  Warp roles: warp 0 TMA producer, warp 1 TMEM owner +
+// MMA issuer, warps 2-5 epilogue, then 16 (FP8: 8) converter warps.
 // Every wait is bounded (globaltimer); on expiry the kernel records an error
 // bit, drains its own copies and MMAs, frees TMEM and returns.
 #include <cuda_bf16.h>
@@ -28,24 +36,27 @@
 namespace ttnn {
 namespace tc {
 
-constexpr int kConvThreads = 256;   // converter warps 6..13
-constexpr int kCvtThreads = 192 + kConvThreads;
 constexpr int MODE_SPLIT = 1;
 constexpr int MODE_FP8 = 2;
 constexpr int MODE_SPLIT3 = 3;   // binary32 M and binary32 DRM blocks, both split
 template <int MODE>
 __host__ __device__ constexpr bool is_split() { return MODE == MODE_SPLIT || MODE == MODE_SPLIT3; }
 
+// Threads of the converter warps, warp 6 on.
+template <int MODE>
+__host__ __device__ constexpr int conv_threads() { return is_split<MODE>() ? 512 : 256; }
+
 struct CvtParams {
+  const float* A;        // SPLIT: M, row-major
   int64_t nL, nR;
   int C, G, nb, tiles, stages;
   int wRpad, wLpad;
   int ncolt;             // column tiles of M (row stride of the scale array)
   const float* scale;    // FP8: [ceil(nL/128)][ncolt]
   float* D1;             // [nL][wRpad] (C == 1)
-  float* D1p;            // [C][nb*128][wRpad] chunk partials (C > 1)
+  float* D1p;            // [C][nb * 4][wRpad][32] chunk partials (C > 1)
   int* cnt;              // [nb][4] chunk arrivals per row block and epilogue warp, zero at launch
-  int discard;           // partial rows are whole 128-byte lines
+  int discard;           // partials are whole 128-byte lines
   float* D2p;            // [G][C*tiles*128][wLpad]
   int* err;
 };
@@ -61,24 +72,6 @@ struct Layout {
   static constexpr uint32_t bparts = MODE == MODE_SPLIT3 ? 2u : 1u;
 };
 
-__device__ __forceinline__ void named_sync_conv() {
-  asm volatile("bar.sync 1, %0;" ::"n"(kConvThreads) : "memory");
-}
-// AND of `ok` over the 128 converter threads (named barrier 1 with a
-// reduction): every converter takes the same branch, so the named barriers
-// of the in-place conversion are always reached by all of them.
-__device__ __forceinline__ bool conv_all(bool ok) {
-  uint32_t r;
-  asm volatile(
-      "{\n\t.reg .pred p, q;\n\t"
-      "setp.ne.u32 p, %1, 0;\n\t"
-      "bar.red.and.pred q, 1, %2, p;\n\t"
-      "selp.u32 %0, 1, 0, q;\n\t}\n"
-      : "=r"(r)
-      : "r"((uint32_t)ok), "n"(kConvThreads)
-      : "memory");
-  return r != 0;
-}
 __device__ __forceinline__ void fence_proxy_async() {
   asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
 }
@@ -87,39 +80,25 @@ __device__ __forceinline__ uint32_t pack_bf16(float a, float b) {
   return *reinterpret_cast<const uint32_t*>(&v);
 }
 
-// SPLIT: one 64-column half (h) of the binary32 tile at `tile`, in place.
-// Raw layout: [128 rows][64 floats] (256-byte rows).  Output: hi box at
-// tile + h*32K, lo box at tile + h*32K + 16K, each [128 rows][64 bf16] with
-// the 128-byte swizzle (16-byte chunk c of row y at chunk c ^ (y & 7)).
-// Thread task: 4 consecutive floats of a row (16 lanes cover a row, so every
-// shared-memory phase touches 128 contiguous bytes), giving 8 bytes of hi
-// and 8 bytes of lo.
-__device__ __forceinline__ void convert_split_half(uint8_t* tile, int h, int ct) {
-  uint8_t* half = tile + h * 32768;
-  constexpr int kTasks = 2048 / kConvThreads;
-  float4 v[kTasks];
-#pragma unroll
-  for (int i = 0; i < kTasks; ++i) {
-    const int id = i * kConvThreads + ct;
-    v[i] = *reinterpret_cast<const float4*>(half + (id >> 4) * 256 + (id & 15) * 16);
-  }
-  named_sync_conv();   // every read of this half precedes every write into it
-#pragma unroll
-  for (int i = 0; i < kTasks; ++i) {
-    const int id = i * kConvThreads + ct;
-    const int y = id >> 4, q = id & 15;   // floats 4q..4q+3 of row y
-    const float h0 = __bfloat162float(__float2bfloat16_rn(v[i].x));
-    const float h1 = __bfloat162float(__float2bfloat16_rn(v[i].y));
-    const float h2 = __bfloat162float(__float2bfloat16_rn(v[i].z));
-    const float h3 = __bfloat162float(__float2bfloat16_rn(v[i].w));
-    const uint2 hi = make_uint2(pack_bf16(h0, h1), pack_bf16(h2, h3));
-    // the differences are exact in binary32
-    const uint2 lo = make_uint2(pack_bf16(v[i].x - h0, v[i].y - h1),
-                                pack_bf16(v[i].z - h2, v[i].w - h3));
-    const uint32_t off = (uint32_t)(y * 128 + (((q >> 1) ^ (y & 7)) << 4) + (q & 1) * 8);
-    *reinterpret_cast<uint2*>(half + off) = hi;
-    *reinterpret_cast<uint2*>(half + 16384 + off) = lo;
-  }
+// 16 bytes read once.  Shared memory leaves 28 KB of L1, less than the loads
+// that are in flight: they are kept from allocating there (48^5 binary32: 229
+// us against 238).
+__device__ __forceinline__ float4 ld_once(const float* p) {
+  float4 v;
+  asm volatile("ld.global.nc.L1::no_allocate.v4.f32 {%0, %1, %2, %3}, [%4];"
+               : "=f"(v.x), "=f"(v.y), "=f"(v.z), "=f"(v.w)
+               : "l"(p));
+  return v;
+}
+// SPLIT: four neighbouring entries of a row as 8 bytes of the hi tile and 8 of
+// the lo tile (16 KB on).
+__device__ __forceinline__ void split_store(uint32_t addr, float4 v) {
+  const uint32_t h0 = pack_bf16(v.x, v.y), h1 = pack_bf16(v.z, v.w);
+  // the differences are exact in binary32
+  const uint32_t l0 = pack_bf16(v.x - __uint_as_float(h0 << 16), v.y - __uint_as_float(h0 & 0xFFFF0000u));
+  const uint32_t l1 = pack_bf16(v.z - __uint_as_float(h1 << 16), v.w - __uint_as_float(h1 & 0xFFFF0000u));
+  asm volatile("st.shared.v2.b32 [%0], {%1, %2};" ::"r"(addr), "r"(h0), "r"(h1) : "memory");
+  asm volatile("st.shared.v2.b32 [%0], {%1, %2};" ::"r"(addr + 16384), "r"(l0), "r"(l1) : "memory");
 }
 
 __device__ __forceinline__ float2 e4m3x2_to_float2(uint32_t two) {
@@ -130,10 +109,10 @@ __device__ __forceinline__ float2 e4m3x2_to_float2(uint32_t two) {
 
 // FP8: the [128][128] E4M3 tile at `raw` -> two bf16 boxes at `op`, op + 16K.
 __device__ __forceinline__ void convert_fp8(const uint8_t* raw, uint8_t* op, float s, int ct) {
-  constexpr int kTasks = 2048 / kConvThreads;
+  constexpr int kConv = conv_threads<MODE_FP8>(), kTasks = 2048 / kConv;
 #pragma unroll
   for (int i = 0; i < kTasks; ++i) {
-    const int id = i * kConvThreads + ct;
+    const int id = i * kConv + ct;
     const int y = id >> 4, c = id & 15;
     const uint2 q = *reinterpret_cast<const uint2*>(raw + y * 128 + c * 8);
     const float2 f0 = e4m3x2_to_float2(q.x & 0xFFFFu), f1 = e4m3x2_to_float2(q.x >> 16);
@@ -149,7 +128,7 @@ __device__ __forceinline__ void convert_fp8(const uint8_t* raw, uint8_t* op, flo
 }
 
 template <int MODE>
-__global__ void __launch_bounds__(kCvtThreads, 1)
+__global__ void __launch_bounds__(192 + conv_threads<MODE>(), 1)
     pass_cvt_kernel(const __grid_constant__ CUtensorMap mapA,
                     const __grid_constant__ CUtensorMap mapBR,
                     const __grid_constant__ CUtensorMap mapBL,
@@ -169,7 +148,6 @@ __global__ void __launch_bounds__(kCvtThreads, 1)
   const uint32_t br_bytes = (uint32_t)p.wRpad * 128 * 2;
   const uint32_t bl_bytes = (uint32_t)p.wLpad * 128 * 2;
   const uint32_t stage_bytes = Lay::op + Lay::raw + Lay::bparts * br_bytes;
-  const uint32_t raw_tx = is_split<MODE>() ? 65536u : 16384u;
   const uint32_t base = smem_u32(smem);
   const uint32_t bl_base = base + S * stage_bytes;
 
@@ -185,7 +163,7 @@ __global__ void __launch_bounds__(kCvtThreads, 1)
     abort_flag = 0;
     for (int s = 0; s < S; ++s) {
       mbar_init(smem_u32(&bar_full[s]), 1);
-      mbar_init(smem_u32(&bar_conv[s]), kConvThreads / 32);
+      mbar_init(smem_u32(&bar_conv[s]), conv_threads<MODE>() / 32);
       mbar_init(smem_u32(&bar_empty[s]), 1);
     }
     for (int k = 0; k < 2; ++k) {
@@ -242,13 +220,8 @@ __global__ void __launch_bounds__(kCvtThreads, 1)
           const uint32_t sb = base + stage * stage_bytes;
           const uint32_t bar = smem_u32(&bar_full[stage]);
           const int col = (int)(col0 + t * kTileN);
-          mbar_expect_tx(bar, raw_tx + Lay::bparts * br_bytes);
-          if (is_split<MODE>()) {
-            tma_2d(sb, &mapA, col, row, bar, pol_stream);
-            tma_2d(sb + 32768, &mapA, col + 64, row, bar, pol_stream);
-          } else {
-            tma_2d(sb + Lay::op, &mapA, col, row, bar, pol_stream);
-          }
+          mbar_expect_tx(bar, Lay::raw + Lay::bparts * br_bytes);
+          if (!is_split<MODE>()) tma_2d(sb + Lay::op, &mapA, col, row, bar, pol_stream);
           const uint32_t sbr = sb + Lay::op + Lay::raw;
           tma_2d(sbr, &mapBR, col, 0, bar, pol_keep);
           tma_2d(sbr + br_bytes / 2, &mapBR, col + 64, 0, bar, pol_keep);
@@ -280,7 +253,7 @@ __global__ void __launch_bounds__(kCvtThreads, 1)
       // ---------------- MMA issuer ----------------
       const uint32_t id1 = idesc_bf16(kTileM, p.wRpad, false);
       const uint32_t id2 = idesc_bf16(kTileN, p.wLpad, true);
-      constexpr int nparts = is_split<MODE>() ? 2 : 1;   // hi (+ lo)
+      constexpr int nparts = MODE == MODE_SPLIT3 ? 3 : MODE == MODE_SPLIT ? 2 : 1;
       int stage = 0;
       uint32_t ph = 0;
       bool ok = true;
@@ -290,53 +263,35 @@ __global__ void __launch_bounds__(kCvtThreads, 1)
         if (ok) ok = mbar_wait(smem_u32(&bar_blfull[buf]), (u >> 1) & 1, &abort_flag);
         if (!ok) break;
         fence_after();
-        const uint32_t blb = bl_base + buf * Lay::bparts * bl_bytes;
+        const uint64_t bl = sdesc(bl_base + buf * Lay::bparts * bl_bytes, 16, 1024);
         const uint32_t d1 = tmem + d1_col + buf * p.wRpad;
         for (int t = 0; t < nt; ++t) {
-          ok = mbar_wait(smem_u32(&bar_conv[stage]), ph, &abort_flag);
+          ok = mbar_wait(smem_u32(&bar_full[stage]), ph, &abort_flag) &&
+               mbar_wait(smem_u32(&bar_conv[stage]), ph, &abort_flag);
           if (!ok) break;
           fence_after();
           const uint32_t sa = base + stage * stage_bytes;
-          const uint32_t sbr = sa + Lay::op + Lay::raw;
-#pragma unroll
-          for (int part = 0; part < nparts; ++part) {
-            const uint32_t pa = sa + part * 16384;
-#pragma unroll
-            for (int kk = 0; kk < 8; ++kk) {
-              const uint64_t da = sdesc(pa + (kk >> 2) * Lay::box + (kk & 3) * 32, 16, 1024);
-              const uint64_t db = sdesc(sbr + (kk >> 2) * (br_bytes / 2) + (kk & 3) * 32, 16, 1024);
-              mma_bf16(d1, da, db, id1, (part | t | kk) != 0);
-            }
-          }
-          if (MODE == MODE_SPLIT3) {
-            // hi part of M against the lo part of the DRM block
-#pragma unroll
-            for (int kk = 0; kk < 8; ++kk) {
-              const uint64_t da = sdesc(sa + (kk >> 2) * Lay::box + (kk & 3) * 32, 16, 1024);
-              const uint64_t db =
-                  sdesc(sbr + br_bytes + (kk >> 2) * (br_bytes / 2) + (kk & 3) * 32, 16, 1024);
-              mma_bf16(d1, da, db, id1, true);
-            }
-          }
+          const uint64_t a1 = sdesc(sa, 16, 1024), a2 = sdesc(sa, Lay::box, 1024);
+          const uint64_t br = sdesc(sa + Lay::op + Lay::raw, 16, 1024);
           const uint32_t d2 = tmem + d2_col + t * p.wLpad;
+          // hi and lo part of M against the (hi part of the) DRM block, then
+          // the hi part of M against the DRM block's lo part
 #pragma unroll
           for (int part = 0; part < nparts; ++part) {
-            const uint32_t pa = sa + part * 16384;
 #pragma unroll
-            for (int kk = 0; kk < 8; ++kk) {
-              const uint64_t da = sdesc(pa + kk * 2048, Lay::box, 1024);
-              const uint64_t db = sdesc(blb + (kk >> 2) * (bl_bytes / 2) + (kk & 3) * 32, 16, 1024);
-              mma_bf16(d2, da, db, id2, (part | u | kk) != 0);
-            }
+            for (int kk = 0; kk < 8; ++kk)
+              mma_bf16(d1,
+                       sdesc_at(a1, (part == 1 ? 16384 : 0) + (kk >> 2) * Lay::box + (kk & 3) * 32),
+                       sdesc_at(br, (part == 2 ? br_bytes : 0) + (kk >> 2) * (br_bytes / 2) + (kk & 3) * 32),
+                       id1, part > 0 || kk > 0 || t > 0);
           }
-          if (MODE == MODE_SPLIT3) {
 #pragma unroll
-            for (int kk = 0; kk < 8; ++kk) {
-              const uint64_t da = sdesc(sa + kk * 2048, Lay::box, 1024);
-              const uint64_t db =
-                  sdesc(blb + bl_bytes + (kk >> 2) * (bl_bytes / 2) + (kk & 3) * 32, 16, 1024);
-              mma_bf16(d2, da, db, id2, true);
-            }
+          for (int part = 0; part < nparts; ++part) {
+#pragma unroll
+            for (int kk = 0; kk < 8; ++kk)
+              mma_bf16(d2, sdesc_at(a2, (part == 1 ? 16384 : 0) + kk * 2048),
+                       sdesc_at(bl, (part == 2 ? bl_bytes : 0) + (kk >> 2) * (bl_bytes / 2) + (kk & 3) * 32),
+                       id2, part > 0 || kk > 0 || u > 0);
           }
           mma_commit(smem_u32(&bar_empty[stage]));
           if (++stage == S) {
@@ -360,32 +315,73 @@ __global__ void __launch_bounds__(kCvtThreads, 1)
     int stage = 0;
     uint32_t ph = 0;
     bool ok = true;
-    // FP8: the scale of the next tile is loaded while the current one converts
-    auto scale_of = [&](int u, int t) -> float {
-      if (MODE != MODE_FP8 || u >= nu) return 1.f;
-      return __ldg(p.scale + (int64_t)(b0 + u) * p.ncolt + (int)(col0 / kTileN) + t);
-    };
-    float s_next = scale_of(0, 0);
-    for (int u = 0; u < nu && ok; ++u) {
-      for (int t = 0; t < nt; ++t) {
-        const float s_cur = s_next;
-        s_next = t + 1 < nt ? scale_of(u, t + 1) : scale_of(u + 1, 0);
-        // all converters agree before any of them enters a named barrier
-        ok = conv_all(mbar_wait(smem_u32(&bar_full[stage]), ph, &abort_flag));
-        if (!ok) break;
-        uint8_t* st = smem + stage * stage_bytes;
-        if (is_split<MODE>()) {
-          convert_split_half(st, 0, ct);
-          convert_split_half(st, 1, ct);
-        } else {
-          convert_fp8(st + Lay::op, st, s_cur, ct);
+    if constexpr (is_split<MODE>()) {
+      // Warp w takes rows w, w + 16, ... of a tile, a lane 16 bytes of each
+      // (the whole 512-byte row per load; a half warp stores the 128 swizzled
+      // bytes of one box row).  An entry's place is refilled with the next
+      // tile's as soon as it is stored: 64 KB per SM stay in flight.
+      constexpr int NQ = 8;
+      const int w = ct >> 5;
+      float4 v[NQ];
+      const int64_t step = 16 * p.nR;
+      auto load = [&](int q, const float* src, int64_t rows) {
+        v[q] = 16 * q < rows ? ld_once(src + q * step) : make_float4(0.f, 0.f, 0.f, 0.f);
+      };
+      // first entry of this lane in tile (u, t), and the rows of M from there on
+      auto tile = [&](int u, int t, int64_t* rows) -> const float* {
+        const int64_t row = (int64_t)(b0 + u) * kTileM + w, col = col0 + t * kTileN + 4 * lane;
+        *rows = u < nu && col < p.nR ? p.nL - row : 0;
+        return p.A + row * p.nR + col;
+      };
+      // box row w: rows 16 q on are q * 2 KB further, at the same swizzle
+      const uint32_t dst = (uint32_t)((lane >> 4) * Lay::box + w * 128 +
+                                      ((((lane & 15) >> 1) ^ (w & 7)) << 4) + (lane & 1) * 8);
+      int64_t rows;
+      const float* src = tile(0, 0, &rows);
+#pragma unroll
+      for (int q = 0; q < NQ; ++q) load(q, src, rows);
+      for (int u = 0; u < nu && ok; ++u) {
+        for (int t = 0; t < nt; ++t) {
+          ok = mbar_wait(smem_u32(&bar_empty[stage]), ph ^ 1, &abort_flag);
+          if (!ok) break;
+          src = t + 1 < nt ? tile(u, t + 1, &rows) : tile(u + 1, 0, &rows);
+          const uint32_t o = base + stage * stage_bytes + dst;
+#pragma unroll
+          for (int q = 0; q < NQ; ++q) {
+            split_store(o + q * 2048, v[q]);
+            load(q, src, rows);
+          }
+          fence_proxy_async();   // generic-proxy writes -> visible to the tensor cores
+          __syncwarp();
+          if (lane == 0) mbar_arrive(smem_u32(&bar_conv[stage]));
+          if (++stage == S) {
+            stage = 0;
+            ph ^= 1;
+          }
         }
-        fence_proxy_async();   // generic-proxy writes -> visible to the tensor cores
-        __syncwarp();
-        if (lane == 0) mbar_arrive(smem_u32(&bar_conv[stage]));
-        if (++stage == S) {
-          stage = 0;
-          ph ^= 1;
+      }
+    } else {
+      // the scale of the next tile is loaded while the current one converts
+      auto scale_of = [&](int u, int t) -> float {
+        if (u >= nu) return 1.f;
+        return __ldg(p.scale + (int64_t)(b0 + u) * p.ncolt + (int)(col0 / kTileN) + t);
+      };
+      float s_next = scale_of(0, 0);
+      for (int u = 0; u < nu && ok; ++u) {
+        for (int t = 0; t < nt; ++t) {
+          const float s_cur = s_next;
+          s_next = t + 1 < nt ? scale_of(u, t + 1) : scale_of(u + 1, 0);
+          ok = mbar_wait(smem_u32(&bar_full[stage]), ph, &abort_flag);
+          if (!ok) break;
+          uint8_t* st = smem + stage * stage_bytes;
+          convert_fp8(st + Lay::op, st, s_cur, ct);
+          fence_proxy_async();
+          __syncwarp();
+          if (lane == 0) mbar_arrive(smem_u32(&bar_conv[stage]));
+          if (++stage == S) {
+            stage = 0;
+            ph ^= 1;
+          }
         }
       }
     }
@@ -406,12 +402,15 @@ __global__ void __launch_bounds__(kCvtThreads, 1)
       fence_after();
       const int64_t row = (int64_t)(b0 + u) * kTileM + r_in;
       float* dst = p.C == 1 ? p.D1 + row * p.wRpad
-                            : p.D1p + ((int64_t)c * p.nb * kTileM + row) * p.wRpad;
+                            : d1_partial(p.D1p, p.nb, p.wRpad, c, row - lane) + lane;
       for (int cg = 0; cg < p.wRpad; cg += 16) {
         uint32_t v[16];
         tmem_ld16(tmem + lane_off + d1_col + buf * p.wRpad + cg, v);
         tmem_wait_ld();
-        if (row < p.nL) {
+        if (p.C > 1) {
+#pragma unroll
+          for (int k = 0; k < 16; ++k) dst[(cg + k) * 32] = __uint_as_float(v[k]);
+        } else if (row < p.nL) {
           float4* d4 = reinterpret_cast<float4*>(dst + cg);
 #pragma unroll
           for (int k = 0; k < 4; ++k)
@@ -423,7 +422,7 @@ __global__ void __launch_bounds__(kCvtThreads, 1)
       __syncwarp();
       if (lane == 0) mbar_arrive(smem_u32(&bar_d1empty[buf]));
       if (p.C > 1)
-        fold_d1_rows(&p.cnt[(int64_t)(b0 + u) * 4 + q], p.C, p.D1p, p.D1, p.nb, p.wRpad,
+        fold_d1_rows<1>(&p.cnt[(int64_t)(b0 + u) * 4 + q], p.C, p.D1p, p.D1, p.nb, p.wRpad,
                      (int64_t)(b0 + u) * kTileM + 32 * q, p.nL, p.discard, lane);
     }
     if (!ok) {
@@ -655,10 +654,7 @@ ttnn_status launch_cvt_pass(const ttnn_plan_s& P, const void* A, int64_t nL, int
     return TTNN_EINVAL;
   }
   CUtensorMap mA, mBR, mBL, mBRlo, mBLlo;
-  if (mode == tc::MODE_SPLIT || mode == tc::MODE_SPLIT3)
-    TTNN_TRY(tc::encode_map(&mA, A, CU_TENSOR_MAP_DATA_TYPE_FLOAT32, 4, nR, nL, 64u, 128u,
-                            CU_TENSOR_MAP_SWIZZLE_NONE));
-  else
+  if (mode == tc::MODE_FP8)
     TTNN_TRY(tc::encode_map(&mA, A, CU_TENSOR_MAP_DATA_TYPE_UINT8, 1, nR, nL, 128u, 128u,
                             CU_TENSOR_MAP_SWIZZLE_NONE));
   // SPLIT3: the plan's whole-tensor blocks as bf16 hi and lo halves
@@ -674,6 +670,7 @@ ttnn_status launch_cvt_pass(const ttnn_plan_s& P, const void* A, int64_t nL, int
                           (uint32_t)P.wLpad, CU_TENSOR_MAP_SWIZZLE_128B));
   mBRlo = mBR;
   mBLlo = mBL;
+  if (mode != tc::MODE_FP8) mA = mBR;   // unused: converters load M
   if (mode == tc::MODE_SPLIT3) {
     TTNN_TRY(tc::encode_map(&mBRlo, (const char*)bR + (int64_t)P.wRpad * nR * 2,
                             CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2, nR, P.wRpad, 64u,
@@ -683,6 +680,7 @@ ttnn_status launch_cvt_pass(const ttnn_plan_s& P, const void* A, int64_t nL, int
                             (uint32_t)P.wLpad, CU_TENSOR_MAP_SWIZZLE_128B));
   }
   tc::CvtParams prm;
+  prm.A = (const float*)A;
   prm.nL = nL;
   prm.nR = nR;
   prm.C = g.C;
@@ -701,19 +699,19 @@ ttnn_status launch_cvt_pass(const ttnn_plan_s& P, const void* A, int64_t nL, int
   prm.cnt = g.C > 1 ? (int*)((char*)ws + (g.d1p_elems + g.d2p_elems) * 4 + 256 -
                             (((uintptr_t)ws + (g.d1p_elems + g.d2p_elems) * 4) & 255))
                     : nullptr;
-  prm.discard = (P.wRpad * 4) % 128 == 0 && ((uintptr_t)prm.D1p & 127) == 0;
+  prm.discard = ((uintptr_t)prm.D1p & 127) == 0;
   if (g.C > 1) TTNN_TRY_CUDA(cudaMemsetAsync(prm.cnt, 0, (size_t)g.nb * 16, st));
   if (mode == tc::MODE_SPLIT) {
     TTNN_TRY(tc::smem_limit_once((const void*)tc::pass_cvt_kernel<tc::MODE_SPLIT>, 1));
-    tc::pass_cvt_kernel<tc::MODE_SPLIT><<<g.grid, tc::kCvtThreads, g.smem, st>>>(
+    tc::pass_cvt_kernel<tc::MODE_SPLIT><<<g.grid, 192 + tc::conv_threads<tc::MODE_SPLIT>(), g.smem, st>>>(
         mA, mBR, mBL, mBRlo, mBLlo, prm);
   } else if (mode == tc::MODE_SPLIT3) {
     TTNN_TRY(tc::smem_limit_once((const void*)tc::pass_cvt_kernel<tc::MODE_SPLIT3>, 3));
-    tc::pass_cvt_kernel<tc::MODE_SPLIT3><<<g.grid, tc::kCvtThreads, g.smem, st>>>(
+    tc::pass_cvt_kernel<tc::MODE_SPLIT3><<<g.grid, 192 + tc::conv_threads<tc::MODE_SPLIT3>(), g.smem, st>>>(
         mA, mBR, mBL, mBRlo, mBLlo, prm);
   } else {
     TTNN_TRY(tc::smem_limit_once((const void*)tc::pass_cvt_kernel<tc::MODE_FP8>, 2));
-    tc::pass_cvt_kernel<tc::MODE_FP8><<<g.grid, tc::kCvtThreads, g.smem, st>>>(
+    tc::pass_cvt_kernel<tc::MODE_FP8><<<g.grid, 192 + tc::conv_threads<tc::MODE_FP8>(), g.smem, st>>>(
         mA, mBR, mBL, mBRlo, mBLlo, prm);
   }
   TTNN_TRY(check_launch("tc pass_cvt_kernel"));

@@ -38,11 +38,11 @@ struct Params {
   int wRpad, wLpad;
   int cluster;     // 1: the C chunk CTAs of a row range form a cluster and sum D1 on chip
   float* D1;       // [nL][wRpad] output
-  float* D1p;      // [C][nb*128][wRpad] chunk partials (C > 1, no cluster)
+  float* D1p;      // [C][nb * 4][wRpad][32] chunk partials (C > 1, no cluster)
   float* D2p;      // [G][C*tiles*128][wLpad]
   int* err;
   int* cnt;        // [nb][4] chunk arrivals per row block and epilogue warp (C > 1, no cluster), zero at launch
-  int discard;     // partial rows are whole 128-byte lines: drop them from L2 once summed
+  int discard;     // partials are whole 128-byte lines: drop them from L2 once summed
   uint64_t wait_ns;  // limit of each pipeline wait (drains of own copies keep the 2 s limit)
 };
 
@@ -236,6 +236,8 @@ __global__ void __launch_bounds__(kThreads, 1)
           fence_after();
           const uint32_t sa = base + stage * stage_bytes;
           const uint32_t sbr = sa + a_bytes;
+          // (descriptors by sdesc_at, as in the converting pass, issue faster but
+          // bunch the MMAs against the loads: 64^5 398 us against 389)
 #pragma unroll
           for (int kk = 0; kk < 8; ++kk) {
             const uint64_t da = sdesc(sa + (kk >> 2) * (a_bytes / 2) + (kk & 3) * 32, 16, 1024);
@@ -285,12 +287,15 @@ __global__ void __launch_bounds__(kThreads, 1)
         // that finishes a row block last sums its C partials in chunk order
         // into D1 (deterministic: the order does not depend on who is last)
         float* dst = p.C == 1 ? p.D1 + row * p.wRpad
-                              : p.D1p + ((int64_t)c * p.nb * kTileM + row) * p.wRpad;
+                              : d1_partial(p.D1p, p.nb, p.wRpad, c, row - lane) + lane;
         for (int cg = 0; cg < p.wRpad; cg += 16) {
           uint32_t v[16];
           tmem_ld16(tmem + lane_off + d1_col + buf * p.wRpad + cg, v);
           tmem_wait_ld();
-          if (row < p.nL) {
+          if (p.C > 1) {
+#pragma unroll
+            for (int k = 0; k < 16; ++k) dst[(cg + k) * 32] = __uint_as_float(v[k]);
+          } else if (row < p.nL) {
             float4* d4 = reinterpret_cast<float4*>(dst + cg);
 #pragma unroll
             for (int k = 0; k < 4; ++k)
@@ -302,7 +307,7 @@ __global__ void __launch_bounds__(kThreads, 1)
         __syncwarp();
         if (lane == 0) mbar_arrive(smem_u32(&bar_d1empty[buf]));
         if (p.C > 1)
-          fold_d1_rows(&p.cnt[(int64_t)(b0 + u) * 4 + q], p.C, p.D1p, p.D1, p.nb, p.wRpad,
+          fold_d1_rows<3>(&p.cnt[(int64_t)(b0 + u) * 4 + q], p.C, p.D1p, p.D1, p.nb, p.wRpad,
                        (int64_t)(b0 + u) * kTileM + 32 * q, p.nL, p.discard, lane);
         continue;
       }
@@ -664,7 +669,7 @@ ttnn_status launch_tc_pass(const ttnn_plan_s& P, const void* A, int64_t nL, int6
   prm.cnt = fold ? (int*)((char*)ws + (g.d1p_elems + g.d2p_elems) * 4 + 256 -
                           (((uintptr_t)ws + (g.d1p_elems + g.d2p_elems) * 4) & 255))
                  : nullptr;
-  prm.discard = (P.wRpad * 4) % 128 == 0 && ((uintptr_t)prm.D1p & 127) == 0;
+  prm.discard = ((uintptr_t)prm.D1p & 127) == 0;
   if (fold) TTNN_TRY_CUDA(cudaMemsetAsync(prm.cnt, 0, (size_t)g.nb * 16, st));
   TTNN_TRY(tc::smem_limit_once((const void*)tc::pass_kernel, 0));
   if (g.cluster) {

@@ -85,6 +85,20 @@ __device__ __forceinline__ uint64_t sdesc(uint32_t saddr, uint32_t lbo, uint32_t
   return d;
 }
 
+// The descriptor of the same layout `bytes` (a multiple of 16) further on: one
+// add to its low word.  (Shared memory ends below the address field's 256 KB,
+// so nothing carries out of it.)  The thread that issues the MMAs builds two
+// descriptors per MMA; made from the address each, that alone took longer
+// than the MMA.
+__device__ __forceinline__ uint64_t sdesc_at(uint64_t d, uint32_t bytes) {
+  uint64_t r;
+  asm("{\n\t.reg .b32 lo, hi;\n\tmov.b64 {lo, hi}, %1;\n\tadd.u32 lo, lo, %2;\n\t"
+      "mov.b64 %0, {lo, hi};\n\t}\n"
+      : "=l"(r)
+      : "l"(d), "r"(bytes >> 4));
+  return r;
+}
+
 // Instruction descriptor of kind::f16: D f32, A/B bf16, A K- or MN-major,
 // B K-major, shape M x N.
 __host__ __device__ constexpr uint32_t idesc_bf16(int M, int N, bool a_mn_major) {
@@ -147,13 +161,21 @@ __global__ void reduce_partials(const float* P, int K, int64_t stride_k, int64_t
                                 float* D);
 
 // D1 of a pass split into C column chunks: every chunk CTA writes its partial
-// rows of a row block (D1p = [C][nb*128][wRpad]) and then, per epilogue warp
-// (its 32 rows row0..row0+31), counts its arrival in *slot.  The warp that
-// arrives last sums the C partials in chunk order (the same order as
-// reduce_partials, whoever is last) into D1, with coalesced loads of the 32
-// contiguous rows, and drops the dead partial lines from L2 (`discard`: rows
-// are whole 128-byte lines).  Called by all 32 lanes after their own stores;
-// no thread waits on another.
+// of a row block, each epilogue warp its 32 rows (row0 on) column by column:
+// D1p = [C][nb * 4][wRpad][32], so a store is one whole line of 32 rows.
+// (Row by row, as D1 is laid out, a warp's store touched 32 lines, and the
+// load/store pipe they share with the converter warps cost a 48^5 binary32
+// pass up to 32 of 245 us.)
+__device__ __forceinline__ float* d1_partial(float* D1p, int64_t nb, int wRpad, int c, int64_t row0) {
+  return D1p + ((int64_t)c * nb * kTileM + row0) * wRpad;
+}
+// Then it counts its arrival in *slot.  The warp that arrives last sums the C
+// partials in chunk order (the same order as reduce_partials, whoever is last)
+// into D1, a lane 4 rows by 4 columns at a time, the loads of B partials in
+// flight together, and drops the dead partial lines from L2 (`discard`: D1p is
+// 128-byte aligned).  Called by all 32 lanes after their own stores; no thread
+// waits on another.
+template <int B>
 __device__ __forceinline__ void fold_d1_rows(int* slot, int C, const float* D1p, float* D1,
                                              int64_t nb, int wRpad, int64_t row0, int64_t nL,
                                              int discard, int lane) {
@@ -164,74 +186,48 @@ __device__ __forceinline__ void fold_d1_rows(int* slot, int C, const float* D1p,
   last = __shfl_sync(0xffffffffu, last, 0);
   if (!last) return;
   __threadfence();
-  const int per = wRpad / 4;                       // float4 per row
-  const int64_t cs4 = nb * kTileM * per;           // chunk stride
-  const int64_t lim = (nL - row0) * per;           // valid float4 of the 32 rows
-  const float4* src = reinterpret_cast<const float4*>(D1p) + row0 * per;
-  float4* out = reinterpret_cast<float4*>(D1) + row0 * per;
-  const int n4 = 32 * per;
-  if (C <= 4) {
-    // every partial's loads of a batch in flight at once (one L2 round trip
-    // per batch instead of one per partial), then the sums in chunk order
-    for (int e0 = lane; e0 < n4; e0 += 128) {
-      float4 v[4][4];
+  const int i = lane & 7, j = lane >> 3;           // rows 4 i on, columns 4 j on (of 16)
+  const int64_t cs = nb * kTileM * wRpad;          // chunk stride
+  const float* src = D1p + row0 * wRpad;
+  for (int cg = 0; cg < wRpad; cg += 16) {
+    const float4* s4 = reinterpret_cast<const float4*>(src + (cg + 4 * j) * 32 + 4 * i);
+    float4 acc[4];   // column 4 j + m: rows 4 i .. 4 i + 3
 #pragma unroll
-      for (int cc = 0; cc < 4; ++cc)
+    for (int m = 0; m < 4; ++m) acc[m] = __ldcg(s4 + m * 8);
+    for (int c0 = 1; c0 < C; c0 += B) {
+      float4 v[B][4];
 #pragma unroll
-        for (int j = 0; j < 4; ++j) {
-          const int e = e0 + 32 * j;
-          v[cc][j] = (cc < C && e < n4) ? __ldcg(src + cc * cs4 + e) : make_float4(0.f, 0.f, 0.f, 0.f);
+      for (int b = 0; b < B; ++b)
+#pragma unroll
+        for (int m = 0; m < 4; ++m)
+          if (c0 + b < C) v[b][m] = __ldcg(s4 + (c0 + b) * (cs / 4) + m * 8);
+#pragma unroll
+      for (int b = 0; b < B; ++b) {
+        if (c0 + b >= C) break;
+#pragma unroll
+        for (int m = 0; m < 4; ++m) {
+          acc[m].x += v[b][m].x;
+          acc[m].y += v[b][m].y;
+          acc[m].z += v[b][m].z;
+          acc[m].w += v[b][m].w;
         }
-#pragma unroll
-      for (int j = 0; j < 4; ++j) {
-        float4 acc = v[0][j];
-#pragma unroll
-        for (int cc = 1; cc < 4; ++cc) {
-          if (cc >= C) break;
-          acc.x += v[cc][j].x;
-          acc.y += v[cc][j].y;
-          acc.z += v[cc][j].z;
-          acc.w += v[cc][j].w;
-        }
-        const int e = e0 + 32 * j;
-        if (e < n4 && e < lim) out[e] = acc;
       }
     }
-  }
-  for (int e0 = lane; C > 4 && e0 < n4; e0 += 128) {
-    float4 acc[4];
-#pragma unroll
-    for (int j = 0; j < 4; ++j) {
-      const int e = e0 + 32 * j;
-      acc[j] = e < n4 ? __ldcg(src + e) : make_float4(0.f, 0.f, 0.f, 0.f);
-    }
-    for (int cc = 1; cc < C; ++cc) {
-      float4 v[4];
-#pragma unroll
-      for (int j = 0; j < 4; ++j) {
-        const int e = e0 + 32 * j;
-        v[j] = e < n4 ? __ldcg(src + cc * cs4 + e) : make_float4(0.f, 0.f, 0.f, 0.f);
-      }
-#pragma unroll
-      for (int j = 0; j < 4; ++j) {
-        acc[j].x += v[j].x;
-        acc[j].y += v[j].y;
-        acc[j].z += v[j].z;
-        acc[j].w += v[j].w;
-      }
-    }
-#pragma unroll
-    for (int j = 0; j < 4; ++j) {
-      const int e = e0 + 32 * j;
-      if (e < n4 && e < lim) out[e] = acc[j];
-    }
+    const int64_t row = row0 + 4 * i;
+    float* out = D1 + row * wRpad + cg + 4 * j;
+    if (row < nL) *reinterpret_cast<float4*>(out) = make_float4(acc[0].x, acc[1].x, acc[2].x, acc[3].x);
+    if (row + 1 < nL)
+      *reinterpret_cast<float4*>(out + wRpad) = make_float4(acc[0].y, acc[1].y, acc[2].y, acc[3].y);
+    if (row + 2 < nL)
+      *reinterpret_cast<float4*>(out + 2 * wRpad) = make_float4(acc[0].z, acc[1].z, acc[2].z, acc[3].z);
+    if (row + 3 < nL)
+      *reinterpret_cast<float4*>(out + 3 * wRpad) = make_float4(acc[0].w, acc[1].w, acc[2].w, acc[3].w);
   }
   if (discard) {
-    const int lines = 32 * wRpad * 4 / 128;
+    __syncwarp();
     for (int cc = 0; cc < C; ++cc)
-      for (int l = lane; l < lines; l += 32)
-        asm volatile("discard.global.L2 [%0], 128;" ::"l"((const char*)(src + cc * cs4) +
-                                                            (int64_t)l * 128)
+      for (int l = lane; l < wRpad; l += 32)
+        asm volatile("discard.global.L2 [%0], 128;" ::"l"((const char*)(src + cc * cs) + (int64_t)l * 128)
                      : "memory");
   }
 }
