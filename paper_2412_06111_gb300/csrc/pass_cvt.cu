@@ -716,11 +716,8 @@ ttnn_status launch_cvt_pass(const ttnn_plan_s& P, const void* A, int64_t nL, int
   }
   TTNN_TRY(check_launch("tc pass_cvt_kernel"));
   if (P.prof_kernel_end) cudaEventRecord(P.prof_kernel_end, st);
-  const int sms = tc::sm_count();
-  tc::reduce_partials<<<sms * 4, 256, 0, st>>>(prm.D2p, g.G, (int64_t)g.C * g.tiles * tc::kTileN * P.wLpad,
-                                               nR, P.wLpad, (float*)D2);
-  TTNN_TRY(check_launch("reduce_partials(D2)"));
-  return TTNN_OK;
+  return tc::launch_reduce_partials(prm.D2p, g.G, (int64_t)g.C * g.tiles * tc::kTileN * P.wLpad, nR,
+                                    P.wLpad, (float*)D2, st);
 }
 
 }  // namespace ttnn

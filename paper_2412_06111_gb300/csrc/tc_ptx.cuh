@@ -157,8 +157,8 @@ int sm_count();
 // quarter), which stay free for a recovery running on another stream.
 int pass_sms(const ttnn_plan_s& P);
 // D[i][w] = sum_k P[k][i][w] for w < wpad (rows i < rows).
-__global__ void reduce_partials(const float* P, int K, int64_t stride_k, int64_t rows, int wpad,
-                                float* D);
+ttnn_status launch_reduce_partials(const float* P, int K, int64_t stride_k, int64_t rows, int wpad,
+                                   float* D, cudaStream_t st);
 
 // D1 of a pass split into C column chunks: every chunk CTA writes its partial
 // of a row block, each epilogue warp its 32 rows (row0 on) column by column:
@@ -170,11 +170,10 @@ __device__ __forceinline__ float* d1_partial(float* D1p, int64_t nb, int wRpad, 
   return D1p + ((int64_t)c * nb * kTileM + row0) * wRpad;
 }
 // Then it counts its arrival in *slot.  The warp that arrives last sums the C
-// partials in chunk order (the same order as reduce_partials, whoever is last)
-// into D1, a lane 4 rows by 4 columns at a time, the loads of B partials in
-// flight together, and drops the dead partial lines from L2 (`discard`: D1p is
-// 128-byte aligned).  Called by all 32 lanes after their own stores; no thread
-// waits on another.
+// partials in chunk order (whoever is last) into D1, a lane 4 rows by 4 columns
+// at a time, the loads of B partials in flight together, and drops the dead
+// partial lines from L2 (`discard`: D1p is 128-byte aligned).  Called by all 32
+// lanes after their own stores; no thread waits on another.
 template <int B>
 __device__ __forceinline__ void fold_d1_rows(int* slot, int C, const float* D1p, float* D1,
                                              int64_t nb, int wRpad, int64_t row0, int64_t nL,
