@@ -1131,6 +1131,7 @@ static ttnn_status launch_ops(LaunchGroup g, const std::vector<const Op*>& ops, 
   for (size_t k = 0; k < ops.size(); k += kLargeOps) {
     const int n = (int)std::min<size_t>(ops.size() - k, kLargeOps);
     TTNN_TRY(n <= kSmallOps ? launch_group<kSmallOps>(g, ops.data() + k, n, st)
+             : n <= kMidOps ? launch_group<kMidOps>(g, ops.data() + k, n, st)
                             : launch_group<kLargeOps>(g, ops.data() + k, n, st));
   }
   return TTNN_OK;

@@ -94,8 +94,11 @@ struct CpOp {
 // The ops of one launch.  Most levels hold a few ops: they travel in a small
 // batch (about 4 KB of kernel parameters); a launch with the large one costs
 // 1 us more on the host and 2 to 3 us more on the device (measured with a
-// 31 KB batch against 4 KB).
+// 31 KB batch against 4 KB).  The middle one is for the first levels of a
+// walk: with it a pass of 8 small streaming updates keeps the host busy for
+// 480 us instead of 532, and a 64^5 update takes 521 us instead of 527.
 constexpr int kSmallOps = 8;
+constexpr int kMidOps = 20;
 constexpr int kLargeOps = 48;
 
 template <typename OpT, int CAP>
@@ -118,6 +121,7 @@ struct TcOp {
 
 class Program {
  public:
+  Program() { ops_.reserve(64); }   // a walk's ops: growing by moves took 6 % of a small update's host time
   // Registers a buffer written by the program (or produced before it, level 0).
   void buffer(const void* p, int64_t bytes, int level = 0);
   // Records an op; its level follows the buffers it reads.
