@@ -25,6 +25,11 @@ static int num_sms() {
 }
 
 static std::atomic<long long> g_launches{0};
+bool& pdl_of_thread() {
+  thread_local bool on = true;
+  return on;
+}
+
 void count_launch() { g_launches.fetch_add(1, std::memory_order_relaxed); }
 long long launches_so_far() { return g_launches.load(); }
 
@@ -81,6 +86,7 @@ ttnn_status launch_convert_f64_to_f32(const double* src, float* dst, int64_t n, 
 constexpr int kConvBlock = 2048;
 
 __global__ void convert_batch_kernel(const __grid_constant__ ConvertBatch b) {
+  pdl_begin();
   int lo = 0, hi = b.count - 1;
   while (lo < hi) {
     const int mid = (lo + hi + 1) / 2;
@@ -124,7 +130,7 @@ ttnn_status launch_convert_batch(const ConvertBatch& batch, cudaStream_t st) {
     set_error("conversion batch too large");
     return TTNN_EUNSUPPORTED;
   }
-  convert_batch_kernel<<<(unsigned)blocks, 256, 0, st>>>(b);
+  launch_pdl(convert_batch_kernel, (unsigned)blocks, 256, 0, st, b);
   return check_launch("convert_batch_kernel");
 }
 
@@ -150,6 +156,7 @@ __device__ __forceinline__ void store_fmt(void* out, int64_t idx, double v, int 
 }
 
 __global__ void side_kernel(SideSpec s, void* out) {
+  pdl_begin();
   int64_t rows = 1;
   for (int m = 0; m < s.nmodes; ++m) rows *= s.ext[m];
   const int64_t n = rows * s.total_cols;
@@ -185,6 +192,7 @@ __global__ void side_kernel(SideSpec s, void* out) {
 
 template <typename T>
 __global__ void side_gather_kernel(SideSpec s, const T* src, int64_t src_ld, T* out) {
+  pdl_begin();
   int64_t rows = 1;
   for (int m = 0; m < s.nmodes; ++m) rows *= s.ext[m];
   const int64_t n = rows * s.total_cols;
@@ -211,19 +219,19 @@ ttnn_status launch_side_gather(const SideSpec& s, const void* src, int64_t src_l
   const int64_t blocks = std::min<int64_t>(ceil_div(n, 256), 65535);
   switch (s.store) {
     case 0:
-      side_gather_kernel<uint64_t><<<(unsigned)blocks, 256, 0, st>>>(s, (const uint64_t*)src, src_ld,
+      launch_pdl(side_gather_kernel<uint64_t>, (unsigned)blocks, 256, 0, st, s, (const uint64_t*)src, src_ld,
                                                                      (uint64_t*)out);
       break;
     case 1:
-      side_gather_kernel<uint32_t><<<(unsigned)blocks, 256, 0, st>>>(s, (const uint32_t*)src, src_ld,
+      launch_pdl(side_gather_kernel<uint32_t>, (unsigned)blocks, 256, 0, st, s, (const uint32_t*)src, src_ld,
                                                                      (uint32_t*)out);
       break;
     case 2:
-      side_gather_kernel<uint16_t><<<(unsigned)blocks, 256, 0, st>>>(s, (const uint16_t*)src, src_ld,
+      launch_pdl(side_gather_kernel<uint16_t>, (unsigned)blocks, 256, 0, st, s, (const uint16_t*)src, src_ld,
                                                                      (uint16_t*)out);
       break;
     default:
-      side_gather_kernel<uint8_t><<<(unsigned)blocks, 256, 0, st>>>(s, (const uint8_t*)src, src_ld,
+      launch_pdl(side_gather_kernel<uint8_t>, (unsigned)blocks, 256, 0, st, s, (const uint8_t*)src, src_ld,
                                                                     (uint8_t*)out);
       break;
   }
@@ -255,6 +263,7 @@ __device__ void gather_rows(const GatherJob& g, int64_t e) {
 }
 
 __global__ void side_gather_batch_kernel(const __grid_constant__ GatherBatch b) {
+  pdl_begin();
   const int64_t blk = blockIdx.x;
   int lo = 0, hi = b.n - 1;
   while (lo < hi) {
@@ -291,7 +300,7 @@ ttnn_status launch_side_gather_batch(const GatherJob* jobs, int n, cudaStream_t 
       set_error("side gather batch too large");
       return TTNN_EUNSUPPORTED;
     }
-    side_gather_batch_kernel<<<(unsigned)b.start[b.n], 256, 0, st>>>(b);
+    launch_pdl(side_gather_batch_kernel, (unsigned)b.start[b.n], 256, 0, st, b);
     TTNN_TRY(check_launch("side_gather_batch_kernel"));
   }
   return TTNN_OK;
@@ -346,6 +355,7 @@ __global__ void __launch_bounds__(256) side_gemv_kernel(const __grid_constant__ 
                                                         int64_t rpb, Tacc* part,
                                                         const float* scale, Tacc* mcopy,
                                                         const Ts* brow, Tacc* bcopy, int bcols) {
+  pdl_begin();
   __shared__ Tacc red[8][kGemvCols];
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int64_t r0 = (int64_t)blockIdx.x * rpb;
@@ -408,6 +418,7 @@ __global__ void __launch_bounds__(256) side_gemv_kernel(const __grid_constant__ 
 template <typename Tacc>
 __global__ void __launch_bounds__(256) gemv_reduce_kernel(const Tacc* part, int nblk, int cols,
                                                           int cols_pad, Tacc* D) {
+  pdl_begin();
   const int lane = threadIdx.x & 31;
   const int c = blockIdx.x * 8 + (threadIdx.x >> 5);
   if (c >= cols_pad) return;
@@ -447,23 +458,23 @@ ttnn_status launch_side_gemv(const SideSpec& s, const void* src, int64_t src_ld,
     const dim3 grid((unsigned)nblk, (unsigned)std::max<int64_t>(1, ceil_div(cols, kGemvCols)), 1);
     const int ct = cut ? 1 : 0;
     if (d_f64 && m_store == 0 && s.store == 0)
-      side_gemv_kernel<double, double, double><<<grid, 256, 0, st>>>(
+      launch_pdl(side_gemv_kernel<double, double, double>, grid, 256, 0, st,
           s, (const double*)src, src_ld, ct, (const double*)m, rows, cols, rpb, (double*)part,
           scale, (double*)mcopy, (const double*)brow, (double*)bcopy, bcols);
     else if (!d_f64 && m_store == 1 && s.store == 1)
-      side_gemv_kernel<float, float, float><<<grid, 256, 0, st>>>(
+      launch_pdl(side_gemv_kernel<float, float, float>, grid, 256, 0, st,
           s, (const float*)src, src_ld, ct, (const float*)m, rows, cols, rpb, (float*)part, scale,
           (float*)mcopy, (const float*)brow, (float*)bcopy, bcols);
     else if (!d_f64 && m_store == 2 && s.store == 2)
-      side_gemv_kernel<uint16_t, uint16_t, float><<<grid, 256, 0, st>>>(
+      launch_pdl(side_gemv_kernel<uint16_t, uint16_t, float>, grid, 256, 0, st,
           s, (const uint16_t*)src, src_ld, ct, (const uint16_t*)m, rows, cols, rpb, (float*)part,
           scale, (float*)mcopy, (const uint16_t*)brow, (float*)bcopy, bcols);
     else if (!d_f64 && m_store == kStoreSplit && s.store == 2)
-      side_gemv_kernel<float, uint16_t, float, RV_SPLIT><<<grid, 256, 0, st>>>(
+      launch_pdl(side_gemv_kernel<float, uint16_t, float, RV_SPLIT>, grid, 256, 0, st,
           s, (const uint16_t*)src, src_ld, ct, (const float*)m, rows, cols, rpb, (float*)part,
           scale, (float*)mcopy, (const uint16_t*)brow, (float*)bcopy, bcols);
     else if (!d_f64 && m_store == kStoreFp8 && s.store == 2 && scale)
-      side_gemv_kernel<uint8_t, uint16_t, float, RV_FP8><<<grid, 256, 0, st>>>(
+      launch_pdl(side_gemv_kernel<uint8_t, uint16_t, float, RV_FP8>, grid, 256, 0, st,
           s, (const uint16_t*)src, src_ld, ct, (const uint8_t*)m, rows, cols, rpb, (float*)part,
           scale, (float*)mcopy, (const uint16_t*)brow, (float*)bcopy, bcols);
     else {
@@ -474,8 +485,12 @@ ttnn_status launch_side_gemv(const SideSpec& s, const void* src, int64_t src_ld,
   }
   if (cols_pad == 0) return TTNN_OK;
   const unsigned rb = (unsigned)ceil_div(cols_pad, 8);
-  if (d_f64) gemv_reduce_kernel<double><<<rb, 256, 0, st>>>((const double*)part, (int)nblk, cols, cols_pad, (double*)D);
-  else gemv_reduce_kernel<float><<<rb, 256, 0, st>>>((const float*)part, (int)nblk, cols, cols_pad, (float*)D);
+  if (d_f64)
+    launch_pdl(gemv_reduce_kernel<double>, rb, 256, 0, st, (const double*)part, (int)nblk, cols, cols_pad,
+               (double*)D);
+  else
+    launch_pdl(gemv_reduce_kernel<float>, rb, 256, 0, st, (const float*)part, (int)nblk, cols, cols_pad,
+               (float*)D);
   return check_launch("gemv_reduce_kernel");
 }
 
@@ -485,7 +500,7 @@ ttnn_status launch_side(const SideSpec& s, void* out, cudaStream_t st) {
   const int64_t n = rows * s.total_cols;
   if (n == 0) return TTNN_OK;
   const int64_t blocks = std::min<int64_t>(ceil_div(n, 256), 65535);
-  side_kernel<<<(unsigned)blocks, 256, 0, st>>>(s, out);
+  launch_pdl(side_kernel, (unsigned)blocks, 256, 0, st, s, out);
   return check_launch("side_kernel");
 }
 

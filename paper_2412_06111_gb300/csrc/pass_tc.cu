@@ -438,6 +438,7 @@ __global__ void __launch_bounds__(kThreads, 1)
 __global__ void __launch_bounds__(256)
     reduce_partials(const float* P, int K, int64_t stride_k, int64_t rows, int wpad, float* D) {
   __shared__ float4 part[8][32];
+  pdl_begin();
   const int lane = threadIdx.x & 31, s = threadIdx.x >> 5;
   const int64_t n4 = rows * wpad / 4;
   const int k0 = K * s / 8, k1 = K * (s + 1) / 8;
@@ -476,7 +477,7 @@ __global__ void __launch_bounds__(256)
 ttnn_status launch_reduce_partials(const float* P, int K, int64_t stride_k, int64_t rows, int wpad,
                                    float* D, cudaStream_t st) {
   const int64_t blocks = std::min<int64_t>((rows * wpad / 4 + 31) / 32, (int64_t)sm_count() * 16);
-  reduce_partials<<<(unsigned)blocks, 256, 0, st>>>(P, K, stride_k, rows, wpad, D);
+  launch_pdl(reduce_partials, (unsigned)blocks, 256, 0, st, P, K, stride_k, rows, wpad, D);
   return check_launch("reduce_partials(D2)");
 }
 

@@ -763,6 +763,7 @@ template <bool F64, typename I, int CAP>
 __global__ void __launch_bounds__(kExecThreads, 3)
     level_kernel(const __grid_constant__ LevelBatch<WalkOp, CAP> lb) {
   extern __shared__ __align__(16) unsigned char dsm[];
+  pdl_begin();
   int64_t blk;
   const int k = op_of_block(lb, (int)blockIdx.x, &blk);
   dispatch<F64, I>(lb.ops[k], blk, dsm);
@@ -772,6 +773,7 @@ __global__ void __launch_bounds__(kExecThreads, 3)
 template <int CAP>
 __global__ void __launch_bounds__(kExecThreads)
     cp_level_kernel(const __grid_constant__ LevelBatch<CpOp, CAP> lb) {
+  pdl_begin();
   int64_t blk;
   const CpOp& op = lb.ops[op_of_block(lb, (int)blockIdx.x, &blk)];
   if (op.kind == OP_PROJ) dev_proj(op.pj, blk);
@@ -787,6 +789,7 @@ template <int MINB, int CAP>
 __global__ void __launch_bounds__(kExecThreads, MINB)
     kgemm_level_kernel(const __grid_constant__ LevelBatch<WalkOp, CAP> lb) {
   extern __shared__ __align__(16) unsigned char dsm[];
+  pdl_begin();
   int64_t blk;
   const int k = op_of_block(lb, (int)blockIdx.x, &blk);
   // one instantiation (64-bit column decoding: a few divisions per thread)
@@ -1097,7 +1100,7 @@ static ttnn_status launch_group(LaunchGroup g, const Op* const* ops, int n, cuda
   if (g == LG_CP) {
     LevelBatch<CpOp, CAP> b;
     if ((blocks = fill_batch(b, ops, n)) > 0)
-      cp_level_kernel<CAP><<<(unsigned)blocks, kExecThreads, 0, st>>>(b);
+      launch_pdl(cp_level_kernel<CAP>, (unsigned)blocks, kExecThreads, 0, st, b);
   } else {
     LevelBatch<WalkOp, CAP> b;
     blocks = fill_batch(b, ops, n);
@@ -1106,17 +1109,17 @@ static ttnn_status launch_group(LaunchGroup g, const Op* const* ops, int n, cuda
     } else if (g == LG_KGEMM) {
       // at least three full waves at three blocks per SM: the 80-register form
       if (blocks >= 9 * (int64_t)exec_sms())
-        kgemm_level_kernel<3, CAP><<<gr, kExecThreads, kKgemmSmem, st>>>(b);
+        launch_pdl(kgemm_level_kernel<3, CAP>, gr, kExecThreads, kKgemmSmem, st, b);
       else
-        kgemm_level_kernel<2, CAP><<<gr, kExecThreads, kKgemmSmem, st>>>(b);
+        launch_pdl(kgemm_level_kernel<2, CAP>, gr, kExecThreads, kKgemmSmem, st, b);
     } else if (g == LG_F32) {
-      level_kernel<false, uint32_t, CAP><<<gr, kExecThreads, kExecSmem, st>>>(b);
+      launch_pdl(level_kernel<false, uint32_t, CAP>, gr, kExecThreads, kExecSmem, st, b);
     } else if (g == LG_F32_WIDE) {
-      level_kernel<false, int64_t, CAP><<<gr, kExecThreads, kExecSmem, st>>>(b);
+      launch_pdl(level_kernel<false, int64_t, CAP>, gr, kExecThreads, kExecSmem, st, b);
     } else if (g == LG_F64) {
-      level_kernel<true, uint32_t, CAP><<<gr, kExecThreads, kLaneSmem, st>>>(b);
+      launch_pdl(level_kernel<true, uint32_t, CAP>, gr, kExecThreads, kLaneSmem, st, b);
     } else {
-      level_kernel<true, int64_t, CAP><<<gr, kExecThreads, kLaneSmem, st>>>(b);
+      launch_pdl(level_kernel<true, int64_t, CAP>, gr, kExecThreads, kLaneSmem, st, b);
     }
   }
   if (blocks < 0) {

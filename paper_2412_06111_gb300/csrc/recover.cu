@@ -88,6 +88,7 @@ __global__ void __launch_bounds__(kQrMaxThreads) qr_pinv_kernel(const QrJob* job
                                                              double eps_factor, double u,
                                                              int* kept, int trunc) {
   extern __shared__ double sm[];
+  pdl_begin();
   const QrJob job = jobs[blockIdx.x];
   const int s = job.s, r = job.r;
   double* A = sm;                         // A[j * s + i]
@@ -451,8 +452,7 @@ ttnn_status launch_qr_pinv(const QrJob* jobs_dev, int njobs, int rmax, int state
   TTNN_TRY_CUDA(cudaFuncSetAttribute(qr_pinv_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                      (int)smem));
   const int warps = std::min(kQrMaxWarps, std::max(8, (rmax + 1) / 2));
-  qr_pinv_kernel<<<njobs, warps * 32, smem, st>>>(jobs_dev, state_f64, eps_factor, u, kept_dev,
-                                                  trunc);
+  launch_pdl(qr_pinv_kernel, njobs, warps * 32, smem, st, jobs_dev, state_f64, eps_factor, u, kept_dev, trunc);
   return check_launch("qr_pinv_kernel");
 }
 

@@ -170,6 +170,7 @@ bool retire(ttnn_server_s* S, std::deque<InFlight>& q, std::vector<cudaEvent_t>&
 
 void worker_main(ttnn_server_s* S, int k) {
   cudaSetDevice(S->device);
+  pdl_of_thread() = false;
   Worker& W = S->workers[k];
   std::deque<InFlight> inflight;
   std::vector<cudaEvent_t> pool;
