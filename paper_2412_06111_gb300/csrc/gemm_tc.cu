@@ -700,7 +700,7 @@ static ttnn_status tcg_batch(const TcGemm* const* g, int n, void* pieces, int sm
     q.tile0 = p.tiles;
     // Chain of leading products per drain: 8 MMAs (128 k).  Long binary32
     // reductions take 16: their sums err less than the SIMT GEMM's by more
-    // than the longer chain adds (64^4 x 8 slab: 4.2e-7 against 9.8e-7; short
+    // than the longer chain adds (64^4 x 8 slab: 2.0e-7 against 6.5e-7; short
     // ones would lose that margin), and the drains cost 10 % of the time.
     q.chain = g[k]->chain ? g[k]->chain : f.type != 2 && g[k]->K >= 2048 ? 16 : 8;
     p.tiles += (int)nI;
