@@ -46,13 +46,16 @@ void count_launch();
 // in an update or a recovery: a kernel's blocks may be placed while the kernel
 // before it in the stream still runs, and wait for its end (and the visibility
 // of its writes) before they do anything.  Every kernel launched by launch_pdl
-// begins with pdl_begin(), so the end of a kernel still implies the end of all
+// begins with pdl_begin() or pdl_wait(), so the end of a kernel still implies the end of all
 // before it; any other kernel, copy or event after it sees ordinary stream
 // order.  8 small streaming updates 557 -> 490 us, 64^5 bfloat16 531 -> 512,
 // 24^4 binary64 to cores 128 -> 120.
+// (pdl_wait() alone in a long kernel: the blocks after it would hold room that
+// another stream's kernels could use.)
+__device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 __device__ __forceinline__ void pdl_begin() {
   asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
-  asm volatile("griddepcontrol.wait;" ::: "memory");
+  pdl_wait();
 }
 // Whether this thread's launches are programmatic.  Not those of the server's
 // workers: their streams share the chip, and blocks placed early hold room that
