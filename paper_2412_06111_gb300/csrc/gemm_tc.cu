@@ -48,6 +48,7 @@ struct TcgProb {
   const void* A;
   int64_t lda, I, K;
   float* C;
+  const int32_t* shift;  // TcGemm::shift, or null
   int64_t ldc, unit0;    // first (row tile, k tile) of the product in the launch
   int nkt, tile0;        // k tiles, first row tile in the launch
   int chain;             // MMAs (of 16 k) per drain of the accumulators: 2 (not bfloat16), 4, 8 or 16
@@ -63,6 +64,11 @@ struct TcgParams {
   TcgProb prob[kTcgBatch];
 };
 static_assert(sizeof(TcgParams) <= 4096, "a launch's products travel in the kernel parameters");
+
+// x 2^e for |e| < 252 (one rounding more where the result is subnormal).
+__device__ __forceinline__ float scale2(float x, int e) {
+  return x * __int_as_float((127 + e / 2) << 23) * __int_as_float((127 + e - e / 2) << 23);
+}
 
 // The product of row tile `it` of the launch.
 __device__ __forceinline__ int tcg_prob(const TcgParams& p, int it) {
@@ -508,6 +514,14 @@ __global__ void __launch_bounds__(tcg_threads<EPI>(), 1)
         if (buf == 0) fph ^= 1;
       }
       if (!ok) break;
+      if (b.shift) {
+#pragma unroll
+        for (int c = 0; c < NW; ++c) {
+          if (c >= cn) continue;
+          const int e = __ldg(b.shift + 2 * (cb + c)) + __ldg(b.shift + 2 * (cb + c) + 1);
+          if (e) acc[c] = scale2(acc[c], e);
+        }
+      }
       const bool whole = kt0 == 0 && kt1 == b.nkt;
       const int64_t row = (int64_t)(it - b.tile0) * kTileM + 32 * q + lane;
       if (row < b.I && whole && b.trans) {
@@ -545,6 +559,7 @@ __global__ void __launch_bounds__(tcg_threads<EPI>(), 1)
 struct PrepJob {
   TcCols c[2];
   uint16_t* dst;
+  int32_t* shift;
   int64_t K, Kpad;
   int nb, Npad, bf16, start;   // start: first block
 };
@@ -554,8 +569,50 @@ struct PrepBatch {
 };
 constexpr int kPrepRows = 8;   // rows of a thread
 
-__device__ __forceinline__ float prep_value(const TcCols& c, int64_t j, int64_t k) {
+// The powers of two that column j of a Khatri-Rao operand loses.  Its factors
+// are sketches and environments of a network, of any size: their product may
+// leave binary32 although its sum against the core is representable.  The
+// largest magnitudes of the factors, 2^e0 and 2^e1 (not above e0 + 1, e1 + 1),
+// are brought to 2^32 (2^-32) each if e0 + e1 > 64 (< -64), else left alone:
+// what then over- or underflows in the sum against binary32 entries does so in
+// the result.  Blocks: a column (x) of a job (y).
+__global__ void __launch_bounds__(256) tcg_range_kernel(const __grid_constant__ PrepBatch b) {
+  const PrepJob& j = b.job[blockIdx.y];
+  const TcCols& c = j.c[0];
+  const int col = blockIdx.x, warp = threadIdx.x >> 5;
+  if (!j.shift || col >= j.Npad) return;
+  __shared__ uint32_t big[2][8];
+#pragma unroll
+  for (int f = 0; f < 2; ++f) {
+    uint32_t m = 0u;
+    if (col < c.n)
+      for (int64_t i = threadIdx.x; i < c.krn[f]; i += 256)
+        m = max(m, __float_as_uint(c.kr[f][i * c.ki[f] + col * c.kj[f]]) & 0x7FFFFFFFu);
+    m = __reduce_max_sync(0xffffffffu, m);
+    if ((threadIdx.x & 31) == 0) big[f][warp] = m;
+  }
+  __syncthreads();
+  if (threadIdx.x != 0) return;
+  int e[2];
+  for (int f = 0; f < 2; ++f) {
+    uint32_t m = 0u;
+    for (int w = 0; w < 8; ++w) m = max(m, big[f][w]);
+    // (subnormal: not above 2^(e + 1); 0: any; not finite: 128)
+    e[f] = m < 0x00800000u ? m ? -118 - __clz(m) : 0 : (int)(m >> 23) - 127;
+  }
+  const int to = e[0] + e[1] > 64 ? 32 : -32;
+  const bool off = e[0] + e[1] > 64 || e[0] + e[1] < -64;
+  j.shift[2 * col] = off ? e[0] - to : 0;
+  j.shift[2 * col + 1] = off ? e[1] - to : 0;
+}
+
+__device__ __forceinline__ float prep_value(const TcCols& c, const int32_t* shift, int64_t j, int64_t k) {
   if (c.nkr == 0) return ((const float*)c.p)[j * c.sj + k * c.sk];
+  if (shift && (shift[2 * j] | shift[2 * j + 1])) {
+    const uint32_t d0 = (uint32_t)k / (uint32_t)c.krn[1], d1 = (uint32_t)k - d0 * (uint32_t)c.krn[1];
+    return scale2(c.kr[0][(int64_t)d0 * c.ki[0] + j * c.kj[0]], -shift[2 * j]) *
+           scale2(c.kr[1][(int64_t)d1 * c.ki[1] + j * c.kj[1]], -shift[2 * j + 1]);
+  }
   float v = 1.f;
   uint32_t rem = (uint32_t)k;
 #pragma unroll
@@ -591,7 +648,7 @@ __global__ void __launch_bounds__(256) tcg_prepare_kernel(const __grid_constant_
       *out = (in ? (uint32_t)s[0] : 0u) | ((in1 ? (uint32_t)s[c.sk] : 0u) << 16);
     } else {
       uint32_t w[3];
-      cut3(in ? prep_value(c, row, k) : 0.f, in1 ? prep_value(c, row, k + 1) : 0.f, w);
+      cut3(in ? prep_value(c, j.shift, row, k) : 0.f, in1 ? prep_value(c, j.shift, row, k + 1) : 0.f, w);
 #pragma unroll
       for (int q = 0; q < 3; ++q) out[q * pairs] = w[q];
     }
@@ -694,6 +751,7 @@ static ttnn_status tcg_batch(const TcGemm* const* g, int n, void* pieces, int sm
     q.I = g[k]->I;
     q.K = g[k]->K;
     q.C = (float*)g[k]->C;
+    q.shift = g[k]->shift;
     q.ldc = g[k]->ldc;
     q.trans = g[k]->trans;
     q.unit0 = p.units;
@@ -733,6 +791,7 @@ bool tcg_supported(const TcGemm& g) {
   const int64_t lim = int64_t(1) << 31;
   if (g.type < 1 || g.type > 3 || g.I < 1 || g.Jn < 1 || g.K < 1) return false;
   if (g.Jn > tc::kTcgMaxN) return false;
+  if (g.shift && (g.nb != 1 || g.b[0].nkr != 2)) return false;
   // float4 rows of C
   if (!g.trans && (g.ldc < round_up(g.Jn, 16) || g.ldc % 4)) return false;
   // 32-bit tile counts (of kTcgBatch products) and TMA coordinates
@@ -755,6 +814,7 @@ ttnn_status tcg_prepare(const TcGemm* g, int n, void* const* dst, cudaStream_t s
     PrepBatch pb;
     pb.n = std::min(n - k0, kTcgBatch);
     int64_t blocks = 0;
+    int ranged = 0;   // columns of the widest operand that tcg_range_kernel looks over
     for (int k = 0; k < pb.n; ++k) {
       const TcGemm& m = g[k0 + k];
       PrepJob& j = pb.job[k];
@@ -766,12 +826,18 @@ ttnn_status tcg_prepare(const TcGemm* g, int n, void* const* dst, cudaStream_t s
       j.Kpad = round_up(m.K, (int64_t)tcg_kt(m));
       j.Npad = tcg_npad(m);
       j.bf16 = m.type == 2;
+      j.shift = m.shift;
+      if (m.shift) ranged = std::max(ranged, j.Npad);
       j.start = (int)blocks;
       blocks += ceil_div(j.Kpad / 2, (int64_t)256) * (j.Npad / kPrepRows);
       if (blocks >= (int64_t(1) << 31)) {
         set_error("tensor-core GEMM: operand too large");
         return TTNN_EUNSUPPORTED;
       }
+    }
+    if (ranged) {
+      tcg_range_kernel<<<dim3((unsigned)ranged, (unsigned)pb.n), 256, 0, st>>>(pb);
+      TTNN_TRY(check_launch("tcg_range_kernel"));
     }
     tcg_prepare_kernel<<<(unsigned)blocks, 256, 0, st>>>(pb);
     TTNN_TRY(check_launch("tcg_prepare_kernel"));

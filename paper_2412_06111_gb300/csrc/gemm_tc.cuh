@@ -35,6 +35,10 @@ struct TcGemm {
   int chain = 0;         // MMAs (of 16 k) per drain of the accumulators: 2 (types 1, 3), 8, 16; 0: by size
   TcCols b[2];           // columns of B, one part after the other
   int nb = 1;
+  // [round_up(Jn, 16)][2], for an operand of one part and two Khatri-Rao
+  // factors that the data decide: the powers of two tcg_prepare takes off the
+  // factors of each column, given back to C (tcg_range_kernel)
+  int32_t* shift = nullptr;
   void* C = nullptr;
   int64_t ldc = 0;
   // B as the kernel reads it (tcg_prepare), if the caller keeps it

@@ -2063,6 +2063,7 @@ ttnn_status run_ttn_update(ttnn_plan_s& P, void* acc, const double* const* cores
           g.b[0].krn[k] = (int32_t)f[k]->ax[kf[k]].size;
           view_w(*f[k], kf[k], &g.b[0].ki[k], &g.b[0].kj[k]);
         }
+        g.shift = (int32_t*)C.ws.alloc(round_up(g.Jn, 16) * 8);
         View& e = E[c];
         tc_gemm(C, g, {f[0]->ptr, f[1]->ptr}, &e.ptr, &e.ld);
         e.ax = {Ax{AX_SK, kRankAxis - c, R(c), 0}, Ax{AX_J, -1, g.Jn, 0}};
