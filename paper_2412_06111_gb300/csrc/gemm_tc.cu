@@ -6,9 +6,11 @@
 // products run on the tensor cores.
 //
 // Precision.  bfloat16 operands are multiplied as they are.  A binary32
-// operand is cut into three bfloat16 pieces that sum to it exactly (cut3); the
-// six products down to 2^-16 of the leading one are formed, the other three
-// (2^-24 and below, of either sign) are left out.  The tensor core truncates when it adds to
+// operand is cut into three bfloat16 pieces, the second and third scaled by 2^6
+// and 2^12, which give every entry from 2^-122 in magnitude on exactly (below, a
+// multiple of 2^-145 next to it; cut3).  The six products down to 2^-16 of the
+// leading one are formed, the other three (2^-24 and below, of either sign) are
+// left out.  The tensor core truncates when it adds to
 // its binary32 accumulator, so chains are short: the leading products of 32 to
 // 256 k go into one accumulator, those of each lower order into another, and the
 // epilogue warps add them to registers with rounding to nearest.  The pieces
@@ -162,15 +164,22 @@ struct Pair<double, VEC> {
 // then average to nothing (a 200-rank tree's Psi erred by 6.2e-7 with both cut
 // toward zero, 4.8e-7 so).  The rest of an infinity is NaN: a non-finite entry
 // makes every result it reaches NaN.
+//
+// bfloat16 ends at 2^-133: unscaled, the pieces of a binary32 entry below 2^-110
+// lose its low bits (entries of 1e-35: 4.4e-6 off).  With piece i times 2^(6 i) the
+// products of order o = i + j are 2^(6 o) too large, which the epilogue takes
+// back; 2^6 is the most for which the sums of order 1 (two products below 2^-7
+// of the leading one each) cannot overflow before those of order 0.
+constexpr float kPieceScale = 64.f;
 __device__ __forceinline__ void cut3(float x, float y, uint32_t* w) {
   const uint32_t ux = __float_as_uint(x), uy = __float_as_uint(y);
   w[0] = __byte_perm(ux, uy, 0x7632);
-  x -= __uint_as_float(ux & 0xFFFF0000u);
-  y -= __uint_as_float(uy & 0xFFFF0000u);
+  x = (x - __uint_as_float(ux & 0xFFFF0000u)) * kPieceScale;
+  y = (y - __uint_as_float(uy & 0xFFFF0000u)) * kPieceScale;
   const __nv_bfloat162 v = __floats2bfloat162_rn(x, y);
   w[1] = *reinterpret_cast<const uint32_t*>(&v);
-  x -= __uint_as_float(w[1] << 16);
-  y -= __uint_as_float(w[1] & 0xFFFF0000u);
+  x = (x - __uint_as_float(w[1] << 16)) * kPieceScale;
+  y = (y - __uint_as_float(w[1] & 0xFFFF0000u)) * kPieceScale;
   w[2] = __byte_perm(__float_as_uint(x), __float_as_uint(y), 0x7632);
 }
 
@@ -503,7 +512,7 @@ __global__ void __launch_bounds__(tcg_threads<EPI>(), 1)
           for (int c = 0; c < 8; ++c) {
             float v = __uint_as_float(x[NACC - 1][c]);
 #pragma unroll
-            for (int o = NACC - 2; o >= 0; --o) v += __uint_as_float(x[o][c]);
+            for (int o = NACC - 2; o >= 0; --o) v = fmaf(v, 1.f / kPieceScale, __uint_as_float(x[o][c]));
             acc[cg + c] += v;
           }
         }

@@ -47,3 +47,45 @@ def test_environments_and_sketches_of_any_size(network):
     assert rel(pr, Pr) <= 1e-5
     for v in t.sketched():
         assert rel(om[v], Om[v]) <= 1e-5 and rel(ps[v], Ps[v]) <= 1e-5, v
+
+
+def _sketch_errors(tr, dims, r, p, data, dtype, seed, flags):
+    n = len(tr[0])
+    t = Tree(tr[0], tr[1], dims, [r] * n, [p] * n, tr[2])
+    want = O.sketch_ttnn(data.astype(np.float64), t, O.Drm(t, seed, {api.F32: "f32", api.F64: "f64"}[dtype], "ttnn"))
+    run = Run(tr, dims, [r] * n, [p] * n, seed, dtype=dtype, flags=flags)
+    try:
+        api.ttnn_update_dense(run.state, torch.from_numpy(data).cuda())
+        assert api.ttnn_plan_pass_counts(run.plan) == ((0, 1) if flags else (1, 0))
+        got = run.sketches()
+    finally:
+        run.close()
+    return max([rel(got[2], want[2])] + [rel(got[k][v], want[k][v]) for k in (0, 1) for v in t.sketched()])
+
+
+# binary32 entries whose low bits a bfloat16 piece could not hold (its numbers
+# end at 2^-133) and ones near the largest; no further off than twice the FP32
+# units, whose own error is about 2e-7 (floor 5e-7)
+@pytest.mark.parametrize("scale", [1e-36, 1e-34, 1e-30, 1.0, 1e30, 1e33])
+def test_binary32_tensors_of_any_size(scale):
+    dims = [43, 41, 39, 37]
+    data = W.gaussian(dims, 9).astype(np.float32) * np.float32(scale)
+    tc, simt = (_sketch_errors(W.balanced_binary(4), dims, 11, 6, data, api.F32, 83, f) for f in (0, api.FLAG_SIMT_PASS))
+    assert tc <= max(2 * simt, 5e-7), (tc, simt)
+
+
+def test_small_core_keeps_its_bits():
+    # a large core of 1e-36 below a root of 1e30; binary32 FMAs err by 4e-7
+    tr, dims, r, p = W.balanced_binary(4), [40, 30, 35, 33], 20, 9
+    R, n = [1, 64, 128, 128, 64, 128, 127], 7
+    cores = W.ttn_cores(tr, dims, R, np.random.default_rng(22))
+    cores[0], cores[1] = cores[0] * 1e30, cores[1] * 1e-36
+    t = Tree(tr[0], tr[1], dims, [r] * n, [p] * n, tr[2])
+    Om, Ps, Pr = OR.sketch_ttn_input(cores, t, O.Drm(t, 43, "f32", "round"))
+    run = Run(tr, dims, [r] * n, [p] * n, 43, dtype=api.F32)
+    try:
+        api.ttnn_update_ttn(run.state, [torch.from_numpy(np.ascontiguousarray(cores[v])).cuda() for v in range(n)], R)
+        om, ps, pr = run.sketches()
+    finally:
+        run.close()
+    assert max([rel(pr, Pr)] + [e for v in t.sketched() for e in (rel(om[v], Om[v]), rel(ps[v], Ps[v]))]) <= 1e-6
