@@ -162,8 +162,9 @@ struct Pair<double, VEC> {
 // first is cut toward zero, so that no finite value overflows; the second is
 // rounded, which leaves the third either sign: the piece products left out
 // then average to nothing (a 200-rank tree's Psi erred by 6.2e-7 with both cut
-// toward zero, 4.8e-7 so).  The rest of an infinity is NaN: a non-finite entry
-// makes every result it reaches NaN.
+// toward zero, 4.8e-7 so).  The first piece of an infinity or NaN is it, its
+// other pieces are NaN: where the leading products of a sum are not finite, the
+// epilogue takes them alone, which gives what binary32 multiply-adds give.
 //
 // bfloat16 ends at 2^-133: unscaled, the pieces of a binary32 entry below 2^-110
 // lose its low bits (entries of 1e-35: 4.4e-6 off).  With piece i times 2^(6 i) the
@@ -172,10 +173,10 @@ struct Pair<double, VEC> {
 // of the leading one each) cannot overflow before those of order 0.
 constexpr float kPieceScale = 64.f;
 __device__ __forceinline__ void cut3(float x, float y, uint32_t* w) {
-  const uint32_t ux = __float_as_uint(x), uy = __float_as_uint(y);
-  w[0] = __byte_perm(ux, uy, 0x7632);
-  x = (x - __uint_as_float(ux & 0xFFFF0000u)) * kPieceScale;
-  y = (y - __uint_as_float(uy & 0xFFFF0000u)) * kPieceScale;
+  // (not a cut of the bits: a NaN may have all of its in the lower half)
+  asm("cvt.rz.bf16x2.f32 %0, %1, %2;" : "=r"(w[0]) : "f"(y), "f"(x));
+  x = (x - __uint_as_float(w[0] << 16)) * kPieceScale;
+  y = (y - __uint_as_float(w[0] & 0xFFFF0000u)) * kPieceScale;
   const __nv_bfloat162 v = __floats2bfloat162_rn(x, y);
   w[1] = *reinterpret_cast<const uint32_t*>(&v);
   x = (x - __uint_as_float(w[1] << 16)) * kPieceScale;
@@ -513,6 +514,7 @@ __global__ void __launch_bounds__(tcg_threads<EPI>(), 1)
             float v = __uint_as_float(x[NACC - 1][c]);
 #pragma unroll
             for (int o = NACC - 2; o >= 0; --o) v = fmaf(v, 1.f / kPieceScale, __uint_as_float(x[o][c]));
+            if (NACC > 1 && !isfinite(__uint_as_float(x[0][c]))) v = __uint_as_float(x[0][c]);
             acc[cg + c] += v;
           }
         }

@@ -89,3 +89,45 @@ def test_small_core_keeps_its_bits():
     finally:
         run.close()
     assert max([rel(pr, Pr)] + [e for v in t.sketched() for e in (rel(om[v], Om[v]), rel(ps[v], Ps[v]))]) <= 1e-6
+
+
+def _same_values_that_are_not_finite(got, want):
+    got, want = np.asarray(got, np.float64).ravel(), np.asarray(want, np.float64).ravel()
+    return np.array_equal(np.nan_to_num(got, nan=2.0, posinf=3.0, neginf=-3.0)[~np.isfinite(want)],
+                          np.nan_to_num(want, nan=2.0, posinf=3.0, neginf=-3.0)[~np.isfinite(want)]) and \
+        np.array_equal(np.isfinite(got), np.isfinite(want))
+
+
+def _check_not_finite(dims, r, p, dtype, data, flags=0):
+    """Every sketch has NaN, +Inf and -Inf where the definition has them."""
+    tr = W.balanced_binary(len(dims))
+    n = len(tr[0])
+    t = Tree(tr[0], tr[1], dims, [r] * n, [p] * n, tr[2])
+    with np.errstate(invalid="ignore", over="ignore"):
+        want = O.sketch_ttnn(data.astype(np.float64), t, O.Drm(t, 31, {api.F32: "f32", api.F64: "f64"}[dtype], "ttnn"))
+    run = Run(tr, dims, [r] * n, [p] * n, 31, dtype=dtype, flags=flags)
+    try:
+        api.ttnn_update_dense(run.state, torch.from_numpy(data).cuda())
+        assert api.ttnn_plan_pass_counts(run.plan) == ((0, 1) if flags else (1, 0))
+        got = run.sketches()
+    finally:
+        run.close()
+    assert _same_values_that_are_not_finite(got[2], want[2])
+    for k in (0, 1):
+        for v in t.sketched():
+            assert _same_values_that_are_not_finite(got[k][v], want[k][v]), (k, v)
+
+
+@pytest.mark.parametrize("bad", [np.inf, -np.inf, np.nan])
+def test_binary32_entries_that_are_not_finite(bad):
+    dims = [43, 41, 39, 37]
+    data = W.gaussian(dims, 9).astype(np.float32)
+    data[7, 8, 9, 10] = bad
+    _check_not_finite(dims, 11, 6, api.F32, data)
+
+
+def test_binary32_nan_with_all_its_bits_low():
+    dims = [43, 41, 39, 37]
+    data = W.gaussian(dims, 9).astype(np.float32)
+    data.reshape(-1).view(np.uint32)[123457] = 0x7F800001
+    _check_not_finite(dims, 11, 6, api.F32, data)
