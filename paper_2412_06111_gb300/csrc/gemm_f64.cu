@@ -17,7 +17,8 @@
 // time and erred more than the FP64 units' sums: the columns of B are
 // Khatri-Rao products whose largest entry is 100 times their mean.)  Row
 // exponents only grow within a sum; when one does, its accumulators are
-// shifted.  A NaN or infinity makes the results of its row (column) NaN.
+// shifted.  Digits hold no infinity or NaN: the results of a row (column) with
+// one are taken from the operands themselves (zpieces_kernel).
 //
 // The digits of A are formed by integer instructions in converter warps on
 // the way from global to shared memory (no FP64 instruction is used per
@@ -47,6 +48,8 @@ constexpr int kZSmem = 1024 + 2 * (int)kZStage + kZBBufs * kZDigits * kZMaxN * 1
 struct ZParams {
   const double* A;
   int64_t lda, I, K;
+  const double* B;       // [Jn][ldb], the columns of B^T as given
+  int64_t ldb;
   int nI, nkb;           // row tiles, B tiles along k
   int Npad, Jn;          // columns of this launch, padded and valid
   int stages;
@@ -583,23 +586,36 @@ __global__ void __launch_bounds__(256) zslice_kernel(const __grid_constant__ ZPr
   }
 }
 
-__global__ void __launch_bounds__(256) zpieces_kernel(const double* part, int64_t I, int nI,
-                                                      int nkb, int G, int Npad, double* C,
-                                                      int64_t ldc) {
-  const int it = blockIdx.x;
-  const int64_t total = (int64_t)nI * nkb;
+// Sums the pieces of the row tiles that more than one CTA worked on.  Where an
+// infinity or NaN of A or B has left NaN, the entry is summed from the operands
+// by multiply-adds, as the FP64 units would (up to the first NaN of its sum).
+// Whole tiles are looked over for that as well: a read of C.
+template <bool MN>
+__global__ void __launch_bounds__(256) zpieces_kernel(const ZParams p, int G) {
+  const int it = blockIdx.x, nkb = p.nkb, Npad = p.Npad;
+  const int64_t total = (int64_t)p.nI * nkb;
   auto owner = [&](int64_t u) { return (int)(((u + 1) * G - 1) / total); };
   const int c0 = owner((int64_t)it * nkb), c1 = owner((int64_t)(it + 1) * nkb - 1);
-  if (c0 == c1) return;
-  const int rows = (int)min((int64_t)kTileM, I - (int64_t)it * kTileM);
+  const int rows = (int)min((int64_t)kTileM, p.I - (int64_t)it * kTileM);
   const int64_t tile = (int64_t)kTileM * Npad;
   // only the first CTA's range can begin in an earlier tile
-  const double* p0 = part + (int64_t)(2 * c0 + ((int)(total * c0 / G / nkb) < it)) * tile;
+  const double* p0 = p.part + (int64_t)(2 * c0 + ((int)(total * c0 / G / nkb) < it)) * tile;
   for (int e = blockIdx.y * 256 + threadIdx.x; e < rows * Npad; e += gridDim.y * 256) {
-    double a = p0[e];
+    const int64_t row = (int64_t)it * kTileM + e / Npad;
+    const int col = e % Npad;
+    double* out = p.C + row * p.ldc + col;
+    double a = c0 == c1 ? *out : p0[e];
 #pragma unroll 4
-    for (int c = c0 + 1; c <= c1; ++c) a += part[(int64_t)(2 * c) * tile + e];
-    C[((int64_t)it * kTileM + e / Npad) * ldc + e % Npad] = a;
+    for (int c = c0 + 1; c <= c1; ++c) a += p.part[(int64_t)(2 * c) * tile + e];
+    if (isnan(a) && col < p.Jn) {
+      const double* x = p.A + row * (MN ? 1 : p.lda);
+      const double* y = p.B + col * p.ldb;
+      a = 0.;
+      for (int64_t k = 0; k < p.K && !isnan(a); ++k) a = __fma_rn(x[k * (MN ? p.lda : 1)], y[k], a);
+    } else if (c0 == c1) {
+      continue;
+    }
+    *out = a;
   }
 }
 
@@ -683,6 +699,8 @@ ttnn_status launch_zgemm(const TcGemm& g, const void* prep, void* pieces, int sm
     p.lda = g.lda;
     p.I = g.I;
     p.K = g.K;
+    p.B = (const double*)g.b[0].p + j0 * g.b[0].sj;
+    p.ldb = g.b[0].sj;
     p.nI = o.nI;
     p.nkb = o.nkb;
     p.Npad = std::min(kZMaxN, o.W - j0);
@@ -702,10 +720,10 @@ ttnn_status launch_zgemm(const TcGemm& g, const void* prep, void* pieces, int sm
     const bool vec = inner % 2 == 0 && g.lda % 2 == 0 && (uintptr_t)g.A % 16 == 0;
     if (g.mn) TTNN_TRY(vec ? z_launch<true, true>(o, mB, p, st) : z_launch<true, false>(o, mB, p, st));
     else TTNN_TRY(vec ? z_launch<false, true>(o, mB, p, st) : z_launch<false, false>(o, mB, p, st));
-    if (o.grid == 1) continue;
     const int per = (int)std::max<int64_t>(1, std::min<int64_t>(16, 2432 / std::max(1, o.nI)));
-    zpieces_kernel<<<dim3((unsigned)o.nI, (unsigned)per), 256, 0, st>>>(
-        p.part, g.I, o.nI, o.nkb, o.grid, p.Npad, p.C, p.ldc);
+    const dim3 pg((unsigned)o.nI, (unsigned)per);
+    if (g.mn) zpieces_kernel<true><<<pg, 256, 0, st>>>(p, o.grid);
+    else zpieces_kernel<false><<<pg, 256, 0, st>>>(p, o.grid);
     TTNN_TRY(check_launch("zpieces_kernel"));
   }
   return TTNN_OK;

@@ -131,3 +131,20 @@ def test_binary32_nan_with_all_its_bits_low():
     data = W.gaussian(dims, 9).astype(np.float32)
     data.reshape(-1).view(np.uint32)[123457] = 0x7F800001
     _check_not_finite(dims, 11, 6, api.F32, data)
+
+
+# a row tile of one CTA and tiles cut over many; an entry early and one late
+@pytest.mark.parametrize("bad", [np.inf, -np.inf, np.nan])
+@pytest.mark.parametrize("dims,at", [([12, 10, 12], 5), ([20, 24, 90], 777), ([37, 35, 129], 160000),
+                                     ([190, 110, 200], 3000000)])
+def test_binary64_entries_that_are_not_finite(dims, at, bad):
+    data = W.gaussian(dims, 9)
+    data.reshape(-1)[at] = bad
+    _check_not_finite(dims, 6, 4, api.F64, data)
+
+
+def test_binary64_infinities_of_both_signs_in_one_row():
+    dims = [20, 24, 90]
+    data = W.gaussian(dims, 9)
+    data[3, 4, 7], data[3, 4, 60], data[3, 5, 7] = np.inf, -np.inf, np.inf
+    _check_not_finite(dims, 6, 4, api.F64, data)
