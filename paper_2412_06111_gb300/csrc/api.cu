@@ -82,7 +82,7 @@ static ttnn_status grow_workspace(ttnn_plan_s& P, int64_t bytes) {
   cudaFree(P.ws);
   P.dev_bytes += bytes - P.ws_bytes;
   P.ws = fresh;
-  P.ws_bytes = bytes;
+  P.ws_bytes = P.ws_limit = bytes;
   return TTNN_OK;
 }
 

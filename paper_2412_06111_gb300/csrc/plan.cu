@@ -1279,8 +1279,11 @@ ttnn_status dense_update_need(ttnn_plan_s& P, const Box& box, int64_t* need) {
     P.roomy = true;
     TTNN_TRY(run_dense_update(P, nullptr, nullptr, box, nullptr, 1.0, nullptr, true, &n));
     if (n > P.ws_limit) {
+      int64_t least = 0;
       P.roomy = false;
-      TTNN_TRY(run_dense_update(P, nullptr, nullptr, box, nullptr, 1.0, nullptr, true, &n));
+      TTNN_TRY(run_dense_update(P, nullptr, nullptr, box, nullptr, 1.0, nullptr, true, &least));
+      P.roomy = least >= n;   // (the general forms may take more)
+      n = std::min(n, least);
     }
     it = P.ws_need_cache.emplace(key, std::make_pair(n, P.roomy)).first;
   }

@@ -135,8 +135,8 @@ ttnn_status build_plan(ttnn_plan_s& P, const ttnn_tree* tree, int32_t d, const i
 // Runs (or, with dry = true, sizes) one dense update.  Returns the peak
 // workspace bytes through *peak when dry.
 // Workspace bytes a dense update of `box` needs (dry run, cached per shape):
-// with the forms that need the most scratch if that is within P.ws_limit, else
-// without them (P.roomy tells).
+// with the forms that trade scratch for speed if that is within P.ws_limit or
+// no more than without them, else without them (P.roomy tells).
 ttnn_status dense_update_need(ttnn_plan_s& P, const Box& box, int64_t* need);
 // Workspace bytes of a CP update (any rank: ranks are taken kProjQ at a time).
 int64_t cp_update_need(const ttnn_plan_s& P);
