@@ -105,6 +105,27 @@ static Box full_box(const ttnn_plan_s& P) {
   return b;
 }
 
+// Scratch of a plan's updates: the larger of a whole-tensor update (cached DRM
+// blocks), an update of a box as large as the tensor (blocks generated into
+// the workspace: bounds every box update) and a CP update; TTN-format updates
+// grow the workspace on demand.
+static ttnn_status update_scratch(ttnn_plan_s& P, int64_t* need) {
+  *need = 0;
+  if (!(P.flags & TTNN_FLAG_STRUCTURED_ONLY)) {
+    Box b = full_box(P);
+    TTNN_TRY(dense_update_need(P, b, need));
+    if (!(P.flags & TTNN_FLAG_DENSE_DRM)) {   // that form takes whole tensors only
+      b.full = false;
+      int64_t need_b = 0;
+      TTNN_TRY(dense_update_need(P, b, &need_b));
+      *need = std::max(*need, need_b);
+    }
+  }
+  if (P.variant == TTNN_VARIANT_TTNN && !(P.flags & TTNN_FLAG_DENSE_DRM))
+    *need = std::max(*need, cp_update_need(P));
+  return TTNN_OK;
+}
+
 }  // namespace ttnn
 
 using namespace ttnn;
@@ -244,8 +265,11 @@ ttnn_status ttnn_plan_create(const ttnn_tree* tree, int32_t d, const int64_t* di
                                  st)) != TTNN_OK)
         return fail(s);
     }
-    if (const int64_t bytes = tcg_plan_bytes(P)) {
-      if ((s = palloc(&P.prep_block, bytes)) != TTNN_OK) return fail(s);
+    // (where there is no memory for them, updates prepare these operands in
+    // the workspace)
+    const int64_t prep = tcg_plan_bytes(P);
+    if (prep > 0 && palloc(&P.prep_block, prep) == TTNN_OK) {
+      P.prep_bytes = prep;
       if ((s = tcg_plan_prepare(P, st)) != TTNN_OK) return fail(s);
     }
     if (omega_via_d2(P, nL, nR)) {
@@ -253,27 +277,19 @@ ttnn_status ttnn_plan_create(const ttnn_tree* tree, int32_t d, const int64_t* di
       if ((s = make_side_xo(P, fb, P.xWo, nR, st))) return fail(s);
     }
   }
-  // workspaces: updates -- the larger of a whole-tensor update (cached DRM
-  // blocks), an update of a box as large as the tensor (blocks generated into
-  // the workspace: bounds every box update) and a CP update; TTN-format
-  // updates grow it on demand -- and, apart, the recovery's
+  // workspaces: the updates' and, apart, the recovery's
   int64_t need_u = 0, need_r = 0;
-  if (dense) {
-    if ((s = dense_update_need(P, fb, &need_u))) return fail(s);
-    if (!(P.flags & TTNN_FLAG_DENSE_DRM)) {   // that form takes whole tensors only
-      Box bb = fb;
-      bb.full = false;
-      int64_t need_b = 0;
-      if ((s = dense_update_need(P, bb, &need_b))) return fail(s);
-      need_u = std::max(need_u, need_b);
-    }
-  }
-  if (P.variant == TTNN_VARIANT_TTNN && !(P.flags & TTNN_FLAG_DENSE_DRM))
-    need_u = std::max(need_u, cp_update_need(P));
+  if ((s = update_scratch(P, &need_u))) return fail(s);
   if ((s = run_recover(P, nullptr, nullptr, st, true, &need_r))) return fail(s);
   P.ws_bytes = need_u + 4096;
+  if ((s = palloc((void**)&P.ws, P.ws_bytes)) != TTNN_OK) {
+    // no memory for the forms that take the most scratch: without them
+    P.ws_limit = 0;
+    if (update_scratch(P, &need_u) != TTNN_OK || need_u + 4096 >= P.ws_bytes) return fail(s);
+    P.ws_bytes = need_u + 4096;
+    if ((s = palloc((void**)&P.ws, P.ws_bytes)) != TTNN_OK) return fail(s);
+  }
   P.ws_limit = P.ws_bytes;
-  if ((s = palloc((void**)&P.ws, P.ws_bytes)) != TTNN_OK) return fail(s);
   P.ws_rec_bytes = need_r + 4096;
   if ((s = palloc((void**)&P.ws_rec, P.ws_rec_bytes)) != TTNN_OK) return fail(s);
   if ((s = palloc((void**)&P.jobs_dev, std::max(1, P.n_sketched) * (int64_t)sizeof(QrJob))) != TTNN_OK) return fail(s);

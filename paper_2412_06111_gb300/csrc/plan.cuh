@@ -70,8 +70,10 @@ struct ttnn_plan_s {
   // tensor-core pass of whole-tensor updates)
   void* sideRs = nullptr;
   void* sideLs = nullptr;
-  // whole-tensor updates on the tensor-core GEMM: its prepared operands
+  // whole-tensor updates on the tensor-core GEMM: its prepared operands (null
+  // where there was no memory for them)
   void* prep_block = nullptr;
+  int64_t prep_bytes = 0;
   void* prep[2] = {nullptr, nullptr};
   void* dxy = nullptr;          // unstructured DRMs of every node, walk type (TTNN_FLAG_DENSE_DRM)
   char* ws = nullptr;

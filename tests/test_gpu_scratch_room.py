@@ -45,3 +45,42 @@ def test_grown_workspace_is_used(dims):
         assert _distance(run, tr, dims, r, p, "bf16", dense, 5) <= 1e-5
     finally:
         run.close()
+
+
+@pytest.mark.parametrize("dtype,fmt,tol", [(api.F64, "f64", 1e-12), (api.F32, "f32", 1e-5)])
+def test_plan_creation_goes_without_optional_memory(dtype, fmt, tol):
+    # each device allocation of a plan fails in turn: where the block only
+    # makes updates faster the plan is made without it, and its updates agree
+    tr, dims, r, p = W.balanced_binary(3), [45, 47, 1009], 6, 4
+    n = len(tr[0])
+    data = W.gaussian(dims, 8)
+    tdt = torch.float64 if dtype == api.F64 else torch.float32
+    dev = torch.from_numpy(data).to(tdt).cuda()
+    dense = dev.double().cpu().numpy()
+    make = lambda: Run(tr, dims, [r] * n, [p] * n, 3, dtype=dtype)
+    whole = make()
+    full = api.ttnn_plan_device_bytes(whole.plan)[0]
+    whole.close()
+    less = 0
+    try:
+        for k in range(1, 64):
+            api.ttnn_debug_fail_alloc(k)
+            try:
+                run = make()
+            except api.TtnnError as e:
+                assert e.status == 2
+                continue
+            api.ttnn_debug_fail_alloc(0)
+            size = api.ttnn_plan_device_bytes(run.plan)[0]
+            try:
+                api.ttnn_update_dense(run.state, dev)
+                assert _distance(run, tr, dims, r, p, fmt, dense, 3) <= tol
+            finally:
+                run.close()
+            assert size <= full
+            less += size < full
+            if size == full:
+                break
+    finally:
+        api.ttnn_debug_fail_alloc(0)
+    assert less >= 2      # the prepared operands; the larger workspace
