@@ -543,8 +543,23 @@ ttnn_status ttnn_update_ttn(ttnn_state_t S, const double* const* cores_in, const
   TTNN_CHECK_ARG(std::isfinite(lambda), "non-finite lambda");
   const cudaStream_t st = (cudaStream_t)stream;
   int64_t need = 0;
+  P.roomy = true;
   TTNN_TRY(run_ttn_update(P, nullptr, cores_in, ranks_in, lambda, st, true, &need));
-  if (need > P.ws_bytes) TTNN_TRY(grow_workspace(P, need + 4096));
+  if (need > P.ws_bytes) {
+    // where the workspace cannot grow (no memory, or a graph is captured) the
+    // general form runs in what there is, or asks for less
+    cudaStreamCaptureStatus cs = cudaStreamCaptureStatusNone;
+    if (cudaStreamIsCapturing(st, &cs) != cudaSuccess) cudaGetLastError();
+    ttnn_status grown = TTNN_ENOMEM;
+    if (cs == cudaStreamCaptureStatusNone) grown = grow_workspace(P, need + 4096);
+    if (grown != TTNN_OK) {
+      int64_t least = 0;
+      P.roomy = false;
+      TTNN_TRY(run_ttn_update(P, nullptr, cores_in, ranks_in, lambda, st, true, &least));
+      if (least >= need && cs == cudaStreamCaptureStatusNone) return grown;
+      if (least > P.ws_bytes) TTNN_TRY(grow_workspace(P, least + 4096));
+    }
+  }
   return run_ttn_update(P, S->acc, cores_in, ranks_in, lambda, st, false, nullptr);
 }
 

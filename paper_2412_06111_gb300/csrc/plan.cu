@@ -1887,7 +1887,7 @@ ttnn_status run_ttn_update(ttnn_plan_s& P, void* acc, const double* const* cores
   std::vector<char> big(nn, 0);
   for (int v = 0; v < nn; ++v) {
     const TNode& nd = P.nodes[v];
-    if (P.walk_f64 || v == P.root || nd.leaf || nd.ch.size() != 2 || nd.rsub == 0) continue;
+    if (!P.roomy || P.walk_f64 || v == P.root || nd.leaf || nd.ch.size() != 2 || nd.rsub == 0) continue;
     const int64_t c1 = R(nd.ch[0]), c2 = R(nd.ch[1]);
     TcGemm up;
     up.type = 3;

@@ -82,7 +82,7 @@ struct ttnn_plan_s {
   // (its workspace is sized then), later that workspace's size
   int64_t ws_limit = INT64_MAX;
   // the update at hand may take the forms that need more scratch than the
-  // ones they replace (set by dense_update_need for each update)
+  // ones they replace (set for each update, before it is planned)
   bool roomy = true;
   // the recovery's own scratch: a recovery may run on another stream while
   // the next update of another state of the plan uses `ws`

@@ -4,6 +4,7 @@ import numpy as np
 import pytest
 
 import workloads as W
+from oracle import rounding as OR
 from oracle import ttnn as O
 from oracle.tree import Tree
 
@@ -84,3 +85,42 @@ def test_plan_creation_goes_without_optional_memory(dtype, fmt, tol):
     finally:
         api.ttnn_debug_fail_alloc(0)
     assert less >= 2      # the prepared operands; the larger workspace
+
+
+def test_ttn_updates_run_where_the_workspace_cannot_grow():
+    # large cores take more scratch on the tensor cores than in the general
+    # form: without memory for it, and in a capture, the general form runs
+    tr, dims, r, p = W.balanced_binary(4), [64] * 4, 25, 12
+    n, R = len(tr[0]), [96] * len(tr[0])
+    cores = W.ttn_cores(tr, dims, R, np.random.default_rng(2))
+    dev = [torch.from_numpy(np.ascontiguousarray(cores[v])).cuda() for v in range(n)]
+    t = Tree(tr[0], tr[1], dims, [r] * n, [p] * n, tr[2])
+    Om, Ps, Pr = OR.sketch_ttn_input(cores, t, O.Drm(t, 6, "f32", "round"))
+
+    def distance(run, scale):
+        om, ps, pr = run.sketches()
+        return max([rel(pr, scale * Pr)] + [e for v in t.sketched() for e in
+                                            (rel(om[v], scale * Om[v]), rel(ps[v], scale * Ps[v]))])
+
+    make = lambda: Run(tr, dims, [r] * n, [p] * n, 6, dtype=api.F32, flags=api.FLAG_STRUCTURED_ONLY)
+    run, room = make(), make()
+    try:
+        api.ttnn_update_ttn(room.state, dev, R)
+        assert distance(room, 1) <= 1e-5
+        api.ttnn_debug_fail_alloc(1)
+        api.ttnn_update_ttn(run.state, dev, R)
+        api.ttnn_debug_fail_alloc(0)
+        assert distance(run, 1) <= 1e-5
+        small = api.ttnn_plan_device_bytes(run.plan)[1]
+        assert small < api.ttnn_plan_device_bytes(room.plan)[1]
+        graph = torch.cuda.CUDAGraph()
+        stream = torch.cuda.Stream()
+        with torch.cuda.graph(graph, stream=stream):
+            api.ttnn_update_ttn(run.state, dev, R, stream=stream.cuda_stream)
+        graph.replay()
+        assert distance(run, 2) <= 1e-5
+        assert api.ttnn_plan_device_bytes(run.plan)[1] == small
+    finally:
+        api.ttnn_debug_fail_alloc(0)
+        run.close()
+        room.close()
