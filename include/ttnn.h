@@ -428,7 +428,10 @@ ttnn_status ttnn_server_create(const ttnn_server_opts* opts, ttnn_server_t* out)
 void ttnn_server_destroy(ttnn_server_t server);
 /* Opens a stream: a plan + zeroed state as ttnn_plan_create /
  * ttnn_state_create (same arguments).  Admission: EBUSY (nothing kept) when
- * the stream's device memory would take the open streams over the budget. */
+ * the stream's device memory would take the open streams over the budget, also
+ * without the memory that only makes updates faster (prepared operands, scratch
+ * of the tensor-core GEMMs): near the budget the new stream and idle ones whose
+ * state handle was not asked for give that up. */
 ttnn_status ttnn_server_open(ttnn_server_t server, const ttnn_tree* tree, int32_t d,
                              const int64_t* dims, const int32_t* ranks,
                              const int32_t* oversample, uint64_t seed, const ttnn_opts* opts,

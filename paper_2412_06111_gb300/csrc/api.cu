@@ -126,6 +126,39 @@ static ttnn_status update_scratch(ttnn_plan_s& P, int64_t* need) {
   return TTNN_OK;
 }
 
+// Workspace bytes with no more than the general forms need (at most the
+// present ones).
+static int64_t least_workspace(ttnn_plan_s& P) {
+  const int64_t limit = P.ws_limit;
+  int64_t need = 0;
+  P.ws_limit = 0;
+  const ttnn_status s = update_scratch(P, &need);
+  P.ws_limit = limit;
+  return s == TTNN_OK ? std::min(need + 4096, P.ws_bytes) : P.ws_bytes;
+}
+
+int64_t plan_spare_bytes(ttnn_plan_s& P) {
+  return (P.prep_block ? P.prep_bytes : 0) + P.ws_bytes - least_workspace(P);
+}
+
+int64_t plan_trim(ttnn_plan_s& P) {
+  const int64_t before = P.dev_bytes, bytes = least_workspace(P);
+  char* fresh = nullptr;
+  if (bytes < P.ws_bytes && dev_alloc((void**)&fresh, bytes) == TTNN_OK) {
+    cudaFree(P.ws);   // waits for the device
+    P.dev_bytes += bytes - P.ws_bytes;
+    P.ws = fresh;
+    P.ws_bytes = P.ws_limit = bytes;
+  }
+  if (P.prep_block) {
+    cudaFree(P.prep_block);
+    P.prep_block = P.prep[0] = P.prep[1] = nullptr;
+    P.dev_bytes -= P.prep_bytes;
+  }
+  P.ws_need_cache.clear();   // (sized with the prepared operands)
+  return before - P.dev_bytes;
+}
+
 }  // namespace ttnn
 
 using namespace ttnn;

@@ -136,6 +136,13 @@ ttnn_status build_plan(ttnn_plan_s& P, const ttnn_tree* tree, int32_t d, const i
 
 // Runs (or, with dry = true, sizes) one dense update.  Returns the peak
 // workspace bytes through *peak when dry.
+// Device bytes of a plan that only make its updates faster: the prepared
+// operands, and the workspace beyond what the general forms need.
+int64_t plan_spare_bytes(ttnn_plan_s& P);
+// Gives them back; returns the bytes freed.  Nothing may be queued on the plan,
+// and no graph may hold its workspace.
+int64_t plan_trim(ttnn_plan_s& P);
+
 // Workspace bytes a dense update of `box` needs (dry run, cached per shape):
 // with the forms that trade scratch for speed if that is within P.ws_limit or
 // no more than without them, else without them (P.roomy tells).

@@ -56,6 +56,8 @@ struct Slot {
   ttnn_plan_t plan = nullptr;
   ttnn_state_t state = nullptr;
   int64_t bytes = 0;
+  int64_t spare = 0;     // of them, what plan_trim gives back
+  bool shared = false;   // the caller has the state's handle
   int pending = 0;
 };
 
@@ -358,8 +360,32 @@ ttnn_status ttnn_server_open(ttnn_server_t S, const ttnn_tree* tree, int32_t d, 
     ttnn_plan_destroy(plan);
     return s;
   }
-  const int64_t bytes = plan->dev_bytes + state->elems * (plan->walk_f64 ? 8 : 4);
+  int64_t bytes = plan->dev_bytes + state->elems * (plan->walk_f64 ? 8 : 4);
+  const int64_t spare = plan_spare_bytes(*plan);
   std::lock_guard<std::mutex> lk(S->mu);
+  // Beyond the budget, the memory that only makes updates faster is given up:
+  // the new stream's, then that of idle streams, if that makes room.  Not of
+  // streams whose state the caller has asked for: a graph may hold their
+  // workspace.
+  auto idle = [](const Slot& sl) { return sl.pending == 0 && !sl.shared && sl.spare > 0; };
+  int64_t room = S->budget - S->used + spare;
+  for (auto& kv : S->slots)
+    if (idle(kv.second)) room += kv.second.spare;
+  Slot fresh;
+  fresh.spare = spare;
+  if (S->used + bytes > S->budget && bytes <= room) {
+    bytes -= plan_trim(*plan);
+    fresh.spare = 0;
+    for (auto& kv : S->slots) {
+      Slot& sl = kv.second;
+      if (S->used + bytes <= S->budget) break;
+      if (!idle(sl)) continue;
+      const int64_t freed = plan_trim(*sl.plan);
+      sl.bytes -= freed;
+      S->used -= freed;
+      sl.spare = 0;
+    }
+  }
   if (S->used + bytes > S->budget) {
     ttnn_state_destroy(state);
     ttnn_plan_destroy(plan);
@@ -369,10 +395,10 @@ ttnn_status ttnn_server_open(ttnn_server_t S, const ttnn_tree* tree, int32_t d, 
   }
   S->used += bytes;
   const int id = S->next_stream++;
-  Slot& sl = S->slots[id];
-  sl.plan = plan;
-  sl.state = state;
-  sl.bytes = bytes;
+  fresh.plan = plan;
+  fresh.state = state;
+  fresh.bytes = bytes;
+  S->slots[id] = fresh;
   *stream_id = id;
   return TTNN_OK;
 }
@@ -493,6 +519,7 @@ ttnn_status ttnn_server_stream_state(ttnn_server_t S, int32_t stream_id, ttnn_st
   auto it = S->slots.find(stream_id);
   TTNN_CHECK_ARG(it != S->slots.end(), "no open stream %d", stream_id);
   *state = it->second.state;
+  it->second.shared = true;
   return TTNN_OK;
 }
 

@@ -124,3 +124,58 @@ def test_ttn_updates_run_where_the_workspace_cannot_grow():
         api.ttnn_debug_fail_alloc(0)
         run.close()
         room.close()
+
+
+def _served(srv, dims, r, p, k):
+    tr = W.balanced_binary(3)
+    n = len(tr[0])
+    return api.ttnn_server_open(srv, tr, dims, [r] * n, [p] * n, k, sketch_dtype=api.F64)
+
+
+def test_admission_gives_up_memory_that_only_makes_updates_faster():
+    tr, dims, r, p = W.balanced_binary(3), [45, 47, 1009], 6, 4
+    n = len(tr[0])
+    static = 32 << 20     # the library's scratch block counts against the budget
+    probe = api.ttnn_server_create(8 << 30)
+    try:
+        _served(probe, dims, r, p, 1)
+        full = api.ttnn_server_stats(probe)["device_bytes"]
+    finally:
+        api.ttnn_server_destroy(probe)
+    tight = api.ttnn_server_create(full - 1 + static)
+    try:
+        _served(tight, dims, r, p, 1)
+        least = api.ttnn_server_stats(tight)["device_bytes"]
+        assert least < full
+    finally:
+        api.ttnn_server_destroy(tight)
+    # room for a few streams of the least size: the first is opened in full
+    count = max(3, -(-full // least))
+    data = [W.gaussian(dims, 20 + k) for k in range(3)]
+    srv = api.ttnn_server_create(count * least + static)
+    try:
+        ids = [_served(srv, dims, r, p, 1)]
+        assert api.ttnn_server_stats(srv)["device_bytes"] == full
+        dev = [torch.from_numpy(x).cuda() for x in data]
+        assert api.ttnn_server_wait(srv, api.ttnn_server_submit(srv, ids[0], dev[0]), 5_000_000) == 0
+        ids += [_served(srv, dims, r, p, 1) for _ in range(count - 1)]
+        with pytest.raises(api.TtnnError) as ei:
+            _served(srv, dims, r, p, 1)
+        assert ei.value.status == 6                        # EBUSY
+        for s, d in zip(ids[1:], dev[1:]):
+            assert api.ttnn_server_wait(srv, api.ttnn_server_submit(srv, s, d), 5_000_000) == 0
+        # the trimmed stream goes on
+        assert api.ttnn_server_wait(srv, api.ttnn_server_submit(srv, ids[0], dev[1]), 5_000_000) == 0
+        t = Tree(tr[0], tr[1], dims, [r] * n, [p] * n, tr[2])
+        for s, dense in zip(ids, (data[0] + data[1], data[1], data[2])):
+            state = api.ttnn_server_stream_state(srv, s)
+            plan_nodes = Run(tr, dims, [r] * n, [p] * n, 1, dtype=api.F64)
+            try:
+                buf = np.zeros(plan_nodes.sizes[0])
+                api.ttnn_state_save(state, buf)
+                api.ttnn_state_load(plan_nodes.state, buf)
+                assert _distance(plan_nodes, tr, dims, r, p, "f64", dense, 1) <= 1e-12
+            finally:
+                plan_nodes.close()
+    finally:
+        api.ttnn_server_destroy(srv)
