@@ -999,9 +999,44 @@ void Program::add(const TcOp& op, std::initializer_list<const void*> in) {
     if (out >= b.lo && out < b.hi) b.level = std::max(b.level, lvl);
 }
 
+// Debugging: runs what `launch` issues on `st` alone, synchronised, and prints
+// its time.
+template <typename Launch>
+static ttnn_status timed_alone(cudaStream_t st, const Launch& launch) {
+  cudaEvent_t a = nullptr, e = nullptr;
+  TTNN_TRY_CUDA(cudaEventCreate(&a));
+  TTNN_TRY_CUDA(cudaEventCreate(&e));
+  TTNN_TRY_CUDA(cudaEventRecord(a, st));
+  TTNN_TRY(launch());
+  TTNN_TRY_CUDA(cudaEventRecord(e, st));
+  TTNN_TRY_CUDA(cudaEventSynchronize(e));
+  float ms = 0.f;
+  cudaEventElapsedTime(&ms, a, e);
+  cudaEventDestroy(a);
+  cudaEventDestroy(e);
+  fprintf(stderr, "[ttnn] %8.1f us  ", ms * 1e3f);
+  return TTNN_OK;
+}
+
+static ttnn_status dump_tc(const TcOp& o, cudaStream_t st) {
+  TcGemm g = o.g;
+  g.prep = o.prep;
+  TTNN_TRY(timed_alone(st, [&]() -> ttnn_status {
+    void* const prep = o.prep;
+    TTNN_TRY(tcg_prepare(&o.g, 1, &prep, st));
+    return tcg_run(&g, 1, o.pieces, tcg_sms(), o.err, tcg_wait_ns(), st);
+  }));
+  fprintf(stderr, "[ttnn] L%d tensor-core gemm I %lld K %lld J %d type %d mn %d trans %d\n", o.level,
+          (long long)g.I, (long long)g.K, g.Jn, g.type, g.mn, g.trans);
+  return TTNN_OK;
+}
+
 // The tensor-core GEMMs of a level: their operands in one launch, then the
 // products (those of several plans, with error words of their own, apart).
-ttnn_status Program::run_tc(int lvl, cudaStream_t st) const {
+ttnn_status Program::run_tc(int lvl, cudaStream_t st, bool dump) const {
+  for (const TcOp& o : tcs_)
+    if (dump && o.level == lvl) TTNN_TRY(dump_tc(o, st));
+  if (dump) return TTNN_OK;
   std::vector<TcGemm> g;
   std::vector<void*> prep;
   for (const TcOp& o : tcs_) {
@@ -1178,18 +1213,7 @@ static ttnn_status fork_stream(ForkStream** out) {
 
 // Debugging: one op alone, timed (the stream is synchronised) and printed.
 static ttnn_status dump_op(const Op& o, int lvl, cudaStream_t st) {
-  cudaEvent_t a = nullptr, e = nullptr;
-  TTNN_TRY_CUDA(cudaEventCreate(&a));
-  TTNN_TRY_CUDA(cudaEventCreate(&e));
-  TTNN_TRY_CUDA(cudaEventRecord(a, st));
-  TTNN_TRY(launch_ops(group_of(o), {&o}, st));
-  TTNN_TRY_CUDA(cudaEventRecord(e, st));
-  TTNN_TRY_CUDA(cudaEventSynchronize(e));
-  float ms = 0.f;
-  cudaEventElapsedTime(&ms, a, e);
-  cudaEventDestroy(a);
-  cudaEventDestroy(e);
-  fprintf(stderr, "[ttnn] %8.1f us  ", ms * 1e3f);
+  TTNN_TRY(timed_alone(st, [&] { return launch_ops(group_of(o), {&o}, st); }));
   if (o.kind == OP_SCATTER)
     fprintf(stderr, "[ttnn] L%d scatter nd %d nsc %d blocks %lld\n", lvl, o.s.nd, o.s.nsc,
             (long long)o.blocks);
@@ -1235,7 +1259,7 @@ ttnn_status Program::run(cudaStream_t st, bool dump) {
         gst = fs->st;
       }
     }
-    if (tc) TTNN_TRY(run_tc(lvl, gst));
+    if (tc) TTNN_TRY(run_tc(lvl, gst, dump));
     for (int g = 0; g < LG_COUNT; ++g)
       if (!group[g].empty())
         TTNN_TRY(launch_ops((LaunchGroup)g, group[g], g == LG_KGEMM ? gst : st));

@@ -152,7 +152,7 @@ class Program {
     int level;
   };
   int level_of(const void* p) const;
-  ttnn_status run_tc(int lvl, cudaStream_t st) const;
+  ttnn_status run_tc(int lvl, cudaStream_t st, bool dump) const;
   std::vector<Op> ops_;
   std::vector<TcOp> tcs_;
   std::vector<Buf> bufs_;
