@@ -138,8 +138,8 @@ typedef struct {
                                        ranks, written compactly (row-major) from its offset;
                                        ttnn_plan_node reports those shapes after the recovery */
 #define TTNN_FLAG_WAIT_TEST 32u     /* testing the bounded-wait error path: the pipeline waits
-                                       of the tensor-core passes give up at once, so a dense
-                                       update on this plan is abandoned on the device and the
+                                       of the tensor-core passes and GEMMs give up at once, so
+                                       an update that uses them is abandoned on the device and the
                                        next ttnn_recover / ttnn_plan_sync returns TTNN_ETIMEOUT
                                        (the plan and its CUDA context stay usable) */
 

@@ -604,6 +604,7 @@ static void tc_gemm(Ctx& C, TcGemm g, std::initializer_list<const void*> in, cha
   }
   op.pieces = C.tc_pieces;
   op.err = C.P.err_dev;
+  op.wait_ns = (C.P.flags & TTNN_FLAG_WAIT_TEST) ? 0 : tc::kTimeoutNs;
   op.g = g;
   C.prog->add(op, in);
 }

@@ -68,3 +68,48 @@ def test_dump_shows_every_product(case, products, capfd):
         assert distance() <= 1e-5
     finally:
         run.close()
+
+
+ETIMEOUT = 5
+
+
+def _expect_timeout(run, update):
+    update(run)
+    core = torch.zeros(run.sizes[2], dtype=torch.float64, device="cuda")
+    with pytest.raises(api.TtnnError) as ei:
+        api.ttnn_recover(run.state, core)
+    assert ei.value.status == ETIMEOUT
+    api.ttnn_plan_sync(run.plan)   # reported once
+
+
+# products of a walk alone: the large cores; a prefix behind a first-level
+# product on the FP32 units (SIMT_PASS: it has no waits)
+@pytest.mark.parametrize("case,flags", [(LARGE, 0), (PREFIX, api.FLAG_SIMT_PASS)], ids=["large_cores", "prefix"])
+def test_walk_waits_running_out_report_timeout(case, flags):
+    bad, good = (_open(case, api.F32, flags | f) for f in (api.FLAG_WAIT_TEST, 0))
+    try:
+        _expect_timeout(bad, lambda run: _update(run, case))
+        assert _update(good, case)() <= 1e-5   # the context is intact
+    finally:
+        bad.close()
+        good.close()
+
+
+# first-level products on the two GEMMs: odd rows, K- and MN-major operands of
+# every type, one CTA and many
+@pytest.mark.parametrize("dtype,dims", [(api.F32, [43, 41, 39, 37]), (api.BF16, [43, 41, 39, 37]),
+                                        (api.F64, [43, 41, 39, 37]), (api.F64, [8, 4, 6, 8])])
+def test_first_level_waits_running_out_report_timeout(dtype, dims):
+    case = (W.balanced_binary(4), dims, 6, 3)
+    tdt = {api.F64: torch.float64, api.F32: torch.float32, api.BF16: torch.bfloat16}[dtype]
+    data = torch.from_numpy(W.gaussian(dims, 9)).to(tdt).cuda()
+    bad, good = (_open(case, dtype, f) for f in (api.FLAG_WAIT_TEST, 0))
+    try:
+        _expect_timeout(bad, lambda run: api.ttnn_update_dense(run.state, data))
+        assert api.ttnn_plan_pass_counts(bad.plan) == (1, 0)
+        api.ttnn_update_dense(good.state, data)
+        good.recover()
+        assert np.isfinite(good.state_host()).all()
+    finally:
+        bad.close()
+        good.close()
