@@ -118,7 +118,7 @@ typedef struct {
 #define TTNN_FLAG_DUMP_PROGRAM 16u  /* debugging: run every tree-walk / assembly op as its own
                                        launch, synchronise, and print its time, level, kind,
                                        shape and blocks to stderr */
-#define TTNN_FLAG_RESERVE_SMS 64u   /* the tensor-core first-level passes leave max(8, sketched
+#define TTNN_FLAG_RESERVE_SMS 64u   /* the tensor-core passes and GEMMs leave max(8, sketched
                                        nodes) SMs (at most a quarter) free, so that a recovery
                                        of another state issued on another stream runs beside
                                        the next update's pass instead of after it */

@@ -794,7 +794,6 @@ static ttnn_status tcg_batch(const TcGemm* const* g, int n, void* pieces, int sm
 
 }  // namespace tc
 
-int tcg_sms() { return tc::sm_count(); }
 
 bool tcg_supported(const TcGemm& g) {
   if (g.type == 0) return zgemm_supported(g);

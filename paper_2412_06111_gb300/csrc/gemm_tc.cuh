@@ -63,8 +63,6 @@ ttnn_status tcg_run(const TcGemm* g, int n, void* pieces, int sms, int* err, uin
 // only *need = workspace bytes.
 ttnn_status launch_tcg(const TcGemm* g, int n, int sms, int* err, uint64_t wait_ns, void* ws,
                        int64_t ws_bytes, cudaStream_t st, bool dry, int64_t* need);
-// SMs of the current device.
-int tcg_sms();
 
 // The binary64 parts (gemm_f64.cu).
 bool zgemm_supported(const TcGemm& g);

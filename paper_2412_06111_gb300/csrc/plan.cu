@@ -597,7 +597,8 @@ static void tc_gemm(Ctx& C, TcGemm g, std::initializer_list<const void*> in, cha
   TcOp op;
   if (!g.chain) g.chain = 2;   // walks chain several products: the shortest chains
   op.prep = C.ws.alloc(tcg_prep_bytes(g));
-  const int64_t pieces = tcg_piece_bytes(g, tcg_sms());
+  op.sms = tc::pass_sms(C.P);
+  const int64_t pieces = tcg_piece_bytes(g, op.sms);
   if (pieces > C.tc_piece_bytes) {
     C.tc_pieces = C.ws.alloc(pieces);
     C.tc_piece_bytes = pieces;

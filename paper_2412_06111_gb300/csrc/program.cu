@@ -1024,10 +1024,10 @@ static ttnn_status dump_tc(const TcOp& o, cudaStream_t st) {
   TTNN_TRY(timed_alone(st, [&]() -> ttnn_status {
     void* const prep = o.prep;
     TTNN_TRY(tcg_prepare(&o.g, 1, &prep, st));
-    return tcg_run(&g, 1, o.pieces, tcg_sms(), o.err, o.wait_ns, st);
+    return tcg_run(&g, 1, o.pieces, o.sms, o.err, o.wait_ns, st);
   }));
-  fprintf(stderr, "[ttnn] L%d tensor-core gemm I %lld K %lld J %d type %d mn %d trans %d\n", o.level,
-          (long long)g.I, (long long)g.K, g.Jn, g.type, g.mn, g.trans);
+  fprintf(stderr, "[ttnn] L%d tensor-core gemm I %lld K %lld J %d type %d mn %d trans %d SMs %d\n", o.level,
+          (long long)g.I, (long long)g.K, g.Jn, g.type, g.mn, g.trans, o.sms);
   return TTNN_OK;
 }
 
@@ -1050,7 +1050,7 @@ ttnn_status Program::run_tc(int lvl, cudaStream_t st, bool dump) const {
   std::vector<TcGemm> run;
   auto flush = [&]() -> ttnn_status {
     if (run.empty()) return TTNN_OK;
-    TTNN_TRY(tcg_run(run.data(), (int)run.size(), first->pieces, tcg_sms(), first->err, first->wait_ns, st));
+    TTNN_TRY(tcg_run(run.data(), (int)run.size(), first->pieces, first->sms, first->err, first->wait_ns, st));
     run.clear();
     return TTNN_OK;
   };

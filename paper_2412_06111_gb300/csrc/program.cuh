@@ -111,13 +111,14 @@ struct LevelBatch {
 
 // A recorded tensor-core GEMM: its prepared operand, room for pieces (shared
 // by the products of a program: its launches run in order), and what its plan
-// sets for all of its products: error word, limit of each wait.
+// sets for all of its products: error word, limit of each wait, SMs.
 struct TcOp {
   TcGemm g;
   void* prep = nullptr;
   void* pieces = nullptr;
   int* err = nullptr;
   uint64_t wait_ns = 0;
+  int sms = 0;
   int level = 0;
 };
 

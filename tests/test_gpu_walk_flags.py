@@ -113,3 +113,17 @@ def test_first_level_waits_running_out_report_timeout(dtype, dims):
     finally:
         bad.close()
         good.close()
+
+
+@pytest.mark.parametrize("case", [PREFIX, LARGE], ids=["prefix", "large_cores"])
+def test_products_leave_the_reserved_sms(case, capfd):
+    sms = torch.cuda.get_device_properties(0).multi_processor_count
+    for flags, used in ((0, sms), (api.FLAG_RESERVE_SMS, sms - 8)):   # (at most eight sketched nodes)
+        run = _open(case, api.F32, api.FLAG_DUMP_PROGRAM | flags)
+        try:
+            distance = _update(run, case)
+            lines = LINE.findall(capfd.readouterr().err)
+            assert lines and all(line.endswith(" SMs %d" % used) for _, line in lines), lines
+            assert distance() <= 1e-5
+        finally:
+            run.close()
