@@ -53,7 +53,7 @@ struct TcgProb {
   const int32_t* shift;  // TcGemm::shift, or null
   int64_t ldc, unit0;    // first (row tile, k tile) of the product in the launch
   int nkt, tile0;        // k tiles, first row tile in the launch
-  int chain;             // MMAs (of 16 k) per drain of the accumulators: 2 (not bfloat16), 4, 8 or 16
+  int chain;             // MMAs (of 16 k) per drain of the accumulators: 2 (not bfloat16), 8 or 16
   int trans;
 };
 struct TcgParams {
@@ -800,6 +800,8 @@ bool tcg_supported(const TcGemm& g) {
   const int64_t lim = int64_t(1) << 31;
   if (g.type < 1 || g.type > 3 || g.I < 1 || g.Jn < 1 || g.K < 1) return false;
   if (g.Jn > tc::kTcgMaxN) return false;
+  // a whole number of drains per tile or of tiles per drain (the issuer's two forms)
+  if (g.chain != 0 && g.chain != 8 && g.chain != 16 && (g.chain != 2 || g.type == 2)) return false;
   if (g.shift && (g.nb != 1 || g.b[0].nkr != 2)) return false;
   // float4 rows of C
   if (!g.trans && (g.ldc < round_up(g.Jn, 16) || g.ldc % 4)) return false;

@@ -32,7 +32,7 @@ struct TcGemm {
   const void* A = nullptr;
   int64_t lda = 0;
   int mn = 0, type = 1, trans = 0;
-  int chain = 0;         // MMAs (of 16 k) per drain of the accumulators: 2 (types 1, 3), 8, 16; 0: by size
+  int chain = 0;         // MMAs (of 16 k) per drain of the accumulators: 2 (types 1, 3), 8 or 16; 0: by size
   TcCols b[2];           // columns of B, one part after the other
   int nb = 1;
   // [round_up(Jn, 16)][2], for an operand of one part and two Khatri-Rao
