@@ -730,9 +730,10 @@ static ttnn_status tcg_major(bool mn, const TcgParams& p, int grid, size_t smem,
 template <typename T>
 static ttnn_status tcg_form(bool vec, bool mn, const TcgParams& p, int grid, size_t smem,
                             cudaStream_t st) {
-  if (p.Npad > 64 || sizeof(T) == 2)   // (bfloat16 converters need the fewest registers)
-    return vec ? tcg_major<T, true, 8>(mn, p, grid, smem, st) : tcg_major<T, false, 8>(mn, p, grid, smem, st);
-  return vec ? tcg_major<T, true, 4>(mn, p, grid, smem, st) : tcg_major<T, false, 4>(mn, p, grid, smem, st);
+  if constexpr (sizeof(T) > 2)   // (bfloat16 converters need the fewest registers)
+    if (p.Npad <= 64)
+      return vec ? tcg_major<T, true, 4>(mn, p, grid, smem, st) : tcg_major<T, false, 4>(mn, p, grid, smem, st);
+  return vec ? tcg_major<T, true, 8>(mn, p, grid, smem, st) : tcg_major<T, false, 8>(mn, p, grid, smem, st);
 }
 
 // Pairs in one load need even extents and strides and an aligned base.
