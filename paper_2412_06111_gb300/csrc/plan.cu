@@ -1188,14 +1188,17 @@ constexpr int64_t kTcgMinEntries = int64_t(1) << 21;
 constexpr int64_t kZgemmMinEntries = 1024;
 // Smallest first-level product (entries, D1's padding columns counted) whose
 // Khatri-Rao prefix takes the tensor-core GEMM instead of the split-K form
-// (whole updates, bfloat16, r = 20: 64^5 541 us against 554, 96x96x64x16x32
-// 342 against 375, 56^5 387 against 388, 40^5 181 against 170), and instead of
-// contractions mode by mode where s > 32 keeps the split-K form out (64^5,
+// (whole bfloat16 updates, by millions of entries: 11.2, 56^5 r = 20, 357 us
+// against 353; 12.6, 64^5 r = 16, 443 against 441; 13.8, 60^5 r = 20, 453 against
+// 450; 16.8, 64^5 r = 20, 516 against 515, 512 x 64 x 16 x 40^2 r = 12, 410
+// against 422; 17.9, 72^5 r = 16, 766 against 772; 20.1, 68^5 r = 20, 861 against
+// 871; 33.6, 256 x 64 x 32^3 r = 20, 375 against 388: they cross near 15), and
+// instead of contractions mode by mode where s > 32 keeps the split-K form out (64^5,
 // r = 32: 681 against 942; 40^5, r = 24: 190 against 246; 32^5 binary32,
 // r = 32: 213 against 218; 24^3 x 48^2, 0.8 M entries: 158 against 155) or a
 // reduction below 1024 stays whole in few blocks (64^4 x 8, binary32: 387
 // against 456).
-constexpr int64_t kTcPrefixEntries = int64_t(1) << 24;
+constexpr int64_t kTcPrefixEntries = int64_t(15) << 20;
 constexpr int64_t kTcWideEntries = int64_t(1) << 20;
 // Smallest input core (entries times columns) of a TTN-format update that is
 // contracted on the tensor cores (whole updates of 64^4, r + s = 75: rank 128
