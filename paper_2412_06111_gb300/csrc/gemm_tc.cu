@@ -28,6 +28,7 @@
 #include <cuda_bf16.h>
 
 #include <algorithm>
+#include <cfloat>
 #include <type_traits>
 
 #include "gemm_tc.cuh"
@@ -50,7 +51,6 @@ struct TcgProb {
   const void* A;
   int64_t lda, I, K;
   float* C;
-  const int32_t* shift;  // TcGemm::shift, or null
   int64_t ldc, unit0;    // first (row tile, k tile) of the product in the launch
   int nkt, tile0;        // k tiles, first row tile in the launch
   int chain;             // MMAs (of 16 k) per drain of the accumulators: 2 (not bfloat16), 8 or 16
@@ -513,8 +513,12 @@ __global__ void __launch_bounds__(tcg_threads<EPI>(), 1)
           for (int c = 0; c < 8; ++c) {
             float v = __uint_as_float(x[NACC - 1][c]);
 #pragma unroll
-            for (int o = NACC - 2; o >= 0; --o) v = fmaf(v, 1.f / kPieceScale, __uint_as_float(x[o][c]));
-            if (NACC > 1 && !isfinite(__uint_as_float(x[0][c]))) v = __uint_as_float(x[0][c]);
+            for (int o = NACC - 2; o >= 0; --o) {
+              // sums without the leading products are NaN wherever those are
+              // not finite: a finite value in their place leaves the result
+              if (o == 0) v = fmaxf(v, -FLT_MAX);
+              v = fmaf(v, 1.f / kPieceScale, __uint_as_float(x[o][c]));
+            }
             acc[cg + c] += v;
           }
         }
@@ -525,14 +529,6 @@ __global__ void __launch_bounds__(tcg_threads<EPI>(), 1)
         if (buf == 0) fph ^= 1;
       }
       if (!ok) break;
-      if (b.shift) {
-#pragma unroll
-        for (int c = 0; c < NW; ++c) {
-          if (c >= cn) continue;
-          const int e = __ldg(b.shift + 2 * (cb + c)) + __ldg(b.shift + 2 * (cb + c) + 1);
-          if (e) acc[c] = scale2(acc[c], e);
-        }
-      }
       const bool whole = kt0 == 0 && kt1 == b.nkt;
       const int64_t row = (int64_t)(it - b.tile0) * kTileM + 32 * q + lane;
       if (row < b.I && whole && b.trans) {
@@ -588,6 +584,7 @@ constexpr int kPrepRows = 8;   // rows of a thread
 // what then over- or underflows in the sum against binary32 entries does so in
 // the result.  Blocks: a column (x) of a job (y).
 __global__ void __launch_bounds__(256) tcg_range_kernel(const __grid_constant__ PrepBatch b) {
+  pdl_begin();
   const PrepJob& j = b.job[blockIdx.y];
   const TcCols& c = j.c[0];
   const int col = blockIdx.x, warp = threadIdx.x >> 5;
@@ -708,6 +705,20 @@ __global__ void __launch_bounds__(256) tcg_pieces_kernel(const __grid_constant__
   }
 }
 
+// Gives the powers of two of tcg_range_kernel back to the columns of C (x; rows:
+// y).  A kernel of its own: in the epilogue it cost every product more than this
+// launch (a rank-200 update 675 us against 656, 64^5 521 against 516).
+__global__ void __launch_bounds__(256) tcg_unshift_kernel(float* C, const int32_t* shift, int64_t I, int64_t si,
+                                                          int64_t sj) {
+  pdl_begin();
+  const int e = shift[2 * blockIdx.x] + shift[2 * blockIdx.x + 1];
+  if (e == 0) return;
+  for (int64_t i = blockIdx.y * 256 + threadIdx.x; i < I; i += gridDim.y * 256) {
+    float* c = C + i * si + blockIdx.x * sj;
+    *c = scale2(*c, e);
+  }
+}
+
 static int tcg_pieces_of(const TcGemm& g) { return g.type == 2 ? 1 : 3; }
 static int tcg_kt(const TcGemm& g) { return g.type == 2 ? 128 : 64; }
 static int tcg_npad(const TcGemm& g) { return (int)round_up(g.Jn, 16); }
@@ -763,7 +774,6 @@ static ttnn_status tcg_batch(const TcGemm* const* g, int n, void* pieces, int sm
     q.I = g[k]->I;
     q.K = g[k]->K;
     q.C = (float*)g[k]->C;
-    q.shift = g[k]->shift;
     q.ldc = g[k]->ldc;
     q.trans = g[k]->trans;
     q.unit0 = p.units;
@@ -788,9 +798,19 @@ static ttnn_status tcg_batch(const TcGemm* const* g, int n, void* pieces, int sm
   if (f.type == 2) TTNN_TRY(tcg_form<uint16_t>(vec, mn, p, grid, smem, st));
   else if (f.type == 1) TTNN_TRY(tcg_form<float>(vec, mn, p, grid, smem, st));
   else TTNN_TRY(tcg_form<double>(vec, mn, p, grid, smem, st));
-  if (grid == 1) return TTNN_OK;
-  tcg_pieces_kernel<<<dim3((unsigned)(grid - 1), 4), 256, 0, st>>>(p, grid);
-  return check_launch("tcg_pieces_kernel");
+  if (grid > 1) {
+    tcg_pieces_kernel<<<dim3((unsigned)(grid - 1), 4), 256, 0, st>>>(p, grid);
+    TTNN_TRY(check_launch("tcg_pieces_kernel"));
+  }
+  for (int k = 0; k < n; ++k) {
+    if (!g[k]->shift) continue;
+    const int64_t si = g[k]->trans ? 1 : g[k]->ldc, sj = g[k]->trans ? g[k]->ldc : 1;
+    const unsigned by = (unsigned)std::min<int64_t>(ceil_div(g[k]->I, (int64_t)1024), 64);
+    launch_pdl(tcg_unshift_kernel, dim3((unsigned)g[k]->Jn, by), 256, 0, st, (float*)g[k]->C, g[k]->shift,
+               g[k]->I, si, sj);
+    TTNN_TRY(check_launch("tcg_unshift_kernel"));
+  }
+  return TTNN_OK;
 }
 
 }  // namespace tc
@@ -848,7 +868,7 @@ ttnn_status tcg_prepare(const TcGemm* g, int n, void* const* dst, cudaStream_t s
       }
     }
     if (ranged) {
-      tcg_range_kernel<<<dim3((unsigned)ranged, (unsigned)pb.n), 256, 0, st>>>(pb);
+      launch_pdl(tcg_range_kernel, dim3((unsigned)ranged, (unsigned)pb.n), 256, 0, st, pb);
       TTNN_TRY(check_launch("tcg_range_kernel"));
     }
     tcg_prepare_kernel<<<(unsigned)blocks, 256, 0, st>>>(pb);

@@ -37,7 +37,7 @@ struct TcGemm {
   int nb = 1;
   // [round_up(Jn, 16)][2], for an operand of one part and two Khatri-Rao
   // factors that the data decide: the powers of two tcg_prepare takes off the
-  // factors of each column, given back to C (tcg_range_kernel)
+  // factors of each column, given back to C afterwards (tcg_range_kernel)
   int32_t* shift = nullptr;
   void* C = nullptr;
   int64_t ldc = 0;
