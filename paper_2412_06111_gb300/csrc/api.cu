@@ -581,8 +581,11 @@ ttnn_status ttnn_update_ttn(ttnn_state_t S, const double* const* cores_in, const
   if (need > P.ws_bytes) {
     // where the workspace cannot grow (no memory, or a graph is captured) the
     // general form runs in what there is, or asks for less
-    cudaStreamCaptureStatus cs = cudaStreamCaptureStatusNone;
-    if (cudaStreamIsCapturing(st, &cs) != cudaSuccess) cudaGetLastError();
+    cudaStreamCaptureStatus cs = cudaStreamCaptureStatusActive;
+    if (cudaStreamIsCapturing(st, &cs) != cudaSuccess) {   // (another stream's, seen from the default one)
+      cudaGetLastError();
+      cs = cudaStreamCaptureStatusActive;
+    }
     ttnn_status grown = TTNN_ENOMEM;
     if (cs == cudaStreamCaptureStatusNone) grown = grow_workspace(P, need + 4096);
     if (grown != TTNN_OK) {
