@@ -21,7 +21,7 @@
 // instead of six.
 //
 // Warp roles: warp 0 copies B tiles by TMA, warp 1 owns TMEM and issues the
-// MMAs, the next 4 or 8 drain accumulators (TMEM lane quarter = warp % 4), the
+// MMAs, the next 8 drain accumulators (TMEM lane quarter = warp % 4), the
 // last 16 load, convert and store A tiles (128-byte swizzle).  Every wait is
 // bounded; on expiry the kernel sets an error bit, drains its own copies and
 // MMAs, frees TMEM and returns.
@@ -39,11 +39,11 @@ namespace tc {
 
 constexpr int kTcgMaxN = 80;      // columns of a product
 constexpr int kTcgConv = 16;      // converter warps (8 left the latency of the loads bare: twice the time)
-// Epilogue warps: one per lane quarter, or for products of more than 64
-// columns two (a half of the columns each: 80 sums do not fit the registers
-// that 16 converter warps leave; with two throughout, the converters spill).
-template <int EPI>
-__host__ __device__ constexpr int tcg_threads() { return 32 * (2 + EPI + kTcgConv); }
+// Epilogue warps: two per lane quarter, a half of the columns each (one per
+// quarter holds twice the sums and spills: 64^5 bfloat16 514 against 509 us, a
+// rank-200 TTN update 659 against 650, an 8 x 64^4 binary32 slab 365 against 367).
+constexpr int kTcgEpi = 8;
+constexpr int kTcgThreads = 32 * (2 + kTcgEpi + kTcgConv);
 constexpr int kTcgMaxStages = 6;
 
 struct TcgProb {
@@ -163,14 +163,16 @@ struct Pair<double, VEC> {
 // rounded, which leaves the third either sign: the piece products left out
 // then average to nothing (a 200-rank tree's Psi erred by 6.2e-7 with both cut
 // toward zero, 4.8e-7 so).  The first piece of an infinity or NaN is it, its
-// other pieces are NaN: where the leading products of a sum are not finite, the
-// epilogue takes them alone, which gives what binary32 multiply-adds give.
+// other pieces are NaN: the sums of lower order are NaN then, and the epilogue
+// leaves what the leading products give, as binary32 multiply-adds would.
 //
 // bfloat16 ends at 2^-133: unscaled, the pieces of a binary32 entry below 2^-110
 // lose its low bits (entries of 1e-35: 4.4e-6 off).  With piece i times 2^(6 i) the
 // products of order o = i + j are 2^(6 o) too large, which the epilogue takes
 // back; 2^6 is the most for which the sums of order 1 (two products below 2^-7
-// of the leading one each) cannot overflow before those of order 0.
+// of the leading one each) cannot overflow before those of order 0.  (The
+// multiplications cost a binary32 box of 8 x 64^4 20 of 371 us; packed in pairs
+// they cost 36, in spills.)
 constexpr float kPieceScale = 64.f;
 __device__ __forceinline__ void cut3(float x, float y, uint32_t* w) {
   // (not a cut of the bits: a NaN may have all of its in the lower half)
@@ -184,6 +186,23 @@ __device__ __forceinline__ void cut3(float x, float y, uint32_t* w) {
   w[2] = __byte_perm(__float_as_uint(x), __float_as_uint(y), 0x7632);
 }
 
+// a s + b and a + b of two columns in one instruction each.
+__device__ __forceinline__ float2 fma2(float2 a, float s, float2 b) {
+  float2 r;
+  asm("{\n\t.reg .b64 a, b, s;\n\tmov.b64 a, {%2, %3};\n\tmov.b64 b, {%4, %5};\n\tmov.b64 s, {%6, %6};\n\t"
+      "fma.rn.f32x2 a, a, s, b;\n\tmov.b64 {%0, %1}, a;\n\t}\n"
+      : "=f"(r.x), "=f"(r.y)
+      : "f"(a.x), "f"(a.y), "f"(b.x), "f"(b.y), "f"(s));
+  return r;
+}
+__device__ __forceinline__ float2 add2(float2 a, float2 b) {
+  float2 r;
+  asm("{\n\t.reg .b64 a, b;\n\tmov.b64 a, {%2, %3};\n\tmov.b64 b, {%4, %5};\n\t"
+      "add.rn.f32x2 a, a, b;\n\tmov.b64 {%0, %1}, a;\n\t}\n"
+      : "=f"(r.x), "=f"(r.y)
+      : "f"(a.x), "f"(a.y), "f"(b.x), "f"(b.y));
+  return r;
+}
 __device__ __forceinline__ void st_shared(uint32_t addr, uint32_t v) {
   asm volatile("st.shared.b32 [%0], %1;" ::"r"(addr), "r"(v) : "memory");
 }
@@ -195,12 +214,11 @@ __device__ __forceinline__ void tmem_ld8(uint32_t taddr, uint32_t* r) {
       : "r"(taddr));
 }
 
-// EPI epilogue warps.
-template <typename T, bool MN, bool VEC, int EPI>
-__global__ void __launch_bounds__(tcg_threads<EPI>(), 1)
+template <typename T, bool MN, bool VEC>
+__global__ void __launch_bounds__(kTcgThreads, 1)
     tcg_kernel(const __grid_constant__ TcgParams p) {
   using F = Form<T>;
-  constexpr int NW = EPI == 4 ? 64 : kTcgMaxN / 2;   // columns an epilogue thread holds sums of
+  constexpr int NW = kTcgMaxN / 2;               // columns an epilogue thread holds sums of
   constexpr int NS = F::NS, KT = F::KT, NACC = F::NACC;
   constexpr int R = MN ? KT : kTileM;            // tile rows in memory order
   constexpr int CB = MN ? 2 : KT / 64;           // 64-column boxes of a row
@@ -238,7 +256,7 @@ __global__ void __launch_bounds__(tcg_threads<EPI>(), 1)
     }
     for (int k = 0; k < 2; ++k) {
       mbar_init(smem_u32(&bar_full[k]), 1);
-      mbar_init(smem_u32(&bar_free[k]), EPI);
+      mbar_init(smem_u32(&bar_free[k]), kTcgEpi);
     }
     mbar_init(smem_u32(&bar_done), 1);
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
@@ -370,9 +388,9 @@ __global__ void __launch_bounds__(tcg_threads<EPI>(), 1)
       }
       mma_commit(smem_u32(&bar_done));
     }
-  } else if (warp >= 2 + EPI) {
+  } else if (warp >= 2 + kTcgEpi) {
     // ---------------- converters ----------------
-    const int cw = (warp - 2 - EPI) % NCW, grp = (warp - 2 - EPI) / NCW;
+    const int cw = (warp - 2 - kTcgEpi) % NCW, grp = (warp - 2 - kTcgEpi) / NCW;
     int stage = 0;
     uint32_t ph = 0;
     bool ok = true;
@@ -484,7 +502,7 @@ __global__ void __launch_bounds__(tcg_threads<EPI>(), 1)
   } else {
     // ---------------- epilogue ----------------
     const int q = warp & 3;
-    const int cn = p.Npad * 4 / EPI, cb = (warp - 2) / 4 * cn;   // this warp's columns (a multiple of 8)
+    const int cn = p.Npad / 2, cb = (warp - 2) / 4 * cn;   // this warp's columns (a multiple of 8)
     const uint32_t lane_off = (uint32_t)(32 * q) << 16;
     int buf = 0;
     uint32_t fph = 0;
@@ -510,16 +528,18 @@ __global__ void __launch_bounds__(tcg_threads<EPI>(), 1)
           for (int o = 0; o < NACC; ++o) tmem_ld8(d + o * p.Npad + cg, x[o]);
           tmem_wait_ld();
 #pragma unroll
-          for (int c = 0; c < 8; ++c) {
-            float v = __uint_as_float(x[NACC - 1][c]);
+          for (int c = 0; c < 8; c += 2) {
+            float2 v = make_float2(__uint_as_float(x[NACC - 1][c]), __uint_as_float(x[NACC - 1][c + 1]));
 #pragma unroll
             for (int o = NACC - 2; o >= 0; --o) {
               // sums without the leading products are NaN wherever those are
               // not finite: a finite value in their place leaves the result
-              if (o == 0) v = fmaxf(v, -FLT_MAX);
-              v = fmaf(v, 1.f / kPieceScale, __uint_as_float(x[o][c]));
+              if (o == 0) v = make_float2(fmaxf(v.x, -FLT_MAX), fmaxf(v.y, -FLT_MAX));
+              v = fma2(v, 1.f / kPieceScale, make_float2(__uint_as_float(x[o][c]), __uint_as_float(x[o][c + 1])));
             }
-            acc[cg + c] += v;
+            const float2 a = add2(make_float2(acc[cg + c], acc[cg + c + 1]), v);
+            acc[cg + c] = a.x;
+            acc[cg + c + 1] = a.y;
           }
         }
         fence_before();
@@ -723,28 +743,20 @@ static int tcg_pieces_of(const TcGemm& g) { return g.type == 2 ? 1 : 3; }
 static int tcg_kt(const TcGemm& g) { return g.type == 2 ? 128 : 64; }
 static int tcg_npad(const TcGemm& g) { return (int)round_up(g.Jn, 16); }
 
-template <typename T, bool MN, bool VEC, int EPI>
+template <typename T, bool MN, bool VEC>
 static ttnn_status tcg_launch(const TcgParams& p, int grid, size_t smem, cudaStream_t st) {
   constexpr int kind = sizeof(T) == 2 ? 0 : sizeof(T) == 4 ? 1 : 2;
-  constexpr int slot = 8 + kind * 8 + (EPI > 4 ? 4 : 0) + (MN ? 2 : 0) + (VEC ? 1 : 0);
-  TTNN_TRY(smem_limit_once((const void*)tcg_kernel<T, MN, VEC, EPI>, slot));
-  tcg_kernel<T, MN, VEC, EPI><<<grid, tcg_threads<EPI>(), smem, st>>>(p);
+  constexpr int slot = 8 + kind * 4 + (MN ? 2 : 0) + (VEC ? 1 : 0);
+  TTNN_TRY(smem_limit_once((const void*)tcg_kernel<T, MN, VEC>, slot));
+  tcg_kernel<T, MN, VEC><<<grid, kTcgThreads, smem, st>>>(p);
   return check_launch("tcg_kernel");
-}
-
-template <typename T, bool VEC, int EPI>
-static ttnn_status tcg_major(bool mn, const TcgParams& p, int grid, size_t smem, cudaStream_t st) {
-  return mn ? tcg_launch<T, true, VEC, EPI>(p, grid, smem, st)
-            : tcg_launch<T, false, VEC, EPI>(p, grid, smem, st);
 }
 
 template <typename T>
 static ttnn_status tcg_form(bool vec, bool mn, const TcgParams& p, int grid, size_t smem,
                             cudaStream_t st) {
-  if constexpr (sizeof(T) > 2)   // (bfloat16 converters need the fewest registers)
-    if (p.Npad <= 64)
-      return vec ? tcg_major<T, true, 4>(mn, p, grid, smem, st) : tcg_major<T, false, 4>(mn, p, grid, smem, st);
-  return vec ? tcg_major<T, true, 8>(mn, p, grid, smem, st) : tcg_major<T, false, 8>(mn, p, grid, smem, st);
+  if (mn) return vec ? tcg_launch<T, true, true>(p, grid, smem, st) : tcg_launch<T, true, false>(p, grid, smem, st);
+  return vec ? tcg_launch<T, false, true>(p, grid, smem, st) : tcg_launch<T, false, false>(p, grid, smem, st);
 }
 
 // Pairs in one load need even extents and strides and an aligned base.
