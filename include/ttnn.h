@@ -82,7 +82,13 @@ typedef enum {
 
 /* Number formats of the tensor and of the pass-side DRM blocks. */
 typedef enum {
-  TTNN_F64 = 0,   /* binary64 everywhere (accumulators binary64) */
+  TTNN_F64 = 0,   /* binary64 everywhere (accumulators binary64); the first-level products of
+                     1024 entries and more are summed from 8-bit digits on the tensor cores:
+                     an entry is held to 62 bits below the largest of its row (its column, for
+                     the other product) of the pass matrix and a DRM entry to 62 below its
+                     column's, so the error bound is of max |a| max |b| instead of sum |a||b|
+                     (in norm no larger than with binary64 multiply-adds; single sketch entries
+                     of sparse or outlier-dominated rows may lose digits: TTNN_FLAG_SIMT_PASS) */
   TTNN_F32 = 1,   /* binary32 tensor, FP32 FMA pass, FP32 accumulators */
   TTNN_BF16 = 2,  /* bfloat16 tensor + DRM blocks on tensor cores, FP32 accumulation */
   TTNN_E4M3 = 3,  /* FP8 E4M3 tensor with one FP32 scale per 128x128 tile, FP32 accumulation */
@@ -108,7 +114,8 @@ typedef struct {
 } ttnn_opts;
 
 #define TTNN_FLAG_NO_SIDE_CACHE 1u  /* do not cache full-size pass DRM blocks */
-#define TTNN_FLAG_SIMT_PASS 2u      /* use the SIMT pass even for BF16 (testing) */
+#define TTNN_FLAG_SIMT_PASS 2u      /* first-level products on the FP32 (binary64 plans: FP64)
+                                       units, by multiply-adds, in every format */
 #define TTNN_FLAG_STRUCTURED_ONLY 8u /* the plan takes CP / TTN-format updates only: no
                                          cached pass blocks, no dense-pass workspace
                                          (ttnn_update_dense returns TTNN_EUNSUPPORTED) */

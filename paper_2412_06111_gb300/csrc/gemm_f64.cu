@@ -11,9 +11,19 @@
 // in one accumulator per order o: over a tile of 32 k that is at most
 // 8 * 32 * 2^14 = 2^22, so the binary32 accumulators hold exact integers and
 // the tensor core's rounding never acts.  The epilogue adds them to 64-bit
-// integers per output (orders 0-3 and 4-7 apart), rounded to binary64 once, at
-// the end.  What is left out, orders 8 and up and the cut bits, is below 2^-58
-// of the largest products.  (With seven digits a 20^6 sketch took 5 % less
+// integers per output (orders 0-3 and 4-7 apart), which are converted and joined
+// at the end of a row tile (three roundings where a half has more than 53 bits
+// or the result is subnormal, else one); the pieces of a tile that several CTAs
+// worked on are added in binary64.
+//
+// What is left out, orders 8 and up and the cut bits, is below 2^-57 (2^-60 rms)
+// of max|a| max|b| per product: an entry far below the largest of its row is held
+// in fewer than 53 bits.  In norm the sketches err no more than with multiply-
+// adds (24^4 to 20^6, 16 sizes: 0.8 to 1.02 of it); an entry whose sum of
+// |a||b| is far below max|a| max|b|, as in a row of few non-zeros or with one
+// outlier, errs more (error over sum |a||b|: Gaussian 6e-17 against 1.1e-16,
+// 0.2 % non-zeros 3.5e-15 against 2.6e-16, 20 outliers of 1e10 1.3e-14 against
+// 1.5e-15).  TTNN_FLAG_SIMT_PASS keeps the FP64 units.  (With seven digits a 20^6 sketch took 5 % less
 // time and erred more than the FP64 units' sums: the columns of B are
 // Khatri-Rao products whose largest entry is 100 times their mean.)  Row
 // exponents only grow within a sum; when one does, its accumulators are

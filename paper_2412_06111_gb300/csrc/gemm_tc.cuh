@@ -25,7 +25,7 @@ struct TcCols {
 // binary64 (B and C too), 1 binary32, 2 bfloat16 (B too), 3 binary64 rounded
 // to binary32; C of types 1 to 3 is binary32, B of 1 and 3.  C(i, j) is at
 // C[i * ldc + j], with every column up to round_up(Jn, 16) <= ldc written
-// (zeros beyond Jn), or with `trans` (types 1 to 3) at C[j * ldc + i].
+// (beyond Jn zeros, or NaN in rows with entries that are not finite), or with `trans` (types 1 to 3) at C[j * ldc + i].
 struct TcGemm {
   int64_t I = 0, K = 0;
   int Jn = 0;

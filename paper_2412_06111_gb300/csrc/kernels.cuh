@@ -128,8 +128,6 @@ ttnn_status launch_side_gather_batch(const GatherJob* jobs, int n, cudaStream_t 
 constexpr int kStoreFp8 = 3, kStoreSplit = 4;
 // With mcopy, mcopy[row] = the sketched value of m[row] in the walk type is
 // written beside; with bcopy, bcopy[c] = brow[c] (side format) for c < bcols.
-// With mcopy, mcopy[row] = the sketched value of m[row] in the walk type is
-// written beside; with bcopy, bcopy[c] = brow[c] (side format) for c < bcols.
 ttnn_status launch_side_gemv(const SideSpec& s, const void* src, int64_t src_ld, bool cut,
                              const void* m, int m_store, const float* scale, int64_t rows,
                              int cols, int cols_pad, void* D, int d_f64, void* mcopy,
