@@ -596,12 +596,22 @@ __global__ void __launch_bounds__(256) zslice_kernel(const __grid_constant__ ZPr
   }
 }
 
+// C(row, col) from the operands, in order, up to the first NaN.
+template <bool MN>
+__device__ __noinline__ double z_direct(const ZParams& p, int64_t row, int col) {
+  const double* x = p.A + row * (MN ? 1 : p.lda);
+  const double* y = p.B + col * p.ldb;
+  double a = 0.;
+  for (int64_t k = 0; k < p.K && !isnan(a); ++k) a = __fma_rn(x[k * (MN ? p.lda : 1)], y[k], a);
+  return a;
+}
+
 // Sums the pieces of the row tiles that more than one CTA worked on.  Where an
 // infinity or NaN of A or B has left NaN, the entry is summed from the operands
 // by multiply-adds, as the FP64 units would (up to the first NaN of its sum).
 // Whole tiles are looked over for that as well: a read of C.
 template <bool MN>
-__global__ void __launch_bounds__(256) zpieces_kernel(const ZParams p, int G) {
+__global__ void __launch_bounds__(256) zpieces_kernel(const __grid_constant__ ZParams p, int G) {
   const int it = blockIdx.x, nkb = p.nkb, Npad = p.Npad;
   const int64_t total = (int64_t)p.nI * nkb;
   auto owner = [&](int64_t u) { return (int)(((u + 1) * G - 1) / total); };
@@ -617,15 +627,9 @@ __global__ void __launch_bounds__(256) zpieces_kernel(const ZParams p, int G) {
     double a = c0 == c1 ? *out : p0[e];
 #pragma unroll 4
     for (int c = c0 + 1; c <= c1; ++c) a += p.part[(int64_t)(2 * c) * tile + e];
-    if (isnan(a) && col < p.Jn) {
-      const double* x = p.A + row * (MN ? 1 : p.lda);
-      const double* y = p.B + col * p.ldb;
-      a = 0.;
-      for (int64_t k = 0; k < p.K && !isnan(a); ++k) a = __fma_rn(x[k * (MN ? p.lda : 1)], y[k], a);
-    } else if (c0 == c1) {
-      continue;
-    }
-    *out = a;
+    const bool redo = ((uint32_t)__double2hiint(a) & 0x7FFFFFFFu) > 0x7FF00000u && col < p.Jn;   // a NaN
+    if (redo) a = z_direct<MN>(p, row, col);
+    if (redo || c0 != c1) *out = a;
   }
 }
 
