@@ -725,16 +725,27 @@ __global__ void __launch_bounds__(256) tcg_pieces_kernel(const __grid_constant__
   }
 }
 
-// Gives the powers of two of tcg_range_kernel back to the columns of C (x; rows:
-// y).  A kernel of its own: in the epilogue it cost every product more than this
-// launch (a rank-200 update 675 us against 656, 64^5 521 against 516).
-__global__ void __launch_bounds__(256) tcg_unshift_kernel(float* C, const int32_t* shift, int64_t I, int64_t si,
-                                                          int64_t sj) {
+// Gives the powers of two of tcg_range_kernel back to the columns of C (column:
+// x; rows: y; product: z).  A kernel of its own: in the epilogue it cost every
+// product more than this launch (a rank-200 update 675 us against 656, 64^5 521
+// against 516).
+struct UnshiftBatch {
+  struct {
+    float* C;
+    const int32_t* shift;
+    int64_t I, si, sj;
+    int Jn;
+  } job[kTcgBatch];
+};
+__global__ void __launch_bounds__(256) tcg_unshift_kernel(const __grid_constant__ UnshiftBatch b) {
   pdl_begin();
-  const int e = shift[2 * blockIdx.x] + shift[2 * blockIdx.x + 1];
+  const auto& j = b.job[blockIdx.z];
+  const int col = blockIdx.x;
+  if (col >= j.Jn) return;
+  const int e = j.shift[2 * col] + j.shift[2 * col + 1];
   if (e == 0) return;
-  for (int64_t i = blockIdx.y * 256 + threadIdx.x; i < I; i += gridDim.y * 256) {
-    float* c = C + i * si + blockIdx.x * sj;
+  for (int64_t i = blockIdx.y * 256 + threadIdx.x; i < j.I; i += gridDim.y * 256) {
+    float* c = j.C + i * j.si + col * j.sj;
     *c = scale2(*c, e);
   }
 }
@@ -814,12 +825,25 @@ static ttnn_status tcg_batch(const TcGemm* const* g, int n, void* pieces, int sm
     tcg_pieces_kernel<<<dim3((unsigned)(grid - 1), 4), 256, 0, st>>>(p, grid);
     TTNN_TRY(check_launch("tcg_pieces_kernel"));
   }
+  UnshiftBatch u;
+  int shifted = 0, most = 0;
+  int64_t rows = 0;
   for (int k = 0; k < n; ++k) {
-    if (!g[k]->shift) continue;
-    const int64_t si = g[k]->trans ? 1 : g[k]->ldc, sj = g[k]->trans ? g[k]->ldc : 1;
-    const unsigned by = (unsigned)std::min<int64_t>(ceil_div(g[k]->I, (int64_t)1024), 64);
-    launch_pdl(tcg_unshift_kernel, dim3((unsigned)g[k]->Jn, by), 256, 0, st, (float*)g[k]->C, g[k]->shift,
-               g[k]->I, si, sj);
+    const TcGemm& m = *g[k];
+    if (!m.shift) continue;
+    auto& j = u.job[shifted++];
+    j.C = (float*)m.C;
+    j.shift = m.shift;
+    j.I = m.I;
+    j.si = m.trans ? 1 : m.ldc;
+    j.sj = m.trans ? m.ldc : 1;
+    j.Jn = m.Jn;
+    most = std::max(most, m.Jn);
+    rows = std::max(rows, m.I);
+  }
+  if (shifted) {
+    const unsigned by = (unsigned)std::min<int64_t>(ceil_div(rows, (int64_t)1024), 64);
+    launch_pdl(tcg_unshift_kernel, dim3((unsigned)most, by, (unsigned)shifted), 256, 0, st, u);
     TTNN_TRY(check_launch("tcg_unshift_kernel"));
   }
   return TTNN_OK;
