@@ -19,7 +19,7 @@
 // What is left out, orders 8 and up and the cut bits, is below 2^-57 (2^-60 rms)
 // of max|a| max|b| per product: an entry far below the largest of its row is held
 // in fewer than 53 bits.  In norm the sketches err no more than with multiply-
-// adds (24^4 to 20^6, 16 sizes: 0.8 to 1.02 of it); an entry whose sum of
+// adds (eight sizes up to 20^6: 0.84 to 1.02 of it); an entry whose sum of
 // |a||b| is far below max|a| max|b|, as in a row of few non-zeros or with one
 // outlier, errs more (error over sum |a||b|: Gaussian 6e-17 against 1.1e-16,
 // 0.2 % non-zeros 3.5e-15 against 2.6e-16, 20 outliers of 1e10 1.3e-14 against
