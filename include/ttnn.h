@@ -114,8 +114,9 @@ typedef struct {
 } ttnn_opts;
 
 #define TTNN_FLAG_NO_SIDE_CACHE 1u  /* do not cache full-size pass DRM blocks */
-#define TTNN_FLAG_SIMT_PASS 2u      /* first-level products on the FP32 (binary64 plans: FP64)
-                                       units, by multiply-adds, in every format */
+#define TTNN_FLAG_SIMT_PASS 2u      /* every product on the FP32 (binary64 plans: FP64) units, by
+                                       multiply-adds, in every format: first-level passes,
+                                       Khatri-Rao prefixes, cores of TTN-format input */
 #define TTNN_FLAG_STRUCTURED_ONLY 8u /* the plan takes CP / TTN-format updates only: no
                                          cached pass blocks, no dense-pass workspace
                                          (ttnn_update_dense returns TTNN_EUNSUPPORTED) */

@@ -1646,7 +1646,8 @@ ttnn_status run_dense_update(ttnn_plan_s& P, void* acc, const void* data, const 
       y.kj[y.nkr] = 1;
     }
     const bool split = krL->s <= 32 && g.K >= 1024;   // the split-K form would fill the chip
-    if (P.roomy && g.K * g.I >= (split ? kTcPrefixEntries : kTcWideEntries) && tcg_supported(g)) {
+    if (P.roomy && !(P.flags & TTNN_FLAG_SIMT_PASS) &&
+        g.K * g.I >= (split ? kTcPrefixEntries : kTcWideEntries) && tcg_supported(g)) {
       char* out;
       int64_t ld;
       tc_gemm(C, g, {D1}, &out, &ld);
@@ -1892,7 +1893,8 @@ ttnn_status run_ttn_update(ttnn_plan_s& P, void* acc, const double* const* cores
   std::vector<char> big(nn, 0);
   for (int v = 0; v < nn; ++v) {
     const TNode& nd = P.nodes[v];
-    if (!P.roomy || P.walk_f64 || v == P.root || nd.leaf || nd.ch.size() != 2 || nd.rsub == 0) continue;
+    if (!P.roomy || (P.flags & TTNN_FLAG_SIMT_PASS) || P.walk_f64) continue;
+    if (v == P.root || nd.leaf || nd.ch.size() != 2 || nd.rsub == 0) continue;
     const int64_t c1 = R(nd.ch[0]), c2 = R(nd.ch[1]);
     TcGemm up;
     up.type = 3;

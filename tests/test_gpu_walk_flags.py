@@ -83,10 +83,10 @@ def _expect_timeout(run, update):
 
 
 # products of a walk alone: the large cores; a prefix behind a first-level
-# product on the FP32 units (SIMT_PASS: it has no waits)
-@pytest.mark.parametrize("case,flags", [(LARGE, 0), (PREFIX, api.FLAG_SIMT_PASS)], ids=["large_cores", "prefix"])
-def test_walk_waits_running_out_report_timeout(case, flags):
-    bad, good = (_open(case, api.F32, flags | f) for f in (api.FLAG_WAIT_TEST, 0))
+# product small enough for the FP32 units (which have no waits)
+@pytest.mark.parametrize("case", [LARGE, PREFIX], ids=["large_cores", "prefix"])
+def test_walk_waits_running_out_report_timeout(case):
+    bad, good = (_open(case, api.F32, f) for f in (api.FLAG_WAIT_TEST, 0))
     try:
         _expect_timeout(bad, lambda run: _update(run, case))
         assert _update(good, case)() <= 1e-5   # the context is intact
@@ -127,3 +127,14 @@ def test_products_leave_the_reserved_sms(case, capfd):
             assert distance() <= 1e-5
         finally:
             run.close()
+
+
+@pytest.mark.parametrize("case", [PREFIX, LARGE], ids=["prefix", "large_cores"])
+def test_simt_pass_keeps_products_off_the_tensor_cores(case, capfd):
+    run = _open(case, api.F32, api.FLAG_DUMP_PROGRAM | api.FLAG_SIMT_PASS)
+    try:
+        distance = _update(run, case)
+        assert not LINE.findall(capfd.readouterr().err)
+        assert distance() <= 1e-5
+    finally:
+        run.close()
