@@ -148,3 +148,11 @@ def test_binary64_infinities_of_both_signs_in_one_row():
     data = W.gaussian(dims, 9)
     data[3, 4, 7], data[3, 4, 60], data[3, 5, 7] = np.inf, -np.inf, np.inf
     _check_not_finite(dims, 6, 4, api.F64, data)
+
+
+# the second and third group of 32 columns take their own part of the operand
+@pytest.mark.parametrize("dims,r,p", [([30, 40, 70], 16, 17), ([50, 52, 90], 40, 16)])
+def test_binary64_infinity_in_later_column_groups(dims, r, p):
+    data = W.gaussian(dims, 9)
+    data[11, 13, 17] = np.inf
+    _check_not_finite(dims, r, p, api.F64, data)
